@@ -188,94 +188,6 @@ __global__ void band_solve_tiles_kernel(const int32_t* __restrict__ node_off,
   }
 }
 
-// The same solve with the factor columns streamed through a shared-memory
-// ring: chunks of kBC columns (contiguous in the band storage) are copied by
-// 4- or 8-byte cp.async, kBS chunks ahead of the row being eliminated, so the
-// serial row chain of a warp reads its multipliers from shared memory instead
-// of waiting on HBM (deeper register prefetch cost occupancy).  The final
-// scalings are folded in: y(j) = v(j) Lc[j][0] once row j's updates are out.
-// Measured on the 2048^2 power grid: FP32 475 us per solve against 700 us
-// for the register-prefetch kernel; FP64 1.8 ms against 1.3 ms (fewer
-// resident warps for the FP64 pipe), so FP64 keeps the other kernel.
-constexpr int kBC = 16;  // columns per chunk
-constexpr int kBS = 4;   // chunks in flight
-
-template <class FT>
-__device__ __forceinline__ void cp_async_elem(FT* smem, const FT* gmem) {
-  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
-  if constexpr (sizeof(FT) == 8)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(a), "l"(gmem) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(gmem) : "memory");
-}
-
-template <class FT, int Q>
-__global__ void __launch_bounds__(32) band_solve_stream_kernel(
-    const int32_t* __restrict__ node_off, const int32_t* __restrict__ bwv,
-    const int64_t* __restrict__ band_off, const FT* __restrict__ Lc, const FT* __restrict__ Uc,
-    FT* __restrict__ v, int64_t stride, int nparts, int n_max, int B_max) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  FT* x = reinterpret_cast<FT*>(smem_raw);
-  FT* ring = x + ((n_max + 1) & ~1);
-  const int t = blockIdx.x % nparts;
-  const int col = blockIdx.x / nparts;
-  const int off = node_off[t];
-  const int n = node_off[t + 1] - off;
-  const int bw = bwv[t];
-  const int B = bw + 1;
-  const int lane = threadIdx.x;
-  FT* vg = v + (size_t)col * stride + off;
-  const FT* lc = Lc + band_off[t];
-  const FT* uc = Uc + band_off[t];
-  for (int i = lane; i < n; i += 32) x[i] = vg[i];
-  const int nch = (n + kBC - 1) / kBC;
-  // chunk c of a pass: columns [c kBC, ...) forward, [n - (c+1) kBC, ...) backward
-  auto issue = [&](const FT* base, int c, bool fwd) {
-    if (c < nch) {
-      const int j0 = fwd ? c * kBC : max(0, n - (c + 1) * kBC);
-      const int j1 = fwd ? min(n, (c + 1) * kBC) : n - c * kBC;
-      FT* dst = ring + (size_t)(c % kBS) * kBC * B_max;
-      const FT* src = base + (size_t)j0 * B;
-      const int cnt = (j1 - j0) * B;
-      for (int e = lane; e < cnt; e += 32) cp_async_elem(dst + e, src + e);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  for (int pass = 0; pass < 2; ++pass) {
-    const bool fwd = pass == 0;
-    const FT* base = fwd ? lc : uc;
-    for (int c = 0; c < kBS; ++c) issue(base, c, fwd);
-    __syncwarp();
-    for (int c = 0; c < nch; ++c) {
-      asm volatile("cp.async.wait_group %0;" ::"n"(kBS - 1) : "memory");
-      __syncwarp();
-      const FT* stg = ring + (size_t)(c % kBS) * kBC * B_max;
-      const int j0 = fwd ? c * kBC : max(0, n - (c + 1) * kBC);
-      const int j1 = fwd ? min(n, (c + 1) * kBC) : n - c * kBC;
-      for (int q = 0; q < j1 - j0; ++q) {
-        const int j = fwd ? j0 + q : j1 - 1 - q;
-        const FT* colj = stg + (size_t)(j - j0) * B;
-        const FT u = x[j];
-        const int m = fwd ? min(bw, n - 1 - j) : min(bw, j);
-#pragma unroll
-        for (int r = 0; r < Q; ++r) {
-          const int a = lane + 1 + 32 * r;
-          if (a <= m) {
-            if (fwd) x[j + a] -= colj[a] * u;
-            else x[j - a] -= colj[a] * u;
-          }
-        }
-        if (lane == 0) x[j] = u * colj[0];
-        __syncwarp();
-      }
-      issue(base, c + kBS, fwd);  // this stage is read: refill it
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncwarp();
-  }
-  for (int i = lane; i < n; i += 32) vg[i] = x[i];
-}
-
 // Band solves of bandwidth <= 32 in 32-row blocks held in registers: lane l
 // keeps row J + l of the current block and row J + 32 + l of the next one.
 // Step q of a block broadcasts u = v(J + q) from lane q (a shuffle, the only
@@ -566,6 +478,9 @@ template <class FT>
 static void launch_band_solve_t(vtm_plan_s* P, FT* v, const FT* Lc, const FT* Uc, int ncols,
                                 int64_t stride, cudaStream_t s) {
   P->launch_count++;
+  // half bandwidths 33..256: blocks of 32 rows (bandblk.cu), 3.7-12 times the
+  // speed of the row-by-row kernel below, which stays for wider bands
+  if (launch_band_solve_blk(P, v, ncols, stride, s)) return;
   // FP32 only: the FP64 solve is bound by GB300's FP64 pipe either way (the
   // register-blocked form measured no faster for the 2048^2 power grid)
   if constexpr (sizeof(FT) == 4) {
@@ -585,20 +500,6 @@ static void launch_band_solve_t(vtm_plan_s* P, FT* v, const FT* Lc, const FT* Uc
       band_solve_reg_kernel<FT><<<P->nparts * ncols, 32, smem, s>>>(
           P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(), P->tabs.band_off.as<int64_t>(), Lc, Uc, v,
           stride, P->nparts);
-      return;
-    }
-  }
-  // FP32 only: an FP64 solve is bound by GB300's FP64 pipe, where the
-  // register-prefetch kernel (more resident warps) does better
-  if (sizeof(FT) == 4 && P->max_bw <= 64) {
-    const int B_max = P->max_bw + 1;
-    const size_t smem = ((size_t)((P->max_nodes + 1) & ~1) + (size_t)kBS * kBC * B_max) * sizeof(FT);
-    if (smem <= 200 * 1024) {
-      auto kern = P->max_bw <= 32 ? band_solve_stream_kernel<FT, 1> : band_solve_stream_kernel<FT, 2>;
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      kern<<<P->nparts * ncols, 32, smem, s>>>(P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(),
-                                                P->tabs.band_off.as<int64_t>(), Lc, Uc, v, stride, P->nparts,
-                                                P->max_nodes, B_max);
       return;
     }
   }
@@ -667,6 +568,10 @@ __global__ void convert_f32_kernel(const double* __restrict__ a, float* __restri
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     b[i] = (float)a[i];
+}
+
+void convert_f32(const double* a, float* b, int64_t n, cudaStream_t s) {
+  convert_f32_kernel<<<1216, 256, 0, s>>>(a, b, n);
 }
 
 __device__ __forceinline__ void store_low(float* p, double v) { *p = (float)v; }
@@ -867,6 +772,7 @@ extern "C" vtm_status vtm_factor(vtm_plan_t P) {
     convert_f32_kernel<<<1216, 256, 0, P->stream>>>(P->d_Uc.as<double>(), P->d_Uc32.as<float>(), ne);
     VTM_CUDA_TRY(cudaGetLastError());
   }
+  VTM_TRY(band_blk_prepare(P));
   if (P->general) {
     VTM_TRY(build_general_operators(P));
   } else {

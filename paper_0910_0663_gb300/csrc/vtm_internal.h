@@ -219,6 +219,9 @@ struct vtm_plan_s {
   vtm::DevBuf d_iperm;                     // int32[n] (batched solves)
   vtm::DevBuf d_Lc, d_Uc;                  // band factors (doubles)
   vtm::DevBuf d_Lc32, d_Uc32, d_v32;       // FP32 factor copies and work vector (inner solves)
+  // inverted 32 x 32 diagonal blocks of the factors (half bandwidths 33..256),
+  // first block of each tile, tiles longest first (bandblk.cu)
+  vtm::DevBuf d_bb_off, d_bb_order, d_bb_Li, d_bb_Ui, d_bb_Li32, d_bb_Ui32;
   vtm::DevBuf d_v32b;                      // second FP32 work vector (the recovery's right-hand side)
   // A in ELL form for the single-column residual ([k][n] values and columns,
   // row lengths): 0 not built, 1 built, 2 rows too uneven (CSR kernel)
@@ -366,5 +369,12 @@ int launch_residual(const int64_t* rowptr, const int32_t* col, const double* val
 // Launch helpers exported between translation units.
 void launch_band_solve(vtm_plan_s* P, double* v, int ncols, int64_t vec_stride, cudaStream_t s);
 void launch_band_solve32(vtm_plan_s* P, float* v, int ncols, int64_t vec_stride, cudaStream_t s);
+void convert_f32(const double* a, float* b, int64_t n, cudaStream_t s);
+
+// bandblk.cu (band solves of half bandwidths 33..256); the launchers return
+// false where the plan has no inverted blocks
+vtm_status band_blk_prepare(vtm_plan_s* P);
+bool launch_band_solve_blk(vtm_plan_s* P, double* v, int ncols, int64_t stride, cudaStream_t s);
+bool launch_band_solve_blk(vtm_plan_s* P, float* v, int ncols, int64_t stride, cudaStream_t s);
 
 }  // namespace vtm
