@@ -123,7 +123,7 @@ typedef struct {
                         2-3% of a solve */
   int sweep_kernel;  /* 0 (default): autotuned -- the first solve of each precision times
                         every sweep kernel that fits the plan's sub-circuits and keeps the
-                        fastest; 1: direct-load kernel; 2: bulk-copy staged kernel;
+                        fastest; 1: direct-load kernel, a tile's outputs in slabs; 2: bulk-copy staged kernel;
                         3: 16-byte vector-load kernel, 256 threads per tile;
                         4: the same with 128 threads (p <= 128 VEC);
                         5, 6: packed symmetric kernel, 128 threads per tile, up to 85 / 64

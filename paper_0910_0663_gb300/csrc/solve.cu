@@ -357,83 +357,6 @@ __device__ __forceinline__ double load_t(const double* p) { return __ldg(p); }
 __device__ __forceinline__ float load_t(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 __device__ __forceinline__ float load_t(const __half* p) { return __half2float(*p); }
 
-template <class TT, class WT>
-__global__ void __launch_bounds__(256) sweep_kernel(
-    const TT* __restrict__ T, const int64_t* __restrict__ T_off, const int32_t* __restrict__ T_ld,
-    const int32_t* __restrict__ port_off, const int32_t* __restrict__ order,
-    const int32_t* __restrict__ twin, const typename KdOf<WT>::type* __restrict__ kd,
-    const uint8_t* __restrict__ run, const WT* __restrict__ c, WT* __restrict__ state,
-    int64_t nports, SweepCtrl* __restrict__ ctrl, double* __restrict__ partials,
-    double* __restrict__ hist, int hist_len, int nparts) {
-  using AT = WT;  // accumulation type: FP64 for FP64 waves, FP32 otherwise
-  extern __shared__ unsigned char smem_raw[];
-  __shared__ int s_k, s_flag;
-  __shared__ bool s_last;
-  if (threadIdx.x == 0) {
-    s_k = *((volatile int*)&ctrl->k);
-    s_flag = *((volatile int*)&ctrl->flag);
-  }
-  __syncthreads();
-  if (s_flag) return;
-  const int k = s_k;
-  const int tile = order[blockIdx.x];
-  const int p0 = port_off[tile];
-  const int p = port_off[tile + 1] - p0;
-  WT* w_in = reinterpret_cast<WT*>(smem_raw);
-  AT* rs = reinterpret_cast<AT*>(smem_raw + sizeof(WT) * ((p + 1) & ~1));
-  const WT* prev = state + (size_t)((k - 1) & 1) * nports * 2;
-  WT* cur = state + (size_t)(k & 1) * nports * 2;
-  // gather the incident waves (delay 1) and the residual terms of sweep k-1
-  for (int s = threadIdx.x; s < p; s += blockDim.x) {
-    const int gs = p0 + s;
-    AT wi = 0, rc = 0;
-    if (k > 1) {
-      const int tw = twin[gs];
-      const AT wi_t = (AT)prev[2 * tw], wo_t = (AT)prev[2 * tw + 1];
-      const AT wi_s = (AT)prev[2 * gs], wo_s = (AT)prev[2 * gs + 1];
-      wi = wo_t;
-      rc = port_residual<AT>(wi_s, wo_s, wi_t, wo_t, kd[gs]);
-    }
-    w_in[s] = (WT)wi;
-    rs[s] = rc;
-  }
-  __syncthreads();
-  double sq = 0.0;
-  if (k > 1) {
-    for (int s = threadIdx.x; s < p; s += blockDim.x) {
-      const int nr = run[p0 + s];
-      if (nr) {
-        double r = 0.0;
-        for (int q = 0; q < nr; ++q) r += (double)rs[s + q];
-        sq += r * r;
-      }
-    }
-  }
-  const double tile_sq = block_sum_value(sq);
-  // apply the reflection matrix: w_out(s) = c(s) + sum_t T(s, t) w_in(t)
-  const TT* Tb = T + T_off[tile];
-  const int ld = T_ld[tile];
-  for (int s = threadIdx.x; s < p; s += blockDim.x) {
-    AT acc = (AT)c[p0 + s];
-    const TT* col = Tb + s;
-#pragma unroll 8
-    for (int t = 0; t < p; ++t) acc += (AT)load_t(col + (size_t)t * ld) * (AT)w_in[t];
-    cur[2 * (p0 + s)] = w_in[s];
-    cur[2 * (p0 + s) + 1] = (WT)acc;
-  }
-  // the last tile to finish reduces the residual of sweep k-1
-  if (threadIdx.x == 0) {
-    partials[tile] = tile_sq;
-    __threadfence();
-    s_last = atomicAdd(&ctrl->counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const double tot = block_sum_fixed(partials, nparts);
-  if (threadIdx.x == 0) sweep_decide(ctrl, k, tot, hist, hist_len);
-}
-
 // ---------------------------------------------------------------------------
 // the sweep with the reflection matrix staged by the bulk-copy engine
 // ---------------------------------------------------------------------------
@@ -929,6 +852,152 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// 16-byte asynchronous copies into shared memory, completing in groups
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Kernel 1: direct 16-byte loads of the full matrices.  A work item is a slab of
+// SW outputs of one tile: SW / VEC lanes hold VEC outputs each, the 256 threads'
+// G = 256 VEC / SW such groups take the inputs t = g, g + G, ... (each a
+// contiguous piece of row t of T_P^T), and the groups' partial sums are added
+// in a fixed order.  Slabs rather than whole tiles: the tiles of uneven plans
+// (up to 1584 ports beside 200) and plans with few tiles then still give every
+// SM the same bytes; the price is that each slab gathers all of its tile's
+// incident waves (4-8 bytes per input from L2, against SW elements of T).  SW is
+// the largest of 128, 64, 32 that gives four items per SM.  The first rows of
+// T, which need no waves, are loaded before the previous sweep is waited for
+// (programmatic dependent launch).
+// Bound by HBM for FP32 / 16 bits (the matrices once per sweep) and by the FP64
+// pipe for FP64.  Measured per FP32 sweep of a thermal grid in 150
+// boxes of up to 1584 ports (259 MB of T_P, 38 us at the copy bandwidth): one
+// CTA per tile 610 us, slabs with T in a register buffer of 8 loads 105 us
+// (scoreboard waits left two in flight), this ring 58 us.  FP64, 64 tiles of 256
+// ports: 26.4 -> 19 us.
+struct __align__(16) SlabItem {
+  int32_t p0, p, m0, ld;  // first port, ports, first output of the slab, row length
+  int64_t T_off;
+  int32_t pad[2];
+};
+
+constexpr int kSlabStages = 12;  // 16-byte loads in flight per thread
+
+template <class TT, class WT, int VEC>
+__global__ void __launch_bounds__(256, 3) sweep_slab_kernel(
+    const TT* __restrict__ T, const SlabItem* __restrict__ items, int lanes,
+    const int32_t* __restrict__ twin, const typename KdOf<WT>::type* __restrict__ kd,
+    const uint8_t* __restrict__ run, const WT* __restrict__ c, WT* __restrict__ state,
+    int64_t nports, SweepCtrl* __restrict__ ctrl, double* __restrict__ partials,
+    double* __restrict__ hist, int hist_len) {
+  using LD = VecLoadG<TT, VEC>;
+  using WP = typename KdOf<WT>::type;  // a (w_in, w_out) pair
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_k, s_flag;
+  __shared__ bool s_last;
+  const int tid = threadIdx.x;
+  const SlabItem it = items[blockIdx.x];
+  const int p0 = it.p0, p = it.p;
+  const int G = 256 / lanes, g = tid / lanes, l = tid % lanes;
+  const int SW = lanes * VEC;
+  const bool active = it.m0 + l * VEC < it.ld;  // rows are padded to whole vectors
+  const TT* Tb = T + it.T_off + it.m0 + l * VEC;
+  constexpr int ST = kSlabStages;
+  // stage b of this thread: 16 bytes of its own (it copies and reads them
+  // itself, so the ring needs no barrier)
+  uint4* ring = reinterpret_cast<uint4*>(smem_raw) + tid;
+  WT* red = reinterpret_cast<WT*>(smem_raw);  // [256 VEC], once the ring is done
+  WT* w_in = reinterpret_cast<WT*>(smem_raw + ST * 256 * 16);
+  int tn = g, sn = 0;  // next input and stage to load
+  auto issue = [&]() {
+    if (active && tn < p) cp_async16(ring + sn * 256, Tb + (size_t)tn * it.ld);
+    cp_async_commit_group();
+    tn += G;
+    sn = sn + 1 == ST ? 0 : sn + 1;
+  };
+#pragma unroll
+  for (int b = 0; b < ST - 1; ++b) issue();
+  pdl_launch_dependents();
+  pdl_wait();  // the previous sweep's waves, decision and counters
+  if (tid == 0) {
+    s_k = *((volatile int*)&ctrl->k);
+    s_flag = *((volatile int*)&ctrl->flag);
+  }
+  __syncthreads();
+  if (s_flag) {
+    cp_async_wait_group<0>();  // no copy into shared memory outlives the CTA
+    return;
+  }
+  const int k = s_k;
+  const WP* prev = reinterpret_cast<const WP*>(state) + (size_t)((k - 1) & 1) * nports;
+  WP* cur = reinterpret_cast<WP*>(state) + (size_t)(k & 1) * nports;
+  // incident waves of the tile (delay 1): the twins' outgoing waves
+  for (int s = tid; s < p; s += 256) w_in[s] = k > 1 ? prev[twin[p0 + s]].y : (WT)0;
+  // residual of sweep k - 1 at the nodes whose ports start in this slab
+  WT sq = 0;
+  if (k > 1) {
+    for (int s = it.m0 + tid; s < min(p, it.m0 + SW); s += 256) {
+      const int nr = run[p0 + s];
+      if (nr) {
+        WT r = 0;
+        for (int q = p0 + s; q < p0 + s + nr; ++q) {
+          const WP ws = prev[q], wt = prev[twin[q]];
+          r += port_residual<WT>(ws.x, ws.y, wt.x, wt.y, kd[q]);
+        }
+        sq += r * r;
+      }
+    }
+  }
+  __syncthreads();
+  WT acc[VEC];
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) acc[e] = 0;
+  int sl = 0;
+#pragma unroll 4
+  for (int t = g; t < p; t += G) {
+    issue();
+    cp_async_wait_group<ST - 1>();  // this thread's bytes of input t have landed
+    if (active) {
+      WT val[VEC];
+      LD::unpack(*reinterpret_cast<const typename LD::raw*>(ring + sl * 256), val);
+      const WT wt = w_in[t];
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) acc[e] += val[e] * wt;
+    }
+    sl = sl + 1 == ST ? 0 : sl + 1;
+  }
+  cp_async_wait_group<0>();
+  __syncthreads();  // the ring becomes the partial sums
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) red[g * SW + l * VEC + e] = acc[e];
+  const double slab_sq = sizeof(WT) == 8 ? block_sum_value((double)sq) : (double)block_sum_value_f((float)sq);
+  // (the sum's barriers stand between the partials and their readers)
+  if (tid < SW && it.m0 + tid < p) {
+    const int s = it.m0 + tid;
+    WT o = c[p0 + s];
+    for (int a = 0; a < G; ++a) o += red[a * SW + tid];
+    WP pair;
+    pair.x = w_in[s];
+    pair.y = o;
+    cur[p0 + s] = pair;
+  }
+  // the last slab to finish reduces the residual of sweep k - 1
+  if (tid == 0) {
+    partials[blockIdx.x] = slab_sq;
+    __threadfence();
+    s_last = atomicAdd(&ctrl->counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const double tot = block_sum_fixed(partials, gridDim.x);
+  if (tid == 0) sweep_decide(ctrl, k, tot, hist, hist_len);
+}
+
 // Incident waves of the tile (zero past p, the padding of the last block)
 // and this thread's share of the squared node residuals of sweep k - 1.
 template <int NT>
@@ -1235,14 +1304,6 @@ constexpr int kWflowWarps = 4;
 constexpr int kWflowCtasPerSm = 7;
 
 // 16-byte asynchronous copy global -> shared (L2 only), its groups and waits
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 // lane's share of one packed block: the bytes it later reads itself (SymLoad)
 template <class TT>
 __device__ __forceinline__ void copy_block_async(TT* dst, const TT* src, int lane) {
@@ -2583,14 +2644,34 @@ static void launch_packed(const vtm_plan_s* P, void (*kern)(KArgs...), int grid,
   cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-template <class TT, class WT>
-static void launch_sweep(vtm_plan_s* P, const TT* T, const WT* c, WT* state, int threads,
-                         size_t smem, double* hist, int hist_len) {
-  sweep_kernel<TT, WT><<<P->nparts, threads, smem, P->stream>>>(
-      T, P->tabs.T_off.as<int64_t>(), P->tabs.T_ld.as<int32_t>(), P->tabs.port_off.as<int32_t>(),
-      P->tabs.order.as<int32_t>(), P->d_twin.as<int32_t>(), kd_of<WT>(P), P->d_run.as<uint8_t>(), c,
-      state, (int64_t)P->port_node.size(), P->d_ctrl.as<SweepCtrl>(), P->d_partials.as<double>(), hist,
-      hist_len, P->nparts);
+// Work items of kernel 1, tiles with most ports first (once per plan and slab width).
+static vtm_status ensure_slabs(vtm_plan_s* P, int sw) {
+  if (P->slab_width == sw) return VTM_OK;
+  std::vector<int32_t> order(P->nparts);
+  for (int32_t t = 0; t < P->nparts; ++t) order[t] = t;
+  auto ports = [&](int32_t t) { return P->port_off[t + 1] - P->port_off[t]; };
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return ports(a) > ports(b); });
+  std::vector<SlabItem> items;
+  for (int32_t t : order)
+    for (int32_t m0 = 0; m0 < ports(t); m0 += sw)
+      items.push_back(SlabItem{P->port_off[t], ports(t), m0, P->T_ld[t], P->T_off[t], {0, 0}});
+  P->nslabs = (int)items.size();
+  VTM_TRY(upload(P->d_slabs, items, P->stream));
+  VTM_TRY(dev_alloc(P->d_slab_part, items.size() * sizeof(double)));
+  VTM_CUDA_TRY(cudaStreamSynchronize(P->stream));  // the host list is about to go
+  P->slab_width = sw;
+  return VTM_OK;
+}
+
+template <class TT, class WT, int VEC>
+static void launch_slab(vtm_plan_s* P, const TT* T, const WT* c, WT* state, double* hist, int hist_len) {
+  static_assert(256 * VEC * sizeof(WT) <= kSlabStages * 256 * 16, "the partial sums reuse the ring");
+  const size_t smem = kSlabStages * 256 * 16 + (size_t)P->max_ports * sizeof(WT) + 16;
+  cudaFuncSetAttribute(sweep_slab_kernel<TT, WT, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  launch_packed(P, sweep_slab_kernel<TT, WT, VEC>, P->nslabs, 256, smem, P->stream, T,
+                (const SlabItem*)P->d_slabs.as<SlabItem>(), P->slab_width / VEC,
+                (const int32_t*)P->d_twin.as<int32_t>(), kd_of<WT>(P), (const uint8_t*)P->d_run.as<uint8_t>(), c, state,
+                (int64_t)P->port_node.size(), P->d_ctrl.as<SweepCtrl>(), P->d_slab_part.as<double>(), hist, hist_len);
 }
 
 // Scoped access-policy window on the plan's stream over the FP32/16-bit
@@ -2680,9 +2761,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   h.bnorm2 = bnorm2 > 0 ? bnorm2 : 1.0;
   *P->h_ctrl = h;
   VTM_TRY(upload_ctrl(P, s));
-  const int threads = P->max_ports <= 64 ? 64 : (P->max_ports <= 128 ? 128 : 256);
-  size_t wsz = prec == VTM_PREC_FP64 ? sizeof(double) : sizeof(float);
-  size_t smem = (size_t)((P->max_ports + 2) & ~1) * wsz * 2 + 16;
+  const size_t wsz = prec == VTM_PREC_FP64 ? sizeof(double) : sizeof(float);
   if (prec == VTM_PREC_FP64) {
     VTM_CUDA_TRY(cudaMemsetAsync(P->d_state64.p, 0, 4 * npt * sizeof(double), s));
   } else {
@@ -2733,6 +2812,17 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   const bool symb_ok = sym_ok && symb_smem <= 160 * 1024;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device);
+  // kernel 1: the widest slab of outputs that still gives four items per SM
+  // (narrower ones re-read the incident waves for less of the matrix)
+  {
+    int sw = 128;
+    for (; sw > 32; sw /= 2) {
+      int64_t items = 0;
+      for (int32_t t = 0; t < P->nparts; ++t) items += (P->port_off[t + 1] - P->port_off[t] + sw - 1) / sw;
+      if (items >= 4 * (int64_t)sms) break;
+    }
+    VTM_TRY(ensure_slabs(P, sw));
+  }
   // one warp per tile: per warp a ring of blocks, w_in, residual terms and
   // outputs of the tile.  One CTA per SM holds ceil(nparts / SMs) tile warps
   // (at most 28, and what shared memory holds) and four service warps, so
@@ -2924,16 +3014,16 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
       return;
     }
     if (prec == VTM_PREC_FP64)
-      launch_sweep<double, double>(P, P->d_T64.as<double>(), P->d_c64.as<double>(),
-                                   P->d_state64.as<double>(), threads, smem, hist, hist_len);
+      launch_slab<double, double, 2>(P, P->d_T64.as<double>(), P->d_c64.as<double>(), P->d_state64.as<double>(),
+                                        hist, hist_len);
     else if (prec == VTM_PREC_FP32)
-      launch_sweep<float, float>(P, P->d_T32.as<float>(), P->d_c32.as<float>(),
-                                 P->d_state32.as<float>(), threads, smem, hist, hist_len);
+      launch_slab<float, float, 4>(P, P->d_T32.as<float>(), P->d_c32.as<float>(), P->d_state32.as<float>(), hist,
+                                      hist_len);
     else
       with16([&](auto h) {
         using H = decltype(h);
-        launch_sweep<H, float>(P, P->d_T16.as<H>(), P->d_c32.as<float>(), P->d_state32.as<float>(), threads,
-                               smem, hist, hist_len);
+        launch_slab<H, float, 8>(P, P->d_T16.as<H>(), P->d_c32.as<float>(), P->d_state32.as<float>(), hist,
+                                    hist_len);
       });
   };
   // Autotuner: on the first solve of this precision, time every kernel that

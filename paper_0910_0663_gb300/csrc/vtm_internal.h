@@ -240,6 +240,9 @@ struct vtm_plan_s {
   // partials of four sweeps, waves in three slots
   vtm::DevBuf d_nbr_off, d_nbr, d_done, d_flow, d_part4, d_fstate32;
   const void* wave_slot = nullptr;  // (w_in, w_out) pairs of the sweep the last inner solve ended on
+  // kernel 1: its work items (slabs of slab_width outputs) and their residual partials
+  vtm::DevBuf d_slabs, d_slab_part;
+  int slab_width = 0, nslabs = 0;
   vtm::DevBuf d_c64, d_c32;                // constant term of the sweep
   vtm::DevBuf d_state64, d_state32;        // [2][nports] (w_in, w_out) pairs
   vtm::DevBuf d_v, d_v2;                   // permuted work vectors [n]
