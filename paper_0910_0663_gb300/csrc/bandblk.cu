@@ -229,20 +229,24 @@ bool band_blk_eligible(const vtm_plan_s* P) { return P->max_bw > 32 && P->max_bw
 vtm_status band_blk_prepare(vtm_plan_s* P) {
   if (!band_blk_eligible(P)) return VTM_OK;
   cudaStream_t s = P->stream;
-  std::vector<int32_t> off(P->nparts + 1, 0), order(P->nparts);
-  for (int32_t t = 0; t < P->nparts; ++t) {
-    off[t + 1] = off[t] + (P->node_off[t + 1] - P->node_off[t] + kBbN - 1) / kBbN;
-    order[t] = t;
+  if (P->bb_blocks == 0) {
+    std::vector<int32_t> off(P->nparts + 1, 0), order(P->nparts);
+    for (int32_t t = 0; t < P->nparts; ++t) {
+      off[t + 1] = off[t] + (P->node_off[t + 1] - P->node_off[t] + kBbN - 1) / kBbN;
+      order[t] = t;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {  // largest tiles first
+      return P->node_off[a + 1] - P->node_off[a] > P->node_off[b + 1] - P->node_off[b];
+    });
+    VTM_TRY(upload(P->d_bb_off, off, s));
+    VTM_TRY(upload(P->d_bb_order, order, s));
+    VTM_CUDA_TRY(cudaStreamSynchronize(s));  // the host tables are about to go
+    P->bb_blocks = off[P->nparts];
   }
-  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {  // largest tiles first
-    return P->node_off[a + 1] - P->node_off[a] > P->node_off[b + 1] - P->node_off[b];
-  });
-  VTM_TRY(upload(P->d_bb_off, off, s));
-  VTM_TRY(upload(P->d_bb_order, order, s));
-  const int64_t ne = (int64_t)off[P->nparts] * kBbN * kBbN;
+  const int64_t ne = (int64_t)P->bb_blocks * kBbN * kBbN;
   VTM_TRY(dev_alloc(P->d_bb_Li, ne * sizeof(double)));
   VTM_TRY(dev_alloc(P->d_bb_Ui, ne * sizeof(double)));
-  band_inverse_kernel<<<dim3((off[P->nparts] + 3) / 4, 2), 128, 0, s>>>(
+  band_inverse_kernel<<<dim3((P->bb_blocks + 3) / 4, 2), 128, 0, s>>>(
       P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(), P->tabs.band_off.as<int64_t>(),
       P->d_bb_off.as<int32_t>(), P->nparts, P->d_Lc.as<double>(), P->d_Uc.as<double>(), P->d_bb_Li.as<double>(),
       P->d_bb_Ui.as<double>());
@@ -253,7 +257,6 @@ vtm_status band_blk_prepare(vtm_plan_s* P) {
     convert_f32(P->d_bb_Li.as<double>(), P->d_bb_Li32.as<float>(), ne, s);
     convert_f32(P->d_bb_Ui.as<double>(), P->d_bb_Ui32.as<float>(), ne, s);
   }
-  VTM_CUDA_TRY(cudaStreamSynchronize(s));  // the host tables are about to go
   return VTM_OK;
 }
 

@@ -2244,6 +2244,7 @@ static vtm_status batch_norms(vtm_plan_s* P, const double* x, const double* b, d
 vtm_status ensure_vals_df(vtm_plan_s* P) {
   if (P->vals_df_state != 0) return VTM_OK;
   bool ok = true;
+  VTM_TRY(ensure_host_vals(P));
   for (double v : P->h_vals) {
     int e = 0;
     if (!std::isfinite(v)) ok = false;

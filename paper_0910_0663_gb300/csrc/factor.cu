@@ -678,22 +678,22 @@ vtm_status build_reflections(vtm_plan_s* P) {
       set_detail("vtm_factor: a sub-circuit with more than 25600 nodes has ports; use more parts");
       return VTM_EINVAL;
     }
-    std::vector<int32_t> port_tile(npt);
-    for (int32_t t = 0; t < P->nparts; ++t)
-      for (int32_t q = P->port_off[t]; q < P->port_off[t + 1]; ++q) port_tile[q] = t;
-    DevBuf d_pt;
-    VTM_TRY(upload(d_pt, port_tile, s));
+    if (!P->d_port_tile.p) {
+      std::vector<int32_t> port_tile(npt);
+      for (int32_t t = 0; t < P->nparts; ++t)
+        for (int32_t q = P->port_off[t]; q < P->port_off[t + 1]; ++q) port_tile[q] = t;
+      VTM_TRY(upload(P->d_port_tile, port_tile, s));
+      VTM_CUDA_TRY(cudaStreamSynchronize(s));  // the host list is about to go
+    }
     VTM_CUDA_TRY(cudaFuncSetAttribute(build_reflection_kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     build_reflection_kernel<<<(unsigned)npt, 32, smem, s>>>(
         P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(), P->tabs.band_off.as<int64_t>(),
         P->d_Lc.as<double>(), P->d_Uc.as<double>(), P->tabs.port_off.as<int32_t>(),
-        d_pt.as<int32_t>(), P->d_port_loc.as<int32_t>(), P->d_beta.as<double>(),
+        P->d_port_tile.as<int32_t>(), P->d_port_loc.as<int32_t>(), P->d_beta.as<double>(),
         P->d_bout.as<double>(), P->d_rho.as<double>(), P->tabs.T_off.as<int64_t>(),
         P->tabs.T_ld.as<int32_t>(), P->d_T64.as<double>());
     VTM_CUDA_TRY(cudaGetLastError());
-    VTM_CUDA_TRY(cudaStreamSynchronize(s));
-    dev_free(d_pt);
   }
   const int64_t ne = std::max<int64_t>(P->T_elems, 8);
   if (P->opts.precision == VTM_PREC_FP32) {
@@ -755,10 +755,7 @@ extern "C" vtm_status vtm_factor(vtm_plan_t P) {
   dev_free(P->d_bk_Gf);
   dev_free(P->d_bk_Gb);
   P->bk_ready = false;
-  // the band arrays hold K_P before the factorisation: re-assemble if a
-  // previous factorisation overwrote them
-  static_assert(sizeof(double) == 8, "");
-  VTM_TRY(assemble_local(P));
+  VTM_TRY(assemble_band(P));  // a factorisation overwrites the band
   VTM_TRY(factor_tiles(P));
   if (P->opts.precision != VTM_PREC_FP64) {
     // FP32 copy of the factors for the right-hand-side preparation of the
@@ -800,6 +797,7 @@ extern "C" vtm_status vtm_get_reflection(vtm_plan_t P, int32_t part, double* T, 
   if (pp > 0)
     VTM_CUDA_TRY(cudaMemcpy(blk.data(), P->d_T64.as<double>() + P->T_off[part],
                             blk.size() * sizeof(double), cudaMemcpyDeviceToHost));
+  VTM_TRY(ensure_host_ports(P));
   // back from the plan's wave scaling: T_P(s, q) = d_s [D^-1 T_P D](s, q) / d_q
   const int32_t p0 = P->port_off[part];
   for (int32_t q = 0; q < pp; ++q)
@@ -849,6 +847,7 @@ extern "C" vtm_status vtm_get_reflection_stored(vtm_plan_t P, int32_t part, doub
   if (cap < (int64_t)pp * pp) return VTM_EINVAL;
   if (pp == 0) return VTM_OK;
   const int32_t p0 = P->port_off[part];
+  VTM_TRY(ensure_host_ports(P));
   auto unscale = [&](int32_t s, int32_t q) { return P->port_d[p0 + s] / P->port_d[p0 + q]; };
   if (is_packed) {
     // blocks (bi <= bj) row-major over (bi, bj); an FP32 block is row-major, a

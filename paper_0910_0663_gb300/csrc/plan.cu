@@ -251,12 +251,17 @@ static vtm_status build_structure(vtm_plan_s* P, std::vector<CutPair>& pairs) {
     cp.wire = P->method == VTM_METHOD_VTM && g > 0;
     double r1 = cp.wire ? a1 + g : a1;
     double r2 = cp.wire ? a2 + g : a2;
+    P->cut_p1.push_back(cp.pos_lohi);
+    P->cut_p2.push_back(cp.pos_hilo);
+    P->cut_flags.push_back((uint8_t)((cp.wire ? 1 : 0) | (r1 != 0.0 ? 2 : 0) | (r2 != 0.0 ? 4 : 0)));
     if (r1 != 0.0) {
+      P->lag_back.push_back(cp.pos_hilo);
       P->lag_i.push_back(cp.lo);
       P->lag_j.push_back(cp.hi);
       P->lag_pos.push_back(cp.pos_lohi);
     }
     if (r2 != 0.0) {
+      P->lag_back.push_back(cp.pos_lohi);
       P->lag_i.push_back(cp.hi);
       P->lag_j.push_back(cp.lo);
       P->lag_pos.push_back(cp.pos_hilo);
@@ -348,40 +353,6 @@ static vtm_status build_structure(vtm_plan_s* P, std::vector<CutPair>& pairs) {
   return VTM_OK;
 }
 
-// True if the current values give the same torn lines and the same set of
-// lagged positions as the ones the plan was built with.
-static bool same_cut_structure(const vtm_plan_s* P) {
-  std::vector<int64_t> wires, lags;
-  for (int64_t i = 0; i < P->n; ++i) {
-    for (int64_t q = P->h_rowptr[i]; q < P->h_rowptr[i + 1]; ++q) {
-      int32_t j = P->h_colidx[q];
-      if (P->h_part[j] == P->h_part[i]) continue;
-      int64_t back = csr_find(P, j, (int32_t)i);
-      if (i > j && back >= 0) continue;
-      int64_t p1 = i < j ? q : back, p2 = i < j ? back : q;
-      double a1 = val_at(P, p1), a2 = val_at(P, p2);
-      double g = -(a1 + a2) / 2.0;
-      bool wire = P->method == VTM_METHOD_VTM && g > 0;
-      if (wire) wires.push_back(p1 >= 0 ? p1 : p2);
-      double r1 = wire ? a1 + g : a1, r2 = wire ? a2 + g : a2;
-      if (r1 != 0.0) lags.push_back(p1);
-      if (r2 != 0.0) lags.push_back(p2);
-    }
-  }
-  std::vector<int64_t> w0, l0;
-  for (size_t s = 0; s < P->port_node.size(); ++s)
-    if (P->port_node[s] < P->port_remote[s])
-      w0.push_back(P->port_pos_ij[s] >= 0 ? P->port_pos_ij[s] : P->port_pos_ji[s]);
-  for (size_t q = 0; q < P->lag_pos.size(); ++q) l0.push_back(P->lag_pos[q]);
-  std::sort(wires.begin(), wires.end());
-  std::sort(lags.begin(), lags.end());
-  std::sort(w0.begin(), w0.end());
-  std::sort(l0.begin(), l0.end());
-  // a lagged entry may vanish (rho = 0) but no new one may appear
-  if (wires != w0) return false;
-  return std::includes(l0.begin(), l0.end(), lags.begin(), lags.end());
-}
-
 // Diagonal of the partial input admittance S~ = C - E~ D~^-1 F~ of every port
 // (Sec. VIII, choice 5): D~ is D_P = A_PP + sum_s g_s e_l e_l^T restricted to
 // the nodes of the sub-circuit within `radius` branches of the port's node;
@@ -389,8 +360,12 @@ static bool same_cut_structure(const vtm_plan_s* P) {
 static vtm_status schur_diag_ports(vtm_plan_s* P, int radius, std::vector<double>& S) {
   const size_t npt = P->port_node.size();
   S.assign(npt, 0.0);
-  std::vector<double> gsum(P->n, 0.0);
-  for (size_t s = 0; s < npt; ++s) gsum[P->port_node[s]] += P->port_g[s];
+  VTM_TRY(ensure_host_vals(P));
+  std::vector<double> gsum(P->n, 0.0), port_g(npt);
+  for (size_t s = 0; s < npt; ++s) {
+    port_g[s] = -(val_at(P, P->port_pos_ij[s]) + val_at(P, P->port_pos_ji[s])) / 2.0;
+    gsum[P->port_node[s]] += port_g[s];
+  }
   std::vector<int32_t> mark(P->n, -1), sel;
   std::vector<double> D, z;
   for (size_t s = 0; s < npt; ++s) {
@@ -456,181 +431,33 @@ static vtm_status schur_diag_ports(vtm_plan_s* P, int radius, std::vector<double
       for (int k = c + 1; k < m; ++k) acc -= D[(size_t)c * m + k] * z[k];
       z[c] = acc / D[(size_t)c * m + c];
     }
-    const double g = P->port_g[s];
+    const double g = port_g[s];
     S[s] = 2 * g - 4 * g * g * z[0];
   }
   return VTM_OK;
 }
 
-// Admittance of every line from the plan's choice (Sec. VIII); both ports of
-// a line get the same value.
-static vtm_status line_admittance(vtm_plan_s* P) {
+// Admittances that the host forms or holds (SCA, or the caller's own): both
+// ports of a line get the same value.  The others follow from the conductances
+// on the device (assemble.cu).
+vtm_status host_admittance(vtm_plan_s* P, std::vector<double>& W) {
+  if (P->w_kind == VTM_W_LINE) {
+    W = P->w_user;
+    return VTM_OK;
+  }
+  if (P->w_kind != VTM_W_SCA) return VTM_EINVAL;
+  if (P->w_sca.empty()) {
+    std::vector<double> S;
+    VTM_TRY(schur_diag_ports(P, P->w_radius, S));
+    P->w_sca = std::move(S);
+  }
   const size_t npt = P->port_node.size();
-  P->port_W.assign(npt, P->W);
-  switch (P->w_kind) {
-    case VTM_W_ALPHA:
-      break;
-    case VTM_W_DIAG:
-      for (size_t s = 0; s < npt; ++s) P->port_W[s] = 2.0 * P->port_g[s];
-      break;
-    case VTM_W_WOB:
-      for (size_t s = 0; s < npt; ++s) P->port_W[s] = P->w_alpha * 2.0 * P->port_g[s];
-      break;
-    case VTM_W_SCA: {
-      std::vector<double> S;
-      VTM_TRY(schur_diag_ports(P, P->w_radius, S));
-      for (size_t s = 0; s < npt; ++s) {
-        const int32_t tw = P->port_twin[s];
-        const bool low = P->h_part[P->port_node[s]] <= P->h_part[P->port_node[tw]];
-        P->port_W[s] = low ? S[s] : S[tw];
-      }
-      break;
-    }
-    case VTM_W_LINE:
-      P->port_W = P->w_user;
-      break;
-    default:
-      return VTM_EINVAL;
-  }
-  for (size_t s = 0; s < npt; ++s)
-    if (!(P->port_W[s] > 0) || !std::isfinite(P->port_W[s])) {
-      set_detail("line admittance not positive at port " + std::to_string(s));
-      return VTM_EINVAL;
-    }
-  return VTM_OK;
-}
-
-// Values: branch conductances, line admittances, the per-port coefficients,
-// lagged couplings and the band of K_P.
-vtm_status assemble_local(vtm_plan_s* P) {
-  const int32_t np = P->nparts;
-  const size_t npt = P->port_node.size();
-  P->port_g.resize(npt);
+  W.resize(npt);
   for (size_t s = 0; s < npt; ++s) {
-    double g = -(val_at(P, P->port_pos_ij[s]) + val_at(P, P->port_pos_ji[s])) / 2.0;
-    if (!(g > 0)) {
-      set_detail("vtm_set_values: a torn branch lost its positive conductance");
-      return VTM_EINVAL;
-    }
-    P->port_g[s] = g;
+    const int32_t tw = P->port_twin[s];
+    const bool low = P->h_part[P->port_node[s]] <= P->h_part[P->port_node[tw]];
+    W[s] = low ? P->w_sca[s] : P->w_sca[tw];
   }
-  if (P->w_dirty || P->port_W.size() != npt) {
-    VTM_TRY(line_admittance(P));
-    P->w_dirty = false;
-  }
-  // waves are carried as w / d_s with d_s = sqrt(W_s / W_ref): for one W on
-  // every line d = 1; otherwise d = sqrt(W_s) (power waves), which keeps the
-  // condensed operator symmetric for a symmetric A
-  const bool scalar_w = P->w_kind == VTM_W_ALPHA;
-  std::vector<double> beta(npt), bin(npt), bout(npt), rho(npt), kd(2 * npt);
-  std::vector<float> kd32(2 * npt);
-  std::vector<float> kddf(4 * npt);  // (g/W, d) as double-float pairs (kernel 12)
-  P->port_d.assign(npt, 1.0);
-  for (size_t s = 0; s < npt; ++s) {
-    const double g = P->port_g[s], W = P->port_W[s];
-    const double d = scalar_w ? 1.0 : std::sqrt(W);
-    P->port_d[s] = d;
-    beta[s] = 2 * g / (2 * g + W);
-    bin[s] = scalar_w ? beta[s] : beta[s] * d;
-    bout[s] = scalar_w ? 2.0 * W * beta[s] : 2.0 * W * beta[s] / d;
-    rho[s] = (W - 2.0 * g) / (W + 2.0 * g);
-    kd[2 * s] = g / W;
-    kd[2 * s + 1] = d;
-    kd32[2 * s] = (float)(g / W);
-    kd32[2 * s + 1] = (float)d;
-    kddf[4 * s] = (float)(g / W);
-    kddf[4 * s + 1] = (float)(g / W - (double)kddf[4 * s]);
-    kddf[4 * s + 2] = (float)d;
-    kddf[4 * s + 3] = (float)(d - (double)kddf[4 * s + 2]);
-  }
-  P->lag_rho.resize(P->lag_i.size());
-  for (size_t q = 0; q < P->lag_i.size(); ++q) {
-    // remainder after the branch part (if the pair carries a line)
-    int32_t i = P->lag_i[q], j = P->lag_j[q];
-    int64_t pji = csr_find(P, j, i);
-    double a = val_at(P, P->lag_pos[q]);
-    double g = -(a + val_at(P, pji)) / 2.0;
-    P->lag_rho[q] = (P->method == VTM_METHOD_VTM && g > 0) ? a + g : a;
-  }
-  std::vector<double> Lc(P->band_elems, 0.0), Uc;
-  if (!P->symmetric) Uc.assign(P->band_elems, 0.0);
-  for (int32_t t = 0; t < np; ++t) {
-    const int32_t B = P->bw[t] + 1;
-    const int32_t off = P->node_off[t];
-    const int32_t cnt = P->node_off[t + 1] - off;
-    double* lc = Lc.data() + P->band_off[t];
-    double* uc = P->symmetric ? nullptr : Uc.data() + P->band_off[t];
-    for (int32_t l = 0; l < cnt; ++l) {
-      int32_t i = P->perm[off + l];
-      for (int64_t q = P->h_rowptr[i]; q < P->h_rowptr[i + 1]; ++q) {
-        int32_t j = P->h_colidx[q];
-        if (P->h_part[j] != t) continue;
-        int32_t m = P->iperm[j] - off;
-        if (m <= l) {
-          lc[(int64_t)m * B + (l - m)] += P->h_vals[q];
-        } else if (uc) {
-          uc[(int64_t)m * B + (m - l)] += P->h_vals[q];
-        }
-      }
-    }
-    for (int32_t s = P->port_off[t]; s < P->port_off[t + 1]; ++s) {
-      const double g = P->port_g[s], W = P->port_W[s];
-      lc[(int64_t)P->port_loc[s] * B] += g - 4 * g * g / (2 * g + W);
-    }
-  }
-  cudaStream_t st = P->stream;
-  // (+ 64 bytes: the bulk copies of the band solves round their last chunk up
-  // to a 16-byte multiple)
-  VTM_TRY(dev_alloc(P->d_Lc, Lc.size() * sizeof(double) + 64));
-  VTM_TRY(dev_alloc(P->d_Uc, Lc.size() * sizeof(double) + 64));
-  VTM_TRY(upload(P->d_Lc, Lc, st));
-  if (!P->symmetric) VTM_TRY(upload(P->d_Uc, Uc, st));
-  VTM_TRY(upload(P->d_beta, bin, st));
-  VTM_TRY(upload(P->d_bout, bout, st));
-  // FP32 copies for the port-wise kernels of the low-precision batched path
-  {
-    std::vector<float> b32(bin.begin(), bin.end()), o32(bout.begin(), bout.end());
-    VTM_TRY(upload(P->d_beta32, b32, st));
-    VTM_TRY(upload(P->d_bout32, o32, st));
-    VTM_CUDA_TRY(cudaStreamSynchronize(st));  // the host vectors are about to go
-  }
-  VTM_TRY(upload(P->d_rho, rho, st));
-  VTM_TRY(upload(P->d_kd, kd, st));
-  VTM_TRY(upload(P->d_kd32, kd32, st));
-  VTM_TRY(upload(P->d_kddf, kddf, st));
-  if (P->general) {
-    // per input: residual coefficients (g/W and d of a port, rho of a lagged
-    // entry) and right-hand-side weight (beta d or -rho); per output: scale
-    // (2 W beta / d or 1) and the diagonal reflection term of a port
-    std::vector<double> coef(P->n_in), dsc(P->n_in, 0.0), sigma(P->n_in), scale(P->n_out),
-        diag(P->n_out, 0.0);
-    for (int64_t a = 0; a < P->n_in; ++a) {
-      const int32_t it = P->in_item[a];
-      if (P->in_kind[a] == 0) {
-        coef[a] = kd[2 * it];
-        dsc[a] = kd[2 * it + 1];
-        sigma[a] = bin[it];
-      } else {
-        coef[a] = P->lag_rho[it];
-        sigma[a] = -P->lag_rho[it];
-      }
-    }
-    for (int64_t o = 0; o < P->n_out; ++o) {
-      const int32_t it = P->out_item[o];
-      if (it >= 0) {
-        scale[o] = bout[it];
-        diag[o] = rho[it];
-      } else {
-        scale[o] = 1.0;
-      }
-    }
-    VTM_TRY(upload(P->d_in_coef, coef, st));
-    VTM_TRY(upload(P->d_in_d, dsc, st));
-    VTM_TRY(upload(P->d_in_sigma, sigma, st));
-    VTM_TRY(upload(P->d_out_scale, scale, st));
-    VTM_TRY(upload(P->d_out_diag, diag, st));
-  }
-  VTM_CUDA_TRY(cudaStreamSynchronize(st));
   return VTM_OK;
 }
 
@@ -792,7 +619,8 @@ using namespace vtm;
 
 std::vector<DevBuf*> vtm_plan_s::all_bufs() {
   return {&tabs.node_off, &tabs.bw, &tabs.band_off, &tabs.port_off, &tabs.T_off, &tabs.T_ld,
-          &tabs.order, &d_rowptr, &d_colidx, &d_vals, &d_perm, &d_iperm, &d_Lc, &d_Uc, &d_Lc32, &d_Uc32, &d_v32, &d_v32b, &d_bb_off, &d_bb_order, &d_bb_Li, &d_bb_Ui, &d_bb_Li32, &d_bb_Ui32, &d_slabs, &d_slab_part, &d_ell_val, &d_ell_col, &d_ell_len,
+          &tabs.order, &d_rowptr, &d_colidx, &d_vals, &d_perm, &d_iperm, &d_Lc, &d_Uc, &d_Lc32, &d_Uc32, &d_v32, &d_v32b, &d_bb_off, &d_bb_order, &d_bb_Li, &d_bb_Ui, &d_bb_Li32, &d_bb_Ui32, &d_slabs, &d_slab_part, &d_cut_p1, &d_cut_p2, &d_cut_flags, &d_ppij, &d_ppji, &d_port_g, &d_port_W, &d_port_d,
+          &d_lag_pos, &d_lag_back, &d_lag_rho, &d_in_item, &d_out_item, &d_vals_new, &d_port_tile, &d_ell_val, &d_ell_col, &d_ell_len,
           &d_port_loc, &d_port_pos, &d_tdesc,
           &d_twin, &d_beta, &d_bout, &d_beta32, &d_bout32, &d_rho, &d_kd, &d_kd32, &d_run, &d_T64, &d_T32, &d_T16, &d_Tp32, &d_Tp16, &d_Tpdf, &d_dfstate, &d_cdf, &d_kddf, &d_nbr_off, &d_nbr, &d_done, &d_flow, &d_part4, &d_fstate32, &d_c64, &d_c32, &d_state64,
           &d_state32, &d_v, &d_v2, &d_xacc, &d_r, &d_bcol, &d_partials, &d_ctrl, &d_hist,
@@ -860,16 +688,18 @@ extern "C" vtm_status vtm_set_admittance(vtm_plan_t P, int kind, double alpha, i
   P->w_radius = radius;
   P->w_user = std::move(user);
   if (kind == VTM_W_ALPHA) P->W = alpha;
-  P->w_dirty = true;
-  vtm_status st = assemble_local(P);
+  P->w_sca.clear();
+  vtm_status st = assemble_ports(P);
   if (st != VTM_OK) {
     P->w_kind = o_kind;
     P->w_alpha = o_alpha;
     P->w_radius = o_radius;
     P->w_user = std::move(o_user);
     P->W = o_W;
-    P->w_dirty = true;
-    assemble_local(P);
+    P->w_sca.clear();
+    const std::string why = g_detail;
+    assemble_ports(P);
+    set_detail(why);
     return st;
   }
   P->factored = false;
@@ -884,6 +714,7 @@ extern "C" vtm_status vtm_get_admittance(vtm_plan_t P, double* W) {
   if (!P || !W) return VTM_EINVAL;
   const size_t npt = P->port_node.size();
   if (npt == 0) return VTM_OK;
+  VTM_TRY(ensure_host_ports(P));
   if (is_device_ptr(W)) {
     VTM_CUDA_TRY(cudaMemcpy(W, P->port_W.data(), npt * sizeof(double), cudaMemcpyHostToDevice));
   } else {
@@ -1096,52 +927,43 @@ extern "C" vtm_status vtm_plan(int64_t n, const int64_t* rowptr, const int32_t* 
   if (cudaEventCreate(&P->ev0) != cudaSuccess || cudaEventCreate(&P->ev1) != cudaSuccess ||
       cudaEventCreate(&P->evs0) != cudaSuccess || cudaEventCreate(&P->evs1) != cudaSuccess)
     return fail(VTM_ECUDA);
-  if ((st = assemble_local(P)) != VTM_OK) return fail(st);
+  // the band of K_P, assembled by vtm_factor (+ 64 bytes: the bulk copies of the
+  // band solves round their last chunk up to a 16-byte multiple)
+  if ((st = dev_alloc(P->d_Lc, P->band_elems * sizeof(double) + 64)) != VTM_OK) return fail(st);
+  if ((st = dev_alloc(P->d_Uc, P->band_elems * sizeof(double) + 64)) != VTM_OK) return fail(st);
+  if ((st = assemble_ports(P)) != VTM_OK) return fail(st);
   *out = P;
   return VTM_OK;
 }
 
 extern "C" vtm_status vtm_set_values(vtm_plan_t P, const double* vals) {
   if (!P || !vals) return VTM_EINVAL;
-  std::vector<double> old = P->h_vals;
-  vtm_status st = fetch(P->h_vals, vals, (size_t)P->nnz);
-  if (st != VTM_OK) return st;
-  for (double v : P->h_vals)
-    if (!std::isfinite(v)) {
-      P->h_vals = old;
-      set_detail("vtm_set_values: non-finite value");
-      return VTM_EINVAL;
-    }
-  if (P->symmetric) {
-    for (int64_t i = 0; i < P->n; ++i)
-      for (int64_t q = P->h_rowptr[i]; q < P->h_rowptr[i + 1]; ++q) {
-        int32_t j = P->h_colidx[q];
-        if (j <= i) continue;
-        int64_t t = csr_find(P, j, (int32_t)i);
-        if (t < 0 || P->h_vals[t] != P->h_vals[q]) {
-          P->h_vals = old;
-          set_detail("vtm_set_values: the plan was made for a symmetric matrix");
-          return VTM_EINVAL;
-        }
-      }
-  }
-  // the torn lines and the lagged couplings must stay the same
-  if (!same_cut_structure(P)) {
-    P->h_vals = old;
-    set_detail("vtm_set_values: the set of torn lines or lagged couplings changed");
-    return VTM_EINVAL;
-  }
-  P->w_dirty = true;
-  st = assemble_local(P);
+  cudaSetDevice(P->device);
+  cudaStream_t s = P->stream;
+  const size_t bytes = (size_t)P->nnz * sizeof(double);
+  VTM_TRY(dev_alloc(P->d_vals_new, bytes));
+  // the values may come from the plan's stream or from the default stream: the
+  // copy follows both
+  VTM_CUDA_TRY(cudaStreamSynchronize(s));
+  VTM_CUDA_TRY(cudaMemcpyAsync(P->d_vals_new.p, vals, bytes, cudaMemcpyDefault, cudaStreamLegacy));
+  VTM_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
+  // finite, symmetric where the plan is, the same torn lines and couplings
+  VTM_TRY(check_values(P, P->d_vals_new.as<double>()));
+  std::swap(P->d_vals, P->d_vals_new);
+  const bool host_vals = P->host_vals;
+  P->host_vals = false;
+  std::vector<double> w_sca;
+  std::swap(w_sca, P->w_sca);
+  vtm_status st = assemble_ports(P);
   if (st != VTM_OK) {
-    P->h_vals = old;
-    P->w_dirty = true;
-    assemble_local(P);
+    std::swap(P->d_vals, P->d_vals_new);
+    std::swap(w_sca, P->w_sca);
+    const std::string why = g_detail;
+    P->host_vals = host_vals && P->w_kind != VTM_W_SCA;  // (SCA read the refused values)
+    assemble_ports(P);
+    set_detail(why);
     return st;
   }
-  VTM_CUDA_TRY(cudaMemcpyAsync(P->d_vals.p, P->h_vals.data(), P->nnz * sizeof(double),
-                               cudaMemcpyHostToDevice, P->stream));
-  VTM_CUDA_TRY(cudaStreamSynchronize(P->stream));
   P->factored = false;
   dev_free(P->d_vals_df);
   P->vals_df_state = 0;
@@ -1166,7 +988,7 @@ extern "C" vtm_status vtm_plan_get_stats(vtm_plan_t P, vtm_plan_stats* s) {
   s->symmetric = P->symmetric ? 1 : 0;
   s->t_bytes = (int64_t)(P->d_T64.bytes + P->d_T32.bytes + P->d_T16.bytes + P->d_E.bytes +
                          P->d_Tp32.bytes + P->d_Tp16.bytes + P->d_Tpdf.bytes);
-  s->factor_bytes = (int64_t)(P->d_Lc.bytes + P->d_Uc.bytes);
+  s->factor_bytes = 2 * P->band_elems * (int64_t)sizeof(double);
   s->sweep_kernel = P->opts.method == VTM_METHOD_ASYNC   ? P->dataflow_kernel
                     : P->tuned_kernel[P->opts.precision] ? P->tuned_kernel[P->opts.precision]
                                                          : P->opts.sweep_kernel;

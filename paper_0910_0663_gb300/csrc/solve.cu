@@ -3396,8 +3396,11 @@ static vtm_status norms(vtm_plan_s* P, const double* x, const double* b, double*
 // stays under half of the nonzeros (else the CSR kernel serves)
 static vtm_status ensure_ell(vtm_plan_s* P) {
   if (P->ell_state != 0) return VTM_OK;
-  int64_t maxlen = 0;
-  for (int64_t i = 0; i < P->n; ++i) maxlen = std::max(maxlen, P->h_rowptr[i + 1] - P->h_rowptr[i]);
+  if (P->max_row < 0) {  // once per plan: the pattern stays
+    P->max_row = 0;
+    for (int64_t i = 0; i < P->n; ++i) P->max_row = std::max(P->max_row, P->h_rowptr[i + 1] - P->h_rowptr[i]);
+  }
+  const int64_t maxlen = P->max_row;
   if (maxlen < 1 || maxlen > 8 || P->n * maxlen > P->nnz + P->nnz / 2) {
     P->ell_state = 2;
     return VTM_OK;
@@ -3846,6 +3849,8 @@ extern "C" vtm_status vtm_adjoint(vtm_plan_t P, const double* g, double* lam, in
   if (!P->factored) return VTM_ENOTFACTORED;
   if (!P->transposed) {
     // A^T in CSR = A in CSC
+    VTM_TRY(ensure_host_vals(P));
+    VTM_TRY(ensure_host_ports(P));
     const int64_t n = P->n;
     std::vector<int64_t> rp(n + 1, 0);
     std::vector<int32_t> ci(P->nnz);

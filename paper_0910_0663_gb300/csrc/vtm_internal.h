@@ -165,7 +165,9 @@ struct vtm_plan_s {
   int w_radius = 2;
   std::vector<double> w_user;
   std::vector<double> port_W, port_d;
-  bool w_dirty = true;  // port_W to be recomputed from the current values
+  std::vector<double> w_sca;  // SCA: partial Schur diagonals of the current values (empty: to be formed)
+  // the host's copies of the values (h_vals) and of port_g, port_W, port_d are current
+  bool host_vals = true, host_ports = false;
   vtm_opts opts{};
   cudaStream_t stream = nullptr;
   bool symmetric = true;
@@ -198,10 +200,15 @@ struct vtm_plan_s {
   std::vector<double> port_g;        // branch conductance
   std::vector<uint8_t> port_run;     // ports left in this node's run (>=1) at a run start, else 0
 
+  // cut pairs: CSR positions (-1: no entry) and flags (1 line, 2 / 4 first / second entry lagged)
+  std::vector<int64_t> cut_p1, cut_p2, lag_back;  // lag_back: position of the opposite entry
+  std::vector<uint8_t> cut_flags;
+  vtm::DevBuf d_cut_p1, d_cut_p2, d_cut_flags, d_ppij, d_ppji, d_port_g, d_port_W, d_port_d, d_lag_pos,
+      d_lag_back, d_lag_rho, d_in_item, d_out_item, d_vals_new, d_port_tile;
+
   // lagged couplings (cut entries that are not branches), by row
   std::vector<int32_t> lag_i, lag_j;
   std::vector<int64_t> lag_pos;
-  std::vector<double> lag_rho;
 
   // reflection-matrix layout
   std::vector<int32_t> T_ld;
@@ -222,11 +229,13 @@ struct vtm_plan_s {
   // inverted 32 x 32 diagonal blocks of the factors (half bandwidths 33..256),
   // first block of each tile, tiles longest first (bandblk.cu)
   vtm::DevBuf d_bb_off, d_bb_order, d_bb_Li, d_bb_Ui, d_bb_Li32, d_bb_Ui32;
+  int bb_blocks = 0;
   vtm::DevBuf d_v32b;                      // second FP32 work vector (the recovery's right-hand side)
   // A in ELL form for the single-column residual ([k][n] values and columns,
   // row lengths): 0 not built, 1 built, 2 rows too uneven (CSR kernel)
   vtm::DevBuf d_ell_val, d_ell_col, d_ell_len;
   int ell_state = 0, ell_k = 0;
+  int64_t max_row = -1;  // longest row of A
   vtm::DevBuf d_port_loc, d_port_pos, d_twin, d_beta, d_run, d_tdesc;  // d_beta: beta d
   vtm::DevBuf d_bout, d_rho, d_kd, d_kd32;  // per port: 2 W beta / d, reflection, (g/W, d)
   vtm::DevBuf d_beta32, d_bout32;           // FP32 copies of beta d and 2 W beta / d
@@ -341,7 +350,14 @@ vtm_status upload(DevBuf& b, const std::vector<T>& h, cudaStream_t s) {
 bool is_device_ptr(const void* p);
 
 // plan.cu
-vtm_status assemble_local(vtm_plan_s* P);  // host band values of K_P + port tables -> device
+vtm_status host_admittance(vtm_plan_s* P, std::vector<double>& W);
+
+// assemble.cu (values on the device)
+vtm_status check_values(vtm_plan_s* P, const double* d_vals);
+vtm_status assemble_ports(vtm_plan_s* P);
+vtm_status assemble_band(vtm_plan_s* P);
+vtm_status ensure_host_vals(vtm_plan_s* P);
+vtm_status ensure_host_ports(vtm_plan_s* P);
 
 // general.cu (channel form: lagged couplings and block Jacobi)
 vtm_status build_general_operators(vtm_plan_s* P);
