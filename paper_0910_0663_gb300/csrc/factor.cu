@@ -5,7 +5,8 @@
 // right-looking band Cholesky (symmetric A) or band LU without pivoting,
 // one CTA per sub-circuit, with the active (bw+1) x (bw+1) window in shared
 // memory addressed circularly.  The factors are stored column-wise:
-//   Lc[j][a] = L(j+a, j) / L(j, j), a = 1..bw;  Lc[j][0] = 1 / L(j, j)
+//   Lc[j][a] = L(j+a, j) / L(j, j), a = 1..bw;  Lc[j][0] = 1 / L(j, j)   (Cholesky; the
+// panel factorisation keeps Lc[j][0] = 1/L(j, j)^2 and Uc[j][0] = 1 instead)
 //   Uc[j][b] = U(j-b, j) / U(j, j), b = 1..bw;  Uc[j][0] = 1 / U(j, j)
 // (multipliers divided by the pivot: see band.cuh) so that both triangular
 // solves are column sweeps with contiguous reads and one FMA per step.
@@ -121,16 +122,246 @@ __global__ void __launch_bounds__(256) band_factor_kernel(const int32_t* __restr
   if (bad && tid == 0) atomicMax(err, t + 1);
 }
 
+// The same factorisation in panels of 16 columns, for windows that fit shared
+// memory.  As LDL^T / LU: multipliers l(i, q) = a(i, q) / piv_q, and
+//   Lc[j][a] = l(j+a, j), Lc[j][0] = 1/piv_j (symmetric) or 1 (LU)
+//   Uc[j][b] = l(j, j-b), Uc[j][0] = 1       (symmetric)
+//            = u(j-b, j)/piv_j, Uc[j][0] = 1/piv_j (LU)
+// which the solves read like the Cholesky form (y = u Lc[j][0] between the
+// passes).  One CTA per tile keeps the band columns j0 .. j0 + bw + 15 in shared
+// memory by column (slot j mod (bw + 16), element i - j).  Per panel: warp 0
+// factors the 16 x 16 diagonal block in registers; a thread per row (and, for
+// LU, per column) below it eliminates its 16 entries; the panel goes out to
+// global memory; and the bw x bw trailing window takes one rank-16 update in
+// 4 x 4 register tiles while the next 16 columns arrive by cp.async.
+// Bound by the FP64 pipe (2 FMA per clock and SM): bw^2/2 FMA per column
+// (symmetric).  The column-by-column kernel above spent about 6 us per column
+// on three barriers and integer divisions.  Measured: 256 tiles of 4096 rows, bw 64:
+// 24.7 -> 10.0 ms (pipe 5.9 ms); 256 tiles of 1024 rows, bw 32: 3.2 -> 1.9 ms.  It stays for bands
+// whose window does not fit (half bandwidths above about 140, LU 102).
+constexpr int kFpN = 16;  // columns per panel
+
+__host__ __device__ constexpr int fp_rows(int bw) { return (bw + kFpN + 5) / 2 * 2; }
+__host__ __device__ constexpr size_t fp_smem(int bw, bool lu) {
+  return sizeof(double) * ((size_t)(lu ? 2 : 1) * (bw + kFpN) * (bw + 1) + 2 * (size_t)kFpN * fp_rows(bw));
+}
+
+__device__ __forceinline__ void cp_async8(double* smem, const double* gmem) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+
+template <bool kLU>
+__global__ void __launch_bounds__(256, 2) band_factor_panel_kernel(
+    const int32_t* __restrict__ node_off, const int32_t* __restrict__ bwv, const int64_t* __restrict__ band_off,
+    double* __restrict__ Lc, double* __restrict__ Uc, int* __restrict__ err) {
+  extern __shared__ __align__(16) double fsm[];
+  __shared__ double D[kFpN * (kFpN + 1)];  // the diagonal block: l below, u on and above the diagonal
+  __shared__ double pinv[kFpN];
+  __shared__ int s_bad;
+  constexpr int N = kFpN, DS = kFpN + 1;
+  const int t = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+  const int n = node_off[t + 1] - node_off[t], bw = bwv[t], B = bw + 1, C = bw + N, RS = fp_rows(bw);
+  double* lc = Lc + band_off[t];
+  double* uc = Uc + band_off[t];
+  double* XL = fsm;           // l(r, q) at [q RS + r], r relative to the panel
+  double* XU = XL + N * RS;   // u(q, r)
+  double* Lw = XU + N * RS;   // window, lower part
+  double* Uw = Lw + (size_t)C * B;  // upper part (LU)
+  for (int e = tid; e < min(n, C) * B; e += nt) {
+    Lw[e] = lc[e];
+    if (kLU) Uw[e] = uc[e];
+  }
+  if (tid == 0) s_bad = 0;
+  __syncthreads();
+  for (int j0 = 0; j0 < n; j0 += N) {
+    const int nc = min(N, n - j0), R = min(n - j0, C);
+    const int s0 = j0 % C;
+    auto slot = [&](int r) {  // of column j0 + r
+      const int s = s0 + r;
+      return (s >= C ? s - C : s) * B;
+    };
+    if (tid < 32) {
+      const int r = tid;
+      double x[N];
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        x[q] = 0.0;
+        if (r < nc && q < nc) {
+          if (q <= r) {
+            if (r - q <= bw) x[q] = Lw[slot(q) + r - q];
+          } else if (q - r <= bw) {
+            x[q] = kLU ? Uw[slot(q) + q - r] : Lw[slot(r) + q - r];
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        if (q < nc) {
+          double piv = __shfl_sync(0xffffffffu, x[q], q);
+          const bool bad = kLU ? !(fabs(piv) > 0.0) : !(piv > 0.0);
+          if (bad || !isfinite(piv)) {
+            if (r == 0) s_bad = 1;
+            piv = 1.0;
+          }
+          const double pi = 1.0 / piv;
+          if (r == q) pinv[q] = pi;
+          if (r > q) x[q] *= pi;
+          const double l = r > q ? x[q] : 0.0;
+#pragma unroll
+          for (int c = q + 1; c < N; ++c) x[c] -= l * __shfl_sync(0xffffffffu, x[c], q);
+        }
+      }
+      if (r < N)
+#pragma unroll
+        for (int q = 0; q < N; ++q) D[r * DS + q] = x[q];
+    }
+    __syncthreads();
+    // rows (and, for LU, columns) below the diagonal block
+    const int M = R - nc;
+    for (int e = tid; e < (kLU ? 2 * M : M); e += nt) {
+      const bool up = kLU && e >= M;
+      const int r = nc + (up ? e - M : e);
+      double x[N];
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        x[q] = 0.0;
+        if (q < nc && r - q <= bw) x[q] = up ? Uw[slot(r) + r - q] : Lw[slot(q) + r - q];
+      }
+      if (!up) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+          asm volatile("" ::: "memory");  // D's rows are read as they are used
+          if (q < nc) {
+            const double l = x[q] * pinv[q];
+            if (!kLU) XU[q * RS + r] = x[q];
+            XL[q * RS + r] = l;
+#pragma unroll
+            for (int c = q + 1; c < N; ++c) x[c] -= l * D[q * DS + c];
+          }
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+          asm volatile("" ::: "memory");
+          if (q < nc) {
+            XU[q * RS + r] = x[q];
+            if (r - q <= bw) Uw[slot(r) + r - q] = x[q];
+#pragma unroll
+            for (int c = q + 1; c < N; ++c) x[c] -= D[c * DS + q] * x[q];
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // the panel to global memory
+    auto l_at = [&](int r, int q) { return r < nc ? D[r * DS + q] : XL[q * RS + r]; };
+    for (int e = tid; e < nc * B; e += nt) {
+      const int q = e / B, a = e - q * B, r = q + a;
+      if (r < R) lc[(size_t)(j0 + q) * B + a] = a == 0 ? (kLU ? 1.0 : pinv[q]) : l_at(r, q);
+      if (kLU && a <= j0 + q)
+        uc[(size_t)(j0 + q) * B + a] = a == 0 ? pinv[q] : (a <= q ? D[(q - a) * DS + q] : Uw[slot(q) + a]) * pinv[q];
+    }
+    if (!kLU)
+      for (int e = tid; e < R * N; e += nt) {
+        const int r = e / N, q = e % N;  // 16 consecutive elements of column j0 + r of Uc
+        if (q < nc && q <= r && r - q <= bw) uc[(size_t)(j0 + r) * B + r - q] = q == r ? 1.0 : l_at(r, q);
+      }
+    __syncthreads();  // the panel's slots are free
+    if (M > 0) {
+      const int cin = min(N, n - (j0 + C));  // columns j0 + C .. take the panel's slots
+      for (int e = tid; e < cin * B; e += nt) {
+        const int q = e / B, a = e - q * B;
+        cp_async8(Lw + slot(q) + a, lc + (size_t)(j0 + C + q) * B + a);
+        if (kLU) cp_async8(Uw + slot(q) + a, uc + (size_t)(j0 + C + q) * B + a);
+      }
+      // trailing window, rows and columns N .. R - 1, in 4 x 4 tiles
+      const int T = (M + 3) / 4, ntile = kLU ? T * T : T * (T + 1) / 2;
+      for (int e = tid; e < ntile; e += nt) {
+        int ti, tj;
+        if (kLU) {
+          ti = e / T;
+          tj = e - ti * T;
+        } else {  // row ti of the lower triangle starts at ti (ti + 1) / 2
+          ti = (int)((sqrtf(8.f * e + 1.f) - 1.f) * 0.5f);
+          while (ti * (ti + 1) / 2 > e) --ti;
+          while ((ti + 1) * (ti + 2) / 2 <= e) ++ti;
+          tj = e - ti * (ti + 1) / 2;
+        }
+        const int i0 = N + 4 * ti, c0 = N + 4 * tj;
+        double acc[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+#pragma unroll 4
+        for (int q = 0; q < N; ++q) {
+          const double2 l01 = *reinterpret_cast<const double2*>(XL + q * RS + i0);
+          const double2 l23 = *reinterpret_cast<const double2*>(XL + q * RS + i0 + 2);
+          const double2 u01 = *reinterpret_cast<const double2*>(XU + q * RS + c0);
+          const double2 u23 = *reinterpret_cast<const double2*>(XU + q * RS + c0 + 2);
+          const double l[4] = {l01.x, l01.y, l23.x, l23.y}, u[4] = {u01.x, u01.y, u23.x, u23.y};
+#pragma unroll
+          for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) acc[a][b] += l[a] * u[b];
+        }
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const int c = c0 + b;
+          if (c >= R) break;
+          const int sc = slot(c);
+#pragma unroll
+          for (int a = 0; a < 4; ++a) {
+            const int i = i0 + a;
+            if (i >= R) break;
+            if (i >= c) Lw[sc + i - c] -= acc[a][b];
+            else if (kLU) Uw[sc + c - i] -= acc[a][b];
+          }
+        }
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+    }
+  }
+  if (s_bad && tid == 0) atomicMax(err, t + 1);
+}
+
+// a pivot that failed in any tile, once the factorisation has finished
+static vtm_status factor_status(vtm_plan_s* P) {
+  VTM_CUDA_TRY(cudaGetLastError());
+  int herr = 0;
+  VTM_CUDA_TRY(cudaMemcpyAsync(&herr, P->d_err.p, sizeof(int), cudaMemcpyDeviceToHost, P->stream));
+  VTM_CUDA_TRY(cudaStreamSynchronize(P->stream));
+  if (herr) {
+    set_detail("vtm_factor: bad pivot in sub-circuit " + std::to_string(herr - 1));
+    return VTM_ESINGULAR;
+  }
+  return VTM_OK;
+}
+
 vtm_status factor_tiles(vtm_plan_s* P) {
   cudaStream_t s = P->stream;
   const int Bmax = P->max_bw + 1;
+  VTM_CUDA_TRY(cudaMemsetAsync(P->d_err.p, 0, sizeof(int), s));
+  const size_t panel = fp_smem(P->max_bw, !P->symmetric);
+  if (panel <= 222 * 1024) {
+    const int threads = P->max_bw <= 48 ? 128 : 256;
+    auto go = [&](auto* kern) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel);
+      kern<<<P->nparts, threads, panel, s>>>(P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(),
+                                             P->tabs.band_off.as<int64_t>(), P->d_Lc.as<double>(),
+                                             P->d_Uc.as<double>(), P->d_err.as<int>());
+    };
+    if (P->symmetric) go(band_factor_panel_kernel<false>);
+    else go(band_factor_panel_kernel<true>);
+    return factor_status(P);
+  }
   size_t win_bytes = (size_t)Bmax * Bmax * sizeof(double);
   size_t vec_bytes = 2 * (size_t)Bmax * sizeof(double);
   DevBuf gwin;
   bool use_smem = win_bytes + vec_bytes <= 200 * 1024;
   size_t smem = use_smem ? win_bytes + vec_bytes : vec_bytes;
   if (!use_smem) VTM_TRY(dev_alloc(gwin, (size_t)P->nparts * win_bytes));
-  VTM_CUDA_TRY(cudaMemsetAsync(P->d_err.p, 0, sizeof(int), s));
   int threads = Bmax <= 40 ? 128 : 256;
   if (P->symmetric) {
     VTM_CUDA_TRY(cudaFuncSetAttribute(band_factor_kernel<false>,
@@ -145,16 +376,9 @@ vtm_status factor_tiles(vtm_plan_s* P) {
         P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(), P->tabs.band_off.as<int64_t>(),
         P->d_Lc.as<double>(), P->d_Uc.as<double>(), gwin.as<double>(), Bmax, P->d_err.as<int>());
   }
-  VTM_CUDA_TRY(cudaGetLastError());
-  int herr = 0;
-  VTM_CUDA_TRY(cudaMemcpyAsync(&herr, P->d_err.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-  VTM_CUDA_TRY(cudaStreamSynchronize(s));
+  const vtm_status st = factor_status(P);
   dev_free(gwin);
-  if (herr) {
-    set_detail("vtm_factor: bad pivot in sub-circuit " + std::to_string(herr - 1));
-    return VTM_ESINGULAR;
-  }
-  return VTM_OK;
+  return st;
 }
 
 // ---------------------------------------------------------------------------
@@ -672,12 +896,12 @@ vtm_status build_reflections(vtm_plan_s* P) {
   const size_t Tbytes = std::max<int64_t>(P->T_elems, 8) * sizeof(double);
   VTM_TRY(dev_alloc(P->d_T64, Tbytes));
   VTM_CUDA_TRY(cudaMemsetAsync(P->d_T64.p, 0, Tbytes, s));
+  const size_t smem = (size_t)P->max_nodes * sizeof(double);
+  if (npt > 0 && smem > 200 * 1024) {
+    set_detail("vtm_factor: a sub-circuit with more than 25600 nodes has ports; use more parts");
+    return VTM_EINVAL;
+  }
   if (npt > 0) {
-    size_t smem = (size_t)P->max_nodes * sizeof(double);
-    if (smem > 200 * 1024) {
-      set_detail("vtm_factor: a sub-circuit with more than 25600 nodes has ports; use more parts");
-      return VTM_EINVAL;
-    }
     if (!P->d_port_tile.p) {
       std::vector<int32_t> port_tile(npt);
       for (int32_t t = 0; t < P->nparts; ++t)
