@@ -901,7 +901,10 @@ vtm_status build_reflections(vtm_plan_s* P) {
     set_detail("vtm_factor: a sub-circuit with more than 25600 nodes has ports; use more parts");
     return VTM_EINVAL;
   }
-  if (npt > 0) {
+  // 32 ports at a time for symmetric plans (reflect.cu); else a warp per port
+  if (reflect_blk_eligible(P)) {
+    VTM_TRY(build_reflections_blk(P));
+  } else if (npt > 0) {
     if (!P->d_port_tile.p) {
       std::vector<int32_t> port_tile(npt);
       for (int32_t t = 0; t < P->nparts; ++t)

@@ -230,6 +230,9 @@ struct vtm_plan_s {
   // first block of each tile, tiles longest first (bandblk.cu)
   vtm::DevBuf d_bb_off, d_bb_order, d_bb_Li, d_bb_Ui, d_bb_Li32, d_bb_Ui32;
   int bb_blocks = 0;
+  // reflection build: work items, ports of each tile by row, forward results
+  vtm::DevBuf d_refl_items, d_refl_order, d_refl_scratch;
+  int refl_items = 0;
   vtm::DevBuf d_v32b;                      // second FP32 work vector (the recovery's right-hand side)
   // A in ELL form for the single-column residual ([k][n] values and columns,
   // row lengths): 0 not built, 1 built, 2 rows too uneven (CSR kernel)
@@ -389,6 +392,10 @@ int launch_residual(const int64_t* rowptr, const int32_t* col, const double* val
 void launch_band_solve(vtm_plan_s* P, double* v, int ncols, int64_t vec_stride, cudaStream_t s);
 void launch_band_solve32(vtm_plan_s* P, float* v, int ncols, int64_t vec_stride, cudaStream_t s);
 void convert_f32(const double* a, float* b, int64_t n, cudaStream_t s);
+
+// reflect.cu
+bool reflect_blk_eligible(const vtm_plan_s* P);
+vtm_status build_reflections_blk(vtm_plan_s* P);
 
 // bandblk.cu (band solves of half bandwidths 33..256); the launchers return
 // false where the plan has no inverted blocks
