@@ -170,8 +170,8 @@ typedef struct {
                         accumulators in TMEM).  A tensor-core request in another
                         precision, or (2, 4) with a column count that is not a
                         multiple of 8, runs the CUDA-core variant */
-  int wait_polls;    /* polls a bounded device-side wait of the dataflow sweeps
-                        (kernels 8 and 10) makes before it gives up with VTM_ETIMEOUT;
+  int wait_polls;    /* polls a bounded device-side wait of the sweeps that run in one
+                        launch (kernels 8 and 10, and the resident form) makes before it gives up with VTM_ETIMEOUT;
                         0: default 4194304 (a few seconds).  The bulk-copy waits of
                         kernels 2 and 7 keep their own limit: a CTA never leaves while a
                         copy into its shared memory is in flight */
@@ -212,7 +212,11 @@ typedef struct {
   int32_t symmetric;     /* 1: A symmetric -> Cholesky; 0: LU without pivoting */
   int64_t t_bytes;       /* bytes of the stored reflection matrices (all precisions kept) */
   int64_t factor_bytes;  /* bytes of the stored local factors */
-  int32_t sweep_kernel;  /* sweep kernel in use for the plan's precision (see vtm_opts) */
+  int32_t sweep_kernel;  /* sweep kernel in use for the plan's precision (see vtm_opts); 8 also
+                            stands for the resident form the autotuner may pick on plans of
+                            few sub-circuits: every sweep of an inner solve in one launch,
+                            blocks in shared memory, a grid barrier per sweep (bounded by
+                            wait_polls) or one CTA */
   int64_t sum_tri;       /* sum over sub-circuits of p_P (p_P + 1) / 2: the entries of the
                             symmetric reflection matrices on and above the diagonal */
   int64_t packed_bytes;  /* bytes of the packed symmetric copies (0 if none) */

@@ -2602,6 +2602,12 @@ __global__ void __launch_bounds__(32 * kWflowWarps, kWflowCtasPerSm) sweep_wflow
   }
 }
 
+}  // namespace vtm
+
+#include "resident.cuh"
+
+namespace vtm {
+
 // ---------------------------------------------------------------------------
 // host driver
 // ---------------------------------------------------------------------------
@@ -2854,16 +2860,110 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   const int wdf_grid = (P->nparts + wdf_warps - 1) / wdf_warps;
   const int wdf_threads = 32 * (wdf_warps + 4);
   const size_t wdf_smem = wdf_warps * wdf_per_warp;
-  if (wdf_ok) {
-    VTM_TRY(dev_alloc(P->d_dfstate, 3 * (size_t)std::max<int64_t>(npt, 1) * sizeof(float4)));
+  // kernel 13 (every sweep in one launch, blocks in shared memory): packed
+  // copies, at most 15 tiles per SM (FP64: 11) and what its warps and shared memory hold
+  ResArgs ra{};
+  bool res_ok = false, res_local = false;
+  size_t res_smem = 0;
+  int res_grid = 0, res_threads = 0;
+  if ((prec == VTM_PREC_FP64 ? P->d_Tpdf.p != nullptr : sym_ok) && P->opts.sweep_kernel == 0 &&
+      P->opts.method != VTM_METHOD_ASYNC) {
+    const int nblk_max = nb_max * (nb_max + 1) / 2;
+    const int blk = prec == VTM_PREC_FP64 ? ResMode<double>::kBlkBytes : kSymB * kSymB * (int)s_t;
+    constexpr size_t kMax = 224 * 1024;
+    // one CTA where it holds the full matrices
+    const int pr = (P->max_ports + 31) / 32 * 32;
+    if (P->nparts * (pr / 32) <= kSmallRows && npt <= kSmallPorts) {
+      res_smem = prec == VTM_PREC_FP64 ? small_bytes<double>(pr, P->nparts, npt) : small_bytes<float>(pr, P->nparts, npt);
+      res_local = res_ok = res_smem <= kMax;
+      res_grid = 1;
+      res_threads = 32 * (P->nparts * (pr / 32) + kSmallSide + 1);
+      ra.pp = pr;
+    }
+    if (!res_ok) {
+      res_grid = std::min(P->nparts, sms);
+      ra.tpc = (P->nparts + res_grid - 1) / res_grid;
+      const int most = res_warps(prec == VTM_PREC_FP64);
+      if (ra.tpc <= most) {
+        ra.wpt = most / ra.tpc;
+        ra.pp = pp_max;
+        const int warps = ra.tpc * ra.wpt;
+        const size_t b = prec == VTM_PREC_FP64 ? res_base_bytes<double>(pp_max, ra.tpc, warps)
+                                               : res_base_bytes<float>(pp_max, ra.tpc, warps);
+        if (b <= kMax && pp_max <= 128 * ra.wpt && (int64_t)budget * res_grid < (1ll << 31) && budget < (1 << 27)) {
+          ra.nres = std::min((nblk_max + ra.wpt - 1) / ra.wpt, (int)((kMax - b) / ((size_t)warps * blk)));
+          res_smem = b + (size_t)warps * ra.nres * blk;
+          res_threads = 32 * (warps + 1);
+          res_ok = true;
+        }
+      }
+    }
+  }
+  // the instance for this precision, form and ports per lane
+  auto with_res = [&](auto fn) {
+    auto pick = [&](auto t) {
+      using T = decltype(t);
+      if (res_local) fn(sweep_small_kernel<T>);
+      else if (pp_max <= 64 * ra.wpt) fn(sweep_resident_kernel<T, 2>);
+      else fn(sweep_resident_kernel<T, 4>);
+    };
+    if (prec == VTM_PREC_FP64) pick(double{});
+    else if (prec == VTM_PREC_FP32) pick(float{});
+    else with16(pick);
+  };
+  if (res_ok) {
+    int coop = 0, per_sm = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, P->device);
+    with_res([&](auto* kern) {
+      res_ok = coop &&
+               cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem) == cudaSuccess &&
+               cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, res_threads, res_smem) ==
+                   cudaSuccess &&
+               per_sm >= 1;
+    });
+    cudaGetLastError();
+  }
+  if (res_ok) {
+    VTM_TRY(dev_alloc(P->d_res, 64 + 2 * (size_t)res_grid * sizeof(double)));
+    if (prec != VTM_PREC_FP64) VTM_TRY(dev_alloc(P->d_fstate32, 2 * kResSlots * (size_t)std::max<int64_t>(npt, 1) * sizeof(float)));
+  }
+  if (wdf_ok || (res_ok && prec == VTM_PREC_FP64)) {
+    VTM_TRY(dev_alloc(P->d_dfstate, kResSlots * (size_t)std::max<int64_t>(npt, 1) * sizeof(float4)));
     VTM_TRY(dev_alloc(P->d_cdf, (size_t)std::max<int64_t>(npt, 1) * sizeof(float2)));
     split_df_kernel<<<grid_for(std::max<int64_t>(npt, 1)), 256, 0, s>>>(P->d_c64.as<double>(),
                                                                         P->d_cdf.as<float2>(), npt);
     VTM_CUDA_TRY(cudaGetLastError());
     P->launch_count++;
-    VTM_CUDA_TRY(cudaFuncSetAttribute(sweep_wdf_kernel<kWdfKB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)wdf_smem));
+    if (wdf_ok)
+      VTM_CUDA_TRY(cudaFuncSetAttribute(sweep_wdf_kernel<kWdfKB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)wdf_smem));
   }
+  if (res_ok) {
+    ra.Tp = prec == VTM_PREC_FP64 ? P->d_Tpdf.p : prec == VTM_PREC_FP32 ? P->d_Tp32.p : P->d_Tp16.p;
+    ra.tdesc = P->d_tdesc.as<TileDesc>();
+    ra.twin = P->d_twin.as<int32_t>();
+    ra.kd = prec == VTM_PREC_FP64 ? P->d_kddf.p : P->d_kd32.p;
+    ra.run = P->d_run.as<uint8_t>();
+    ra.c = prec == VTM_PREC_FP64 ? P->d_cdf.p : P->d_c32.p;
+    ra.state3 = prec == VTM_PREC_FP64 ? P->d_dfstate.p : P->d_fstate32.p;
+    ra.nports = npt;
+    ra.ctrl = P->d_ctrl.as<SweepCtrl>();
+    ra.bar = reinterpret_cast<unsigned long long*>(P->d_res.p);
+    ra.part = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(P->d_res.p) + 64);
+    ra.hist = hist;
+    ra.hist_len = hist_len;
+    ra.nparts = P->nparts;
+    ra.max_polls = (uint32_t)P->opts.wait_polls;
+  }
+  auto launch_resident = [&]() -> cudaError_t {
+    cudaMemsetAsync(P->d_res.p, 0, 64, s);
+    cudaError_t e = cudaSuccess;
+    with_res([&](auto* kern) {
+      void* args[] = {&ra};
+      e = cudaLaunchCooperativeKernel((const void*)kern, dim3(res_grid), dim3(res_threads), args, res_smem, s);
+    });
+    return e;
+  };
   auto with_wsym = [&](auto fn) {
     const bool wide = pp_max > 128;
     if (prec == VTM_PREC_FP32) {
@@ -3192,21 +3292,23 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
       const bool can_vec128 = nv_max <= 128;
       float best = 1e30f;
       int best_k = 1;
-      for (int cand = 1; cand <= 12; ++cand) {
+      for (int cand = 1; cand <= 13; ++cand) {
         if ((cand == 2 && !can_st) || (cand == 3 && !can_vec) || (cand == 4 && !can_vec128) ||
             ((cand == 5 || cand == 6 || cand == 9) && !sym_ok) || (cand == 7 && !symb_ok) ||
             (cand == 8 && !flow_ok) || (cand == 10 && !wflow_ok) || (cand == 11 && !wmma_ok) ||
-            (cand == 12 && !wdf_ok))
+            (cand == 12 && !wdf_ok) || (cand == 13 && !res_ok))
           continue;
-        if (cand == 8 || cand == 10) {  // one launch of 8 sweeps, per-sweep time against the others' 6
+        if (cand == 8 || cand == 10 || cand == 13) {  // one launch, per-sweep time against the others' 6
           SweepCtrl t = h;
-          t.k_max = 8;
+          // (kernel 13 fills shared memory first: more sweeps to set against that)
+          const int nsw = cand == 13 ? 48 : 8;
+          t.k_max = nsw;
           t.tol2 = -1.0;
           t.stall = 0;
           *P->h_ctrl = t;
           VTM_TRY(upload_ctrl(P, s));
           VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
-          VTM_CUDA_TRY(cand == 10 ? launch_wflow() : launch_flow());
+          VTM_CUDA_TRY(cand == 13 ? launch_resident() : cand == 10 ? launch_wflow() : launch_flow());
           VTM_CUDA_TRY(cudaEventRecord(P->evs1, s));
           VTM_CUDA_TRY(cudaEventSynchronize(P->evs1));
           float ms = 0.f;
@@ -3217,8 +3319,8 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
             set_detail("vtm_solve: a bounded wait of the dataflow sweeps ran out");
             return VTM_ETIMEOUT;
           }
-          if (ms * 6.0f / 8.0f < best) {
-            best = ms * 6.0f / 8.0f;
+          if (ms * 6.0f / nsw < best) {
+            best = ms * 6.0f / nsw;
             best_k = cand;
           }
           continue;
@@ -3249,6 +3351,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
       P->tuned_kernel[prec] = best_k;
       P->tuned_ms[prec] = best / 6.0f;
       // back to the initial state of this inner solve
+      if (hist) VTM_CUDA_TRY(cudaMemsetAsync(hist, 0, hist_len * sizeof(double), s));
       *P->h_ctrl = h;
       VTM_TRY(upload_ctrl(P, s));
       if (prec == VTM_PREC_FP64)
@@ -3265,10 +3368,20 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, staged_kfn, st_threads, st_smem);
     st_grid = std::max(1, std::min(P->nparts, std::max(per_sm, 1) * sms));
   }
-  P->dataflow_kernel = kern;
-  if (kern == 8 || kern == 10) {
+  if (kern == 8 || kern == 10) P->dataflow_kernel = kern;
+  // the chosen double-float slot as FP64 pairs for the recovery
+  auto join_df = [&]() -> vtm_status {
+    join_df_kernel<<<grid_for(std::max<int64_t>(npt, 1)), 256, 0, s>>>(
+        P->d_dfstate.as<float4>() + (size_t)(*sweep_out % (kern == 13 ? kResSlots : 3)) * npt,
+        P->d_state64.as<double>(), npt);
+    VTM_CUDA_TRY(cudaGetLastError());
+    P->launch_count++;
+    P->wave_slot = P->d_state64.as<double>();
+    return VTM_OK;
+  };
+  if (kern == 8 || kern == 10 || kern == 13) {
     VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
-    VTM_CUDA_TRY(kern == 10 ? launch_wflow() : launch_flow());
+    VTM_CUDA_TRY(kern == 13 ? launch_resident() : kern == 10 ? launch_wflow() : launch_flow());
     VTM_CUDA_TRY(cudaEventRecord(P->evs1, s));
     VTM_CUDA_TRY(cudaMemcpyAsync(P->h_ctrl, P->d_ctrl.p, sizeof(SweepCtrl), cudaMemcpyDeviceToHost, s));
     VTM_CUDA_TRY(cudaStreamSynchronize(s));
@@ -3284,8 +3397,10 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
     }
     *flag_out = r.flag;
     *sweep_out = (r.flag == 1 || r.flag == 4) ? r.conv_sweep : std::min(r.k - 1, budget);
+    if (kern == 13 && prec == VTM_PREC_FP64) return join_df();
+    const int slots = kern == 13 ? kResSlots : 3;
     P->wave_slot = P->d_fstate32.as<float>() +
-                   (P->opts.method == VTM_METHOD_ASYNC ? 0 : (size_t)(*sweep_out % 3) * npt * 2);
+                   (P->opts.method == VTM_METHOD_ASYNC ? 0 : (size_t)(*sweep_out % slots) * npt * 2);
     return VTM_OK;
   }
   // Batches of check_every launches, captured once into a CUDA graph when the
@@ -3371,12 +3486,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   if (r.flag == 1 || r.flag == 4) *sweep_out = r.conv_sweep;
   else *sweep_out = std::min(r.k - 1, budget);
   if (kern == 12) {
-    // the chosen double-float slot as FP64 pairs for the recovery
-    join_df_kernel<<<grid_for(std::max<int64_t>(npt, 1)), 256, 0, s>>>(
-        P->d_dfstate.as<float4>() + (size_t)(*sweep_out % 3) * npt, P->d_state64.as<double>(), npt);
-    VTM_CUDA_TRY(cudaGetLastError());
-    P->launch_count++;
-    P->wave_slot = P->d_state64.as<double>();
+    return join_df();
   } else if (prec == VTM_PREC_FP64)
     P->wave_slot = P->d_state64.as<double>() + (size_t)(*sweep_out & 1) * npt * 2;
   else if (kern == 9 || kern == 11)  // three slots

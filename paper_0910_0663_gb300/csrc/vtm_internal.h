@@ -255,6 +255,7 @@ struct vtm_plan_s {
   // kernel 1: its work items (slabs of slab_width outputs) and their residual partials
   vtm::DevBuf d_slabs, d_slab_part;
   int slab_width = 0, nslabs = 0;
+  vtm::DevBuf d_res;  // kernel 13: barrier word, residual partials of two sweeps
   vtm::DevBuf d_c64, d_c32;                // constant term of the sweep
   vtm::DevBuf d_state64, d_state32;        // [2][nports] (w_in, w_out) pairs
   vtm::DevBuf d_v, d_v2;                   // permuted work vectors [n]

@@ -1,0 +1,79 @@
+"""Sweeps of an inner solve in one launch (the resident form the autotuner picks
+for plans of few sub-circuits; it reports as kernel 8): one SM and a grid barrier.
+
+Bars as for the other sweep kernels: FP64 histories within 1e-8 of the oracle's
+(1e-13 absolute), low precision within the rounding of the stored T_P, iterates
+after k sweeps within 1e-12.  A residual term is a difference of FP32 waves in the
+low precisions: six roundings (u = 2^-24) of at most (1 + g/W) 4 |w|, g/W <= 2, and
+|w| <= (W + 2 g) |x| 2 <= 10 |x|, so a history entry carries up to
+720 u |x|_max sqrt(ports) / |b| on top."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import vtm_oracle as O
+from paper_0910_0663_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+# (grid, tile): one SM -- 2 tiles, 16 tiles of 32 ports, 7 tiles of 33..64 ports;
+# grid barrier -- 9 and 25 ragged tiles, 6 tiles of up to 256 ports (streamed
+# blocks), 400 tiles (several per SM)
+ONE = [((1, 6), (1, 3)), ((32, 32), (8, 8)), ((17, 119), (17, 17))]
+GRID = [((50, 50), (17, 19)), ((90, 90), (18, 18)), ((128, 192), (64, 64)), ((240, 240), (12, 12))]
+
+
+def _plan(shape, precision, **kw):
+    from paper_0910_0663_gb300 import vtm
+    (ny, nx), (th, tw) = shape
+    w = wl.grid2d(ny, nx, th, tw, ground=0.05, seed=7)
+    return w, vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts, precision=precision, **kw)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("shape", ONE + GRID)
+def test_histories_follow_the_oracle(shape, precision):
+    w, plan = _plan(shape, precision)
+    A = w.csr()
+    b = torch.from_numpy(w.b[0]).cuda()
+    plan.set_options(history_len=40)
+    x, _ = plan.solve(b, tol=1e-10)
+    h = plan.history
+    x2, _ = plan.solve(b, tol=1e-10)
+    assert torch.equal(x, x2) and np.array_equal(h, plan.history)  # fixed order of every sum
+    assert O.residual_norms(A, x.cpu().numpy()[None], w.b[:1]).max() <= 1e-10
+    if precision == "fp64":  # only the resident form reports 8 on an FP64 plan
+        assert plan.stats()["sweep_kernel"] == 8
+    ref = O.vtm_midpoint(A, w.partition, w.nparts, w.b[:1], W=1 / w.Zc, tol=0, max_sweeps=40)
+    href = ref.history[:, 0]
+    rtol, floor, kmax = {"fp64": (1e-8, 1e-9, 40), "fp32": (1e-3, 1e-4, 40), "fp16": (2e-2, 5e-3, 20),
+                         "bf16": (5e-2, 2e-2, 15)}[precision]
+    k = min(kmax, int(np.count_nonzero((h > 0) & (href[: len(h)] > floor))))
+    assert k >= 1
+    u32 = 720 * 2.0 ** -24 * float(x.abs().max()) * plan.stats()["nports"] ** 0.5 / np.linalg.norm(w.b[0])
+    assert np.allclose(h[:k], href[:k], rtol=rtol, atol=1e-13 if precision == "fp64" else u32)
+
+
+@pytest.mark.parametrize("shape", [ONE[1], GRID[1]])
+@pytest.mark.parametrize("k", [1, 2, 3, 10])
+def test_iterate_after_k_sweeps(shape, k):
+    w, plan = _plan(shape, "fp64", max_sweeps=k)
+    x, info = plan.solve(torch.from_numpy(w.b[0]).cuda(), tol=1e-300, check=False)
+    assert info["sweeps"] == k and plan.stats()["sweep_kernel"] == 8
+    _, its = O.vtm_midpoint(w.csr(), w.partition, w.nparts, w.b[:1], W=1 / w.Zc, tol=0, max_sweeps=k,
+                            keep_iterates=True)
+    ref = its[k - 1][0]
+    assert np.abs(x.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+def test_a_barrier_that_runs_out_is_reported_and_the_plan_recovers():
+    from paper_0910_0663_gb300 import vtm
+    w, plan = _plan(GRID[1], "fp64")
+    b = torch.from_numpy(w.b[0]).cuda()
+    x, _ = plan.solve(b)
+    plan.set_options(wait_polls=1)  # the first poll that finds the barrier open gives up
+    with pytest.raises(vtm.VTMError, match="timed out"):
+        plan.solve(b)
+    plan.set_options(wait_polls=0)
+    x2, _ = plan.solve(b)
+    assert torch.equal(x, x2)
