@@ -23,6 +23,9 @@
 //         at two tiles on the fullest SM); 100 tiles, bw 99, LU: 4057 -> 622 us;
 //         150 boxes of up to 1782 rows, bw <= 112: 1770 -> 287 us
 //   FP32  the same three shapes: 936 -> 179 us (bw 64), 1058 -> 92 us (bw <= 112)
+// With several columns a CTA takes four (each multiplier read once for them): FP64,
+// 110 boxes of up to 2028 rows, bw <= 126, 18 columns: 5.2 ms with the batched
+// row-by-row kernel, 1.62 ms here.
 // Two warps per tile (fewer cross-warp sums, 112 instead of 128 FP64
 // instructions per block) measured 745, 916 and 423 us: too few in flight.
 #include <algorithm>
@@ -89,18 +92,20 @@ __host__ __device__ constexpr int bb_stage_elems(int B) {
   return (kBbN * B + 2 * kVec - 1) / kVec * kVec + kBbN * kBbN;
 }
 
-// the warps' partial sums of one row, added as a tree
+// the warps' partial sums of one row, added as a tree; `step` between the warps
 template <int NW, class FT>
-__device__ __forceinline__ FT sum_warps(const FT* r) {
+__device__ __forceinline__ FT sum_warps(const FT* r, int step) {
   static_assert(NW == 4, "");
-  return (r[0] + r[kBbN]) + (r[2 * kBbN] + r[3 * kBbN]);
+  return (r[0] + r[step]) + (r[2 * step] + r[3 * step]);
 }
 
-template <class FT, int K, int NW, bool FWD>
+// NC columns at once (each multiplier is read once for all of them)
+template <class FT, int K, int NW, int NC, bool FWD>
 __device__ __forceinline__ bool bb_pass(const FT* __restrict__ cols, const FT* __restrict__ inv, int n, int bw,
-                                        FT* v, FT* ring, int stage_elems, int S, uint64_t* bars,
-                                        uint32_t& par, FT* red, int* s_fail) {
-  constexpr int C = kBbN / NW;  // columns per warp
+                                        FT* v, int64_t stride, int nc, FT* ring, int stage_elems, int S,
+                                        uint64_t* bars, uint32_t& par, FT* red, int* s_fail) {
+  constexpr int C = kBbN / NW;  // band columns per warp
+  constexpr int RW = NC * kBbN;  // one warp's row of `red`
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int B = bw + 1;
   const int nblk = (n + kBbN - 1) / kBbN;
@@ -116,19 +121,28 @@ __device__ __forceinline__ bool bb_pass(const FT* __restrict__ cols, const FT* _
     bulk_copy_g2s(dst, reinterpret_cast<const void*>(a0), bytes, bar);
     bulk_copy_g2s(dst + stage_elems - kBbN * kBbN, inv + (int64_t)b * kBbN * kBbN, kBbN * kBbN * sizeof(FT), bar);
   };
-  auto src = [&](int j) -> FT { return j < n ? v[FWD ? j : n - 1 - j] : FT(0); };
+  auto src = [&](int j, int x) -> FT { return j < n && x < nc ? v[x * stride + (FWD ? j : n - 1 - j)] : FT(0); };
   if (threadIdx.x == 0) {
     fence_proxy_async_smem();  // the stages' earlier reads come before the copies
     for (int b = 0; b < S && b < nblk; ++b) issue(b);
   }
-  FT acc[K];  // this warp's updates of the next K blocks, lane = row
+  FT acc[K][NC];  // this warp's updates of the next K blocks, lane = row
+  FT vt[NC];
 #pragma unroll
-  for (int k = 0; k < K; ++k) acc[k] = FT(0);
-  FT vt = src(lane);
+  for (int x = 0; x < NC; ++x) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k][x] = FT(0);
+    vt[x] = src(lane, x);
+  }
+  FT* mine = red + (2 * NW + warp) * RW;  // this warp's copy of t, then of -u
   for (int b = 0; b < nblk; ++b) {
     const int s = b * kBbN, sl = b % S;
-    const FT vn = src(s + kBbN + lane);
-    red[warp * kBbN + lane] = acc[0];
+    FT vn[NC];
+#pragma unroll
+    for (int x = 0; x < NC; ++x) {
+      vn[x] = src(s + kBbN + lane, x);
+      red[warp * RW + x * kBbN + lane] = acc[0][x];
+    }
     if (!mbar_wait_bounded(&bars[sl], (par >> sl) & 1u, kBbPolls)) *(volatile int*)s_fail = 1;
     par ^= 1u << sl;
     __syncthreads();
@@ -146,17 +160,35 @@ __device__ __forceinline__ bool bb_pass(const FT* __restrict__ cols, const FT* _
     }
     const FT* st = ring + (size_t)sl * stage_elems;
     const FT* iv = st + stage_elems - kBbN * kBbN + warp * C * kBbN + lane;
-    FT* mine = red + (2 * NW + warp) * kBbN;  // this warp's copy of t, then of u
-    mine[lane] = vt + sum_warps<NW>(red + lane);
-    __syncwarp();
-    FT part[4] = {FT(0), FT(0), FT(0), FT(0)};
 #pragma unroll
-    for (int c = 0; c < C; ++c) part[c & 3] += iv[c * kBbN] * mine[warp * C + c];
-    red[(NW + warp) * kBbN + lane] = (part[0] + part[1]) + (part[2] + part[3]);
-    __syncthreads();
-    const FT u = sum_warps<NW>(red + NW * kBbN + lane);
+    for (int x = 0; x < NC; ++x) mine[x * kBbN + lane] = vt[x] + sum_warps<NW>(red + x * kBbN + lane, RW);
     __syncwarp();
-    mine[lane] = -u;
+    {
+      constexpr int P = NC == 1 ? 4 : 1;  // chains per column
+      FT part[NC][P];
+#pragma unroll
+      for (int x = 0; x < NC; ++x)
+#pragma unroll
+        for (int y = 0; y < P; ++y) part[x][y] = FT(0);
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        const FT m = iv[c * kBbN];
+#pragma unroll
+        for (int x = 0; x < NC; ++x) part[x][c % P] += m * mine[x * kBbN + warp * C + c];
+      }
+#pragma unroll
+      for (int x = 0; x < NC; ++x) {
+        if constexpr (P == 4) part[x][0] = (part[x][0] + part[x][1]) + (part[x][2] + part[x][3]);
+        red[(NW + warp) * RW + x * kBbN + lane] = part[x][0];
+      }
+    }
+    __syncthreads();
+    FT u[NC];
+#pragma unroll
+    for (int x = 0; x < NC; ++x) u[x] = sum_warps<NW>(red + NW * RW + x * kBbN + lane, RW);
+    __syncwarp();
+#pragma unroll
+    for (int x = 0; x < NC; ++x) mine[x * kBbN + lane] = -u[x];
     __syncwarp();
     const int c0 = first_col(b);
     constexpr int kMask = 16 / sizeof(FT) - 1;
@@ -168,7 +200,13 @@ __device__ __forceinline__ bool bb_pass(const FT* __restrict__ cols, const FT* _
     const int amax = min(bw, n - 1 - s);  // no row past n: 32 k + lane <= n - 1 - s as well
 #pragma unroll
     for (int k = 1; k <= K; ++k) {
-      FT x = k < K ? acc[k] : FT(0), y = FT(0);
+      constexpr int P = NC == 1 ? 2 : 1;
+      FT y[NC][P];
+#pragma unroll
+      for (int x = 0; x < NC; ++x) {
+        y[x][0] = k < K ? acc[k < K ? k : 0][x] : FT(0);
+        if constexpr (P == 2) y[x][1] = FT(0);
+      }
       const bool row = kBbN * k + lane <= n - 1 - s;
 #pragma unroll
       for (int c4 = 0; c4 < C; c4 += 4) {
@@ -178,32 +216,43 @@ __device__ __forceinline__ bool bb_pass(const FT* __restrict__ cols, const FT* _
           for (int c = c4; c < c4 + 4; ++c) {
             const int a = kBbN * k - (warp * C + c) + lane;
             const FT m = (row && a <= bw) ? col[kBbN * k + c * step] : FT(0);
-            if (c & 1) y += m * mine[warp * C + c];
-            else x += m * mine[warp * C + c];
+#pragma unroll
+            for (int x = 0; x < NC; ++x) y[x][c % P] += m * mine[x * kBbN + warp * C + c];
           }
         }
       }
-      acc[k - 1] = x + y;
+#pragma unroll
+      for (int x = 0; x < NC; ++x) {
+        if constexpr (P == 2) acc[k - 1][x] = y[x][0] + y[x][1];
+        else acc[k - 1][x] = y[x][0];
+      }
     }
-    if (warp == 0 && s + lane < n) v[FWD ? s + lane : n - 1 - s - lane] = u * st[dl + (FWD ? lane : last - lane) * B];
-    vt = vn;
+    if (s + lane < n) {
+      const FT dg = st[dl + (FWD ? lane : last - lane) * B];
+#pragma unroll
+      for (int x = 0; x < NC; ++x)  // a column per warp in turn
+        if (warp == (x & (NW - 1)) && x < nc) v[x * stride + (FWD ? s + lane : n - 1 - s - lane)] = u[x] * dg;
+    }
+#pragma unroll
+    for (int x = 0; x < NC; ++x) vt[x] = vn[x];
   }
   return true;
 }
 
-template <class FT, int K, int NW>
+template <class FT, int K, int NW, int NC>
 __global__ void __launch_bounds__(32 * NW) band_solve_blk_kernel(
     const int32_t* __restrict__ node_off, const int32_t* __restrict__ bwv, const int64_t* __restrict__ band_off,
     const int32_t* __restrict__ blk_off, const int32_t* __restrict__ order, const FT* __restrict__ Lc,
     const FT* __restrict__ Uc, const FT* __restrict__ Li, const FT* __restrict__ Ui, FT* __restrict__ v,
-    int64_t stride, int nparts, int stage_elems, int S) {
+    int64_t stride, int nparts, int ncols, int stage_elems, int S) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bars[8];
   __shared__ int s_fail;
-  __shared__ __align__(16) FT red[3 * NW * kBbN];
+  __shared__ __align__(16) FT red[3 * NW * NC * kBbN];
   FT* ring = reinterpret_cast<FT*>(smem_raw);
-  const int t = order[blockIdx.x % nparts];
-  const int col = blockIdx.x / nparts;
+  const int groups = (ncols + NC - 1) / NC;  // of one tile side by side: largest tiles first
+  const int t = order[blockIdx.x / groups];
+  const int col = blockIdx.x % groups * NC, nc = min(NC, ncols - col);
   const int off = node_off[t], n = node_off[t + 1] - off, bw = bwv[t];
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) mbar_init(&bars[i], 1);
@@ -214,11 +263,15 @@ __global__ void __launch_bounds__(32 * NW) band_solve_blk_kernel(
   FT* vg = v + (int64_t)col * stride + off;
   const int64_t io = (int64_t)blk_off[t] * kBbN * kBbN;
   uint32_t par = 0;
-  bool ok = bb_pass<FT, K, NW, true>(Lc + band_off[t], Li + io, n, bw, vg, ring, stage_elems, S, bars, par, red, &s_fail);
+  bool ok = bb_pass<FT, K, NW, NC, true>(Lc + band_off[t], Li + io, n, bw, vg, stride, nc, ring, stage_elems, S, bars,
+                                         par, red, &s_fail);
   __syncthreads();  // y of the whole tile before the backward pass reads it
-  if (ok) ok = bb_pass<FT, K, NW, false>(Uc + band_off[t], Ui + io, n, bw, vg, ring, stage_elems, S, bars, par, red, &s_fail);
+  if (ok)
+    ok = bb_pass<FT, K, NW, NC, false>(Uc + band_off[t], Ui + io, n, bw, vg, stride, nc, ring, stage_elems, S, bars, par,
+                                       red, &s_fail);
   if (!ok)  // the refinement reports the NaN as a divergence
-    for (int i = threadIdx.x; i < n; i += 32 * NW) vg[i] = FT(NAN);
+    for (int i = threadIdx.x; i < n; i += 32 * NW)
+      for (int x = 0; x < nc; ++x) vg[x * stride + i] = FT(NAN);
 }
 
 // Half bandwidths this form serves: above 32 (up to 32 the warp-per-tile
@@ -272,18 +325,19 @@ static void launch_blk_t(vtm_plan_s* P, FT* v, const FT* Lc, const FT* Uc, const
   // than ceil(tiles / SMs) of them on one SM while others stay empty
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device);
-  const int per_sm = (P->nparts * ncols + sms - 1) / sms;
+  const bool multi = ncols >= 3;  // four columns per CTA
+  const int per_sm = (P->nparts * (multi ? (ncols + 3) / 4 : ncols) + sms - 1) / sms;
   const size_t smem = std::max(S * bytes, per_sm <= 3 ? (size_t)(224 / (per_sm + 1) + 1) * 1024 : 0);
-  auto go = [&](auto* kern) {
+  auto go = [&](auto* kern, int nc) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<P->nparts * ncols, 32 * NW, smem, s>>>(
+    kern<<<P->nparts * ((ncols + nc - 1) / nc), 32 * NW, smem, s>>>(
         P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(), P->tabs.band_off.as<int64_t>(),
-        P->d_bb_off.as<int32_t>(), P->d_bb_order.as<int32_t>(), Lc, Uc, Li, Ui, v, stride, P->nparts, stage, S);
+        P->d_bb_off.as<int32_t>(), P->d_bb_order.as<int32_t>(), Lc, Uc, Li, Ui, v, stride, P->nparts, ncols, stage, S);
   };
   const int K = (31 + P->max_bw) / 32;
-  if (K <= 2) go(band_solve_blk_kernel<FT, 2, NW>);
-  else if (K <= 4) go(band_solve_blk_kernel<FT, 4, NW>);
-  else go(band_solve_blk_kernel<FT, 8, NW>);
+  if (K <= 2) multi ? go(band_solve_blk_kernel<FT, 2, NW, 4>, 4) : go(band_solve_blk_kernel<FT, 2, NW, 1>, 1);
+  else if (K <= 4) multi ? go(band_solve_blk_kernel<FT, 4, NW, 4>, 4) : go(band_solve_blk_kernel<FT, 4, NW, 1>, 1);
+  else multi ? go(band_solve_blk_kernel<FT, 8, NW, 4>, 4) : go(band_solve_blk_kernel<FT, 8, NW, 1>, 1);
 }
 
 bool launch_band_solve_blk(vtm_plan_s* P, double* v, int ncols, int64_t stride, cudaStream_t s) {

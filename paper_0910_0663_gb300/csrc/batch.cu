@@ -2160,6 +2160,12 @@ static vtm_status batch_band_solve_blk(vtm_plan_s* P, float* V, int R) {
 
 template <class FT>
 static vtm_status batch_band_solve(vtm_plan_s* P, FT* V, int R, const FT* Lc, const FT* Uc) {
+  // FP64 (column-major vectors): the blocked solves, four columns per CTA
+  if constexpr (sizeof(FT) == 8)
+    if (launch_band_solve_blk(P, V, R, P->n, P->stream)) {
+      P->launch_count++;
+      return VTM_OK;
+    }
   if constexpr (sizeof(FT) == 4) {
     const int mode = P->opts.batch_solve;
     if (mode == 3 || (mode == 0 && P->max_bw <= kBkMaxW)) return batch_band_solve_blk(P, V, R);
