@@ -2075,6 +2075,8 @@ __global__ void pack_tc_kernel(const double* __restrict__ T64, const int64_t* __
 // host driver for a batch of right-hand sides
 // ---------------------------------------------------------------------------
 
+#include "split.cuh"
+
 static int grid_n(int64_t work) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 152 * 16));
 }
@@ -2271,6 +2273,66 @@ vtm_status ensure_vals_df(vtm_plan_s* P) {
   return VTM_OK;
 }
 
+// Lists and digits of the tensor-core FP64 sweep; *ok = false where it does not serve.
+static vtm_status prepare_digits(vtm_plan_s* P, int nt8, bool* ok) {
+  cudaStream_t s = P->stream;
+  *ok = false;
+  if (P->dg_res == 0) {
+    std::vector<DgItem> items;
+    std::vector<DgChunk> chunks;
+    std::vector<int64_t> off(P->nparts, 0);
+    int64_t blocks = 0;
+    int32_t kb = 0;
+    for (int32_t t = 0; t < P->nparts; ++t) {
+      const int32_t p = P->port_off[t + 1] - P->port_off[t], nb = (p + 15) / 16;
+      off[t] = blocks;
+      for (int32_t m = 0; m < nb; m += kDgBlocks) items.push_back(DgItem{t, m, kb, (int32_t)chunks.size(), blocks, 0});
+      for (int32_t m = 0; m < p; m += 16 * kDgChunk) chunks.push_back(DgChunk{t, m, kb + m / 16, 0});
+      kb += nb;
+      blocks += (int64_t)nb * nb;
+    }
+    P->dg_chunks = (int)chunks.size();
+    for (int32_t t = 0; t < P->nparts; ++t)  // the residual's items after them
+      for (int32_t m = 0; m < P->port_off[t + 1] - P->port_off[t]; m += 32) chunks.push_back(DgChunk{t, m, 0, 0});
+    P->dg_res = (int)chunks.size() - P->dg_chunks;
+    auto cost = [&](const DgItem& d) {
+      const int nb = (P->port_off[d.tile + 1] - P->port_off[d.tile] + 15) / 16;
+      return nb * std::min(kDgBlocks, nb - d.mb0);
+    };
+    std::stable_sort(items.begin(), items.end(), [&](const DgItem& a, const DgItem& b) { return cost(a) > cost(b); });
+    VTM_TRY(upload(P->d_dg_items, items, s));
+    P->dg_items = (int)items.size();
+    VTM_TRY(upload(P->d_dg_chunks, chunks, s));
+    VTM_TRY(upload(P->d_dg_off, off, s));
+    VTM_CUDA_TRY(cudaStreamSynchronize(s));  // the host lists are about to go
+    P->dg_blocks = blocks;
+    P->dg_kb = kb;
+  }
+  const size_t bytes = (size_t)P->dg_blocks * kDg * 32 * sizeof(uint4);
+  if (bytes > ((size_t)32 << 30)) return VTM_OK;
+  if (dev_alloc(P->d_dg_T, bytes) != VTM_OK || dev_alloc(P->d_dg_texp, P->port_node.size() * sizeof(int)) != VTM_OK ||
+      dev_alloc(P->d_dg_w, (size_t)P->dg_kb * nt8 * kDg * 32 * sizeof(uint2)) != VTM_OK ||
+      dev_alloc(P->d_dg_wexp, (size_t)P->dg_chunks * 64 * sizeof(int)) != VTM_OK) {
+    cudaGetLastError();
+    dev_free(P->d_dg_T);
+    P->dg_ready = false;
+    return VTM_OK;
+  }
+  if (!P->dg_ready) {
+    row_exponents_kernel<<<dim3(P->nparts, 16), 256, 0, s>>>(P->d_T64.as<double>(), P->tabs.T_off.as<int64_t>(),
+                                                   P->tabs.T_ld.as<int32_t>(), P->tabs.port_off.as<int32_t>(),
+                                                   P->d_dg_texp.as<int>());
+    pack_digits_kernel<<<dim3(P->nparts, 16), 256, 0, s>>>(
+        P->d_T64.as<double>(), P->tabs.T_off.as<int64_t>(), P->tabs.T_ld.as<int32_t>(), P->tabs.port_off.as<int32_t>(),
+        P->d_dg_off.as<int64_t>(), P->d_dg_texp.as<int>(), P->d_dg_T.as<uint4>());
+    VTM_CUDA_TRY(cudaGetLastError());
+    P->launch_count += 2;
+    P->dg_ready = true;
+  }
+  *ok = true;
+  return VTM_OK;
+}
+
 vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, double tol,
                          vtm_info* info, bool record_hist) {
   cudaStream_t s = P->stream;
@@ -2341,6 +2403,12 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
     P->launch_count++;
     P->tc_nitems = nt;
   }
+  // FP64 plans: digits of T_P for the tensor-core sweep (built at the first
+  // batched solve after each factorisation; 18 bytes per entry, so not where
+  // that passes 32 GB or memory runs out)
+  const int nt8 = (R + 7) / 8;
+  bool dg_ok = false;
+  if (prec == VTM_PREC_FP64 && npt > 0 && P->opts.batch_kernel == 0) VTM_TRY(prepare_digits(P, nt8, &dg_ok));
   const bool lowp = prec != VTM_PREC_FP64;
   const size_t wsz = lowp ? sizeof(float) : sizeof(double);
   VTM_TRY(dev_alloc(P->d_bV, (size_t)n * R * sizeof(double)));
@@ -2348,7 +2416,7 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
   VTM_TRY(dev_alloc(P->d_bc, (size_t)std::max<int64_t>(npt, 1) * R * wsz));
   // per-ticket partials, then the group sums; the group counters follow the
   // control block and are cleared with every upload of it
-  const int max_items = std::max(std::max(nitems, P->tc_nitems), 1);
+  const int max_items = std::max(std::max(nitems, P->tc_nitems), std::max(P->dg_res, 1));
   const int ngroups = (max_items + kBGrp - 1) / kBGrp;
   VTM_TRY(dev_alloc(P->d_bpart, (size_t)(max_items + ngroups) * R * sizeof(double)));
   VTM_TRY(dev_alloc(P->d_btol2, 64 * sizeof(double)));
@@ -2509,6 +2577,29 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
               R, P->d_bctrl.as<BatchCtrl>(), P->d_bpart.as<double>(), P->d_btol2.as<double>(), bhist, bhist_len);
           return;
         }
+        if (kv == 5) {  // FP64 on the tensor cores: the waves' digits, then the products
+          const int NT = nt8 == 4 ? 2 : std::min(nt8, kDgMaxNt), ny = (nt8 + NT - 1) / NT;
+          auto go_dg = [&](auto* kern) {
+            const size_t smem = kDgStages * (kDgBlocks * kDg * 32 * sizeof(uint4) + (size_t)NT * kDg * 32 * sizeof(uint2));
+            if (dry) {
+              cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+              return;
+            }
+            batch_digits_kernel<<<P->dg_chunks + P->dg_res, 256, 0, s>>>(
+                P->d_dg_chunks.as<DgChunk>(), P->dg_chunks, P->tabs.port_off.as<int32_t>(), P->d_twin.as<int32_t>(),
+                P->d_kd.as<double2>(), P->d_run.as<uint8_t>(), P->d_bstate.as<double>(), npt, R, nt8,
+                P->d_dg_w.as<uint2>(), P->d_dg_wexp.as<int>(), P->d_bctrl.as<BatchCtrl>(), P->d_bpart.as<double>(),
+                P->d_btol2.as<double>(), bhist, bhist_len);
+            kern<<<P->dg_items * ny, 32 * kDgBlocks, smem, s>>>(
+                P->d_dg_items.as<DgItem>(), P->tabs.port_off.as<int32_t>(), P->d_dg_T.as<uint4>(),
+                P->d_dg_texp.as<int>(), P->d_dg_w.as<uint2>(), P->d_dg_wexp.as<int>(), nt8, ny, P->d_bc.as<double>(),
+                P->d_bstate.as<double>(), npt, R, P->d_bctrl.as<BatchCtrl>());
+          };
+          if (NT == 1) go_dg(batch_sweep_digits_kernel<1>);
+          else if (NT == 2) go_dg(batch_sweep_digits_kernel<2>);
+          else go_dg(batch_sweep_digits_kernel<3>);
+          return;
+        }
         auto go = [&](auto* kern, int threads, const auto* T, const auto* cc, auto* st) {
           const int key = prec * 8 + kv;
           if (P->batch_grid[key] == 0) {
@@ -2558,14 +2649,20 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
         if (kv == 4 && prec != VTM_PREC_BF16) kv = 0;
         if (kv != 4 && (kv & 1) && !(prec == VTM_PREC_BF16 && R % 8 == 0)) kv &= ~1;
       } else {
-        if (P->batch_tuned[prec] == 0 || P->batch_tuned_R[prec] != R) {
+        if (P->batch_tuned[prec] == 0 || P->batch_tuned_R[prec] != R || (P->batch_tuned[prec] == 6) != dg_ok) {
           float best = 1e30f;
-          for (int cand = 0; cand <= 4; ++cand) {
+          for (int cand = 0; cand <= 5; ++cand) {
+            if (dg_ok && cand != 5) continue;  // (FP64: faster at every size, by 3 to 40 times)
+            if (cand == 5 && !dg_ok) continue;
             if (cand == 4 && prec != VTM_PREC_BF16) continue;
-            if (cand != 4 && (cand & 1) && !(prec == VTM_PREC_BF16 && R % 8 == 0)) continue;
+            if (cand < 4 && (cand & 1) && !(prec == VTM_PREC_BF16 && R % 8 == 0)) continue;
             BatchCtrl tt = h;
             tt.k_max = 1 << 30;
             tt.stall = 0;
+            if (dg_ok) {
+              P->batch_tuned[prec] = cand + 1;
+              continue;
+            }
             VTM_TRY(upload_bctrl(tt, s));
             launch_batch(cand);
             VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
@@ -2588,7 +2685,8 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
         }
         kv = P->batch_tuned[prec] - 1;
       }
-      P->batch_used = kv + 1;
+      // (an FP64 plan's tensor-core form counts as 2, warp MMAs)
+      P->batch_used = kv == 5 ? 2 : kv + 1;
       // batches of check_every launches replayed from a CUDA graph when the
       // plan has its own stream, and quarter batches for the tail up to the
       // sweeps this refinement step took in the previous solve (the launches

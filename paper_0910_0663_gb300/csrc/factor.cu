@@ -982,6 +982,7 @@ extern "C" vtm_status vtm_factor(vtm_plan_t P) {
   dev_free(P->d_bk_Gf);
   dev_free(P->d_bk_Gb);
   P->bk_ready = false;
+  P->dg_ready = false;
   VTM_TRY(assemble_band(P));  // a factorisation overwrites the band
   VTM_TRY(factor_tiles(P));
   if (P->opts.precision != VTM_PREC_FP64) {

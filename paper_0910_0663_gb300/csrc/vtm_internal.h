@@ -323,6 +323,12 @@ struct vtm_plan_s {
   // chunks), their offsets into the tiled BF16 copy of T_P, longest first
   int tc_nitems = 0;
   vtm::DevBuf d_tc_items, d_tc_off, d_tc_order, d_Ttc;
+  // FP64 batched sweep on the tensor cores (split.cuh): work items, T_P's digits
+  // and row exponents, the waves' digits and chunk exponents
+  vtm::DevBuf d_dg_items, d_dg_chunks, d_dg_off, d_dg_T, d_dg_texp, d_dg_w, d_dg_wexp;
+  int dg_items = 0, dg_chunks = 0, dg_res = 0, dg_kb = 0;
+  int64_t dg_blocks = 0;
+  bool dg_ready = false;  // the digits follow the current factors
   // blocked batched band solves: per tile the window width W, the offset of
   // its G blocks, tiles longest first, (tile, block) list, G_f and G_b
   // (built at the first FP32 batched solve after each factorisation)
