@@ -21,6 +21,8 @@
 #include <cmath>
 
 #include "band.cuh"
+#include "gridctl.cuh"
+#include "ptx.h"
 #include "vtm_internal.h"
 
 namespace vtm {
@@ -235,6 +237,327 @@ __global__ void __launch_bounds__(1024) general_sweep_kernel(
   }
 }
 
+// The same sweeps in one cooperative launch, one bounded grid barrier per sweep (the
+// control warp of gridctl.cuh).  A CTA owns a contiguous range of output pairs -- of
+// one tile or several -- of equal cost (pairs times inputs): thread (pair, group) takes
+// the inputs group, group + G, ... of its pair, so that every SM's FP64 pipe has the
+// same work, which no split into whole tiles or slabs gives (460 slabs of 64 outputs on
+// 152 SMs: 4 on some, 3 on most).  As many of a thread's elements of E_P as fit stay in
+// shared memory for the whole solve; the rest stream from L2 through a ring of
+// asynchronous copies that never stops: E_P does not change, so the first elements of
+// sweep k + 1 are on their way while barrier k is awaited.  The residual of sweep k - 1
+// is formed in that wait; what its rows need of w_in(k - 1) are the w_out(k - 2) the
+// waves came from, so no incident value is stored before the last sweep.
+// Slots of w_out: 8 (sweeps k - 2 to k + 1 may be in use at once, and the iterate that
+// is kept is up to five sweeps old when every CTA has stopped).
+// Bound by the FP64 pipe and the chain barrier - gather - products - sums around it.
+// Measured, VCCS grid 640 x 640 in 100 tiles (46 MB of E_P, 9.8 us of FP64 pipe): one CTA
+// per tile and launch 39 us per sweep, slabs of 64 outputs 24 us, here 16.5 us; solves of
+// 100 sweeps on 1024 x 1024 in 256 tiles 17.9 -> 6.5 ms, 24 x 24 in 9 tiles 1.39 -> 0.98.
+// Plans with more output pairs per SM than threads (over 230k outputs: 1024 x 1024 in
+// tiles of 16 x 16) keep one CTA per tile: slabs of outputs were slower there (100
+// sweeps in tiles of 16 x 16 14.8 ms against 24.2, of 8 x 8 21.6 against 44.3).
+constexpr int kGenThreads = 768;  // and a control warp: 80 registers per thread
+constexpr int kGenRing = 4, kGenMinSlots = 8;
+struct GenCta {
+  int32_t pair0, np;   // first output pair, pairs
+  int32_t in0, nin;    // inputs of the tiles it touches
+  int32_t q0, q1;      // residual entries (whole runs)
+  int32_t i0, i1;      // inputs it stores after the last sweep
+};
+struct GenRes {
+  const double* E;
+  const int64_t* E_off;
+  const int32_t *E_ld, *in_off, *out_off, *pair_off;
+  const GenCta* ctas;
+  const int32_t *in_src, *in_own_out, *res_in;
+  const uint8_t *in_kind, *res_run;
+  const double *coef, *dsc, *c;
+  double *gin, *gout;
+  int64_t n_in, n_out;
+  SweepCtrl* ctrl;
+  unsigned long long* bar;
+  double *part, *hist;
+  int hist_len, nparts, nslots, vmax;
+  uint32_t max_polls;
+};
+
+__global__ void __launch_bounds__(kGenThreads + 32, 1) general_resident_kernel(const GenRes A) {
+  constexpr int NT = kGenThreads, NW = NT / 32, S = kGenRing;
+  extern __shared__ __align__(16) unsigned char gsm[];
+  __shared__ int s_flag;
+  __shared__ double s_part[2][NW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) s_flag = 0;
+  if (tid < NW) s_part[0][tid] = s_part[1][tid] = 0.0;
+  __syncthreads();
+  if (warp == NW) {
+    res_control(A.ctrl, A.bar, A.part, A.hist, A.hist_len, A.max_polls, &s_flag, s_part[0], NW, NW, lane);
+    return;
+  }
+  // shared memory: [nslots][NT] elements | [NT] sums | [vmax] incident values | [vmax] their sources |
+  // [2 NT] output ids
+  double2* slots = reinterpret_cast<double2*>(gsm) + tid;
+  double2* red = reinterpret_cast<double2*>(gsm) + (size_t)A.nslots * NT;
+  double* vin = reinterpret_cast<double*>(red + NT);
+  int32_t* src = reinterpret_cast<int32_t*>(vin + A.vmax);
+  int32_t* oid = src + A.vmax;
+  const GenCta C = A.ctas[blockIdx.x];
+  const int np = C.np, G = np > 0 ? NT / np : 0;
+  const int l = np > 0 ? tid % np : 0, g = np > 0 ? tid / np : 0;
+  int cnt = 0, vofs = 0, ld = 0;
+  const double* Ep = A.E;
+  if (g < G) {
+    int lo = 0, hi = A.nparts;  // the tile of the pair
+    const int pg = C.pair0 + l;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (A.pair_off[mid] <= pg) lo = mid;
+      else hi = mid;
+    }
+    const int m = 2 * (pg - A.pair_off[lo]), ni = A.in_off[lo + 1] - A.in_off[lo];
+    ld = A.E_ld[lo];
+    cnt = ni > g ? (ni - g + G - 1) / G : 0;
+    Ep = A.E + A.E_off[lo] + m + (size_t)g * ld;
+    vofs = A.in_off[lo] - C.in0 + g;
+    if (g == 0) {
+      const int no = A.out_off[lo + 1] - A.out_off[lo], o = A.out_off[lo] + m;
+      oid[2 * l] = o;
+      oid[2 * l + 1] = m + 1 < no ? o + 1 : -1;
+    }
+  }
+  for (int q = tid; q < C.nin; q += NT) src[q] = A.in_src[C.in0 + q];
+  const size_t step = (size_t)G * ld;
+  // elements 0 .. nres - 1 stay; the others pass through slots nslots - S ..
+  const int nres = cnt <= A.nslots ? cnt : A.nslots - S, nstr = cnt - nres;
+  double2* ring = slots + (size_t)(A.nslots - S) * NT;
+  for (int i = 0; i < nres; ++i) cp_async16(slots + i * NT, Ep + i * step);
+  cp_async_commit_group();
+  cp_async_wait_group<0>();
+  int an = 0, sn = 0;
+  auto issue = [&]() {  // the next streamed element, round and round
+    cp_async16(ring + sn * NT, Ep + (size_t)(nres + an) * step);
+    cp_async_commit_group();
+    an = an + 1 == nstr ? 0 : an + 1;
+    sn = (sn + 1) & (S - 1);
+  };
+  if (nstr > 0)
+#pragma unroll
+    for (int b = 0; b < S - 1; ++b) issue();
+  int sl = 0, k = 1;
+  for (;; ++k) {
+    __syncthreads();  // the waves of sweep k - 1 are out and the flag is read
+    if (*((volatile int*)&s_flag)) break;
+    const double* prev = A.gout + (size_t)((k - 1) & (kGenSlots - 1)) * A.n_out;
+    for (int q = tid; q < C.nin; q += NT) vin[q] = __ldcg(prev + src[q]);
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+    double x = 0.0, y = 0.0;
+    const double* v = vin + vofs;
+#pragma unroll 4
+    for (int i = 0; i < nres; ++i) {
+      const double2 e = slots[i * NT];
+      const double w = *v;
+      x += e.x * w;
+      y += e.y * w;
+      v += G;
+    }
+    for (int i = 0; i < nstr; ++i) {
+      issue();
+      cp_async_wait_group<S - 1>();  // this thread's oldest element has landed
+      const double2 e = ring[sl * NT];
+      const double w = *v;
+      x += e.x * w;
+      y += e.y * w;
+      v += G;
+      sl = (sl + 1) & (S - 1);
+    }
+    red[tid] = make_double2(x, y);
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+    double* cur = A.gout + (size_t)(k & (kGenSlots - 1)) * A.n_out;
+    const double* rs = reinterpret_cast<const double*>(red);
+    for (int q = tid; q < 2 * np; q += NT) {
+      const int o = oid[q];
+      if (o < 0) continue;
+      double tot = __ldg(A.c + o);
+#pragma unroll 8
+      for (int b = 0; b < G; ++b) tot += rs[(size_t)b * 2 * np + q];
+      cur[o] = tot;
+    }
+    __syncthreads();  // every wave of sweep k is written
+    if (k > 1) {  // the residual of sweep k - 1, while the grid barrier is awaited
+      const double* pp = A.gout + (size_t)((k - 2) & (kGenSlots - 1)) * A.n_out;
+      double sq = 0.0;
+      for (int q = C.q0 + tid; q < C.q1; q += NT) {
+        const int nr = A.res_run[q];
+        if (!nr) continue;
+        double r = 0.0;
+        for (int e = 0; e < nr; ++e) {
+          const int a = A.res_in[q + e], s = A.in_src[a];
+          const double wo_t = __ldcg(prev + s), wi_s = __ldcg(pp + s);
+          if (A.in_kind[a] != 0) {
+            r += A.coef[a] * (wi_s - wo_t);
+          } else {
+            const int own = A.in_own_out[a];
+            const double wo_s = __ldcg(prev + own), wi_t = __ldcg(pp + own);
+            const double Ss = wi_s + wo_s, St = wi_t + wo_t;
+            r += 0.5 * A.dsc[a] * (0.5 * (Ss + St) - A.coef[a] * (Ss - St) - wi_s - wi_t);
+          }
+        }
+        sq += r * r;
+      }
+      for (int o = 16; o > 0; o >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, o);
+      if (lane == 0) s_part[k & 1][warp] = sq;
+    }
+  }
+  cp_async_wait_group<0>();  // no copy into shared memory outlives the CTA
+  const int flag = *((volatile int*)&s_flag);
+  if (flag == 5) return;
+  // the decision of sweep k - 1 closed sweep k - 3: its iterate, or the one before
+  const int it = flag == 1 ? k - 4 : k - 3;
+  const double* from = A.gout + (size_t)((it - 1) & (kGenSlots - 1)) * A.n_out;
+  for (int a = C.i0 + tid; a < C.i1; a += NT) A.gin[(size_t)(it & 1) * A.n_in + a] = __ldcg(from + A.in_src[a]);
+}
+
+// the CTAs of the resident form; gen_ctas stays 0 where it does not apply
+static vtm_status plan_general_resident(vtm_plan_s* P) {
+  P->gen_ctas = -1;
+  int coop = 0, sms = 152;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, P->device);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device);
+  if (!coop || P->n_in == 0 || P->n_out == 0) return VTM_OK;
+  std::vector<int32_t> pair_off(P->nparts + 1, 0), res_in(P->n_in);
+  int64_t cost = 0;  // elements of E_P in pairs, and the sums
+  auto pairs = [&](int32_t t) { return (P->out_off[t + 1] - P->out_off[t] + 1) / 2; };
+  auto pair_cost = [&](int32_t t) { return (int64_t)(P->in_off[t + 1] - P->in_off[t]) + 4; };
+  for (int32_t t = 0; t < P->nparts; ++t) {
+    pair_off[t + 1] = pair_off[t] + pairs(t);
+    cost += pairs(t) * pair_cost(t);
+    for (int32_t a = P->in_off[t]; a < P->in_off[t + 1]; ++a) res_in[a] = P->in_off[t] + P->res_perm[a];
+  }
+  // at least eight elements per thread
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, cost / (8 * kGenThreads)));
+  std::vector<GenCta> ctas(grid);
+  auto run_start = [&](int64_t q) {
+    while (q < P->n_in && !P->res_run[q]) ++q;
+    return (int32_t)q;
+  };
+  int32_t t = 0, pr = 0;  // next pair: pair `pr` of tile t
+  int64_t done = 0;
+  int32_t vmax = 1;
+  for (int b = 0; b < grid; ++b) {
+    GenCta& c = ctas[b];
+    const int64_t upto = cost * (b + 1) / grid;
+    while (t < P->nparts && pr >= pairs(t)) {
+      ++t;
+      pr = 0;
+    }
+    c.pair0 = t < P->nparts ? pair_off[t] + pr : pair_off[P->nparts];
+    c.np = 0;
+    c.in0 = t < P->nparts ? P->in_off[t] : 0;
+    int32_t last = t;
+    while (t < P->nparts && done < upto) {
+      if (pr >= pairs(t)) {
+        ++t;
+        pr = 0;
+        continue;
+      }
+      const int64_t pc = pair_cost(t);
+      const int32_t take = (int32_t)std::min<int64_t>(pairs(t) - pr, (upto - done + pc - 1) / pc);
+      c.np += take;
+      pr += take;
+      done += take * pc;
+      last = t;
+    }
+    c.nin = c.np > 0 ? P->in_off[last + 1] - c.in0 : 0;
+    vmax = std::max(vmax, c.nin);
+    if (c.np > kGenThreads) return VTM_OK;
+    c.i0 = (int32_t)(P->n_in * b / grid);
+    c.i1 = (int32_t)(P->n_in * (b + 1) / grid);
+    c.q0 = run_start(c.i0);
+    c.q1 = run_start(c.i1);
+  }
+  vmax = (vmax + 1) / 2 * 2;
+  const int64_t fixed = (int64_t)kGenThreads * 16 + 12 * (int64_t)vmax + 8 * kGenThreads;
+  int optin = 0, fits = 0;
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->device);
+  cudaFuncAttributes fa{};
+  VTM_CUDA_TRY(cudaFuncGetAttributes(&fa, general_resident_kernel));
+  const int nslots = (int)((optin - (int64_t)fa.sharedSizeBytes - fixed) / (kGenThreads * 16));
+  if (nslots < kGenMinSlots) return VTM_OK;
+  P->gen_smem = fixed + (int64_t)nslots * kGenThreads * 16;
+  // the same limit for every plan: another thread's plan never lowers it
+  VTM_CUDA_TRY(cudaFuncSetAttribute(general_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    optin - (int)fa.sharedSizeBytes));
+  VTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, general_resident_kernel, kGenThreads + 32,
+                                                             (size_t)P->gen_smem));
+  if (fits < 1) return VTM_OK;
+  cudaStream_t s = P->stream;
+  VTM_TRY(upload(P->d_gen_ctas, ctas, s));
+  VTM_TRY(upload(P->d_gen_pair, pair_off, s));
+  VTM_TRY(upload(P->d_gen_res, res_in, s));
+  VTM_TRY(dev_alloc(P->d_gen_part, 64 + 2 * (size_t)grid * sizeof(double)));
+  VTM_CUDA_TRY(cudaStreamSynchronize(s));  // the host lists are about to go
+  P->gen_nslots = nslots;
+  P->gen_vmax = vmax;
+  P->gen_ctas = grid;
+  return VTM_OK;
+}
+
+static vtm_status general_sweeps_resident(vtm_plan_s* P, int budget, double* hist, int hist_len, int* sweep_out,
+                                          int* flag_out) {
+  cudaStream_t s = P->stream;
+  GenRes a{};
+  a.E = P->d_E.as<double>();
+  a.E_off = P->d_E_off.as<int64_t>();
+  a.E_ld = P->d_E_ld.as<int32_t>();
+  a.in_off = P->d_in_off.as<int32_t>();
+  a.out_off = P->d_out_off.as<int32_t>();
+  a.pair_off = P->d_gen_pair.as<int32_t>();
+  a.ctas = P->d_gen_ctas.as<GenCta>();
+  a.in_src = P->d_in_src.as<int32_t>();
+  a.in_own_out = P->d_in_own_out.as<int32_t>();
+  a.res_in = P->d_gen_res.as<int32_t>();
+  a.in_kind = P->d_in_kind.as<uint8_t>();
+  a.res_run = P->d_res_run.as<uint8_t>();
+  a.coef = P->d_in_coef.as<double>();
+  a.dsc = P->d_in_d.as<double>();
+  a.c = P->d_cg.as<double>();
+  a.gin = P->d_gin.as<double>();
+  a.gout = P->d_gout.as<double>();
+  a.n_in = P->n_in;
+  a.n_out = P->n_out;
+  a.ctrl = P->d_ctrl.as<SweepCtrl>();
+  a.bar = reinterpret_cast<unsigned long long*>(P->d_gen_part.p);
+  a.part = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(P->d_gen_part.p) + 64);
+  a.hist = hist;
+  a.hist_len = hist_len;
+  a.nparts = P->nparts;
+  a.nslots = P->gen_nslots;
+  a.vmax = P->gen_vmax;
+  a.max_polls = 1u << 22;  // seconds: a bound, not a limit that a solve can meet
+  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gen_part.p, 0, 64, s));
+  void* args[] = {&a};
+  VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
+  VTM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)general_resident_kernel, dim3(P->gen_ctas),
+                                           dim3(kGenThreads + 32), args, (size_t)P->gen_smem, s));
+  VTM_CUDA_TRY(cudaEventRecord(P->evs1, s));
+  VTM_CUDA_TRY(cudaMemcpyAsync(P->h_ctrl, P->d_ctrl.p, sizeof(SweepCtrl), cudaMemcpyDeviceToHost, s));
+  VTM_CUDA_TRY(cudaStreamSynchronize(s));
+  float ms = 0.f;
+  VTM_CUDA_TRY(cudaEventElapsedTime(&ms, P->evs0, P->evs1));
+  P->sweep_ms += ms;
+  const SweepCtrl& r = *P->h_ctrl;
+  P->sweep_launch_count += std::max(r.k - 1, 1);  // sweeps run by the one launch
+  P->launch_count += 1;
+  if (r.flag == 5) {
+    set_detail("vtm_solve: a bounded wait of the resident sweeps ran out");
+    return VTM_ETIMEOUT;
+  }
+  *flag_out = r.flag;
+  *sweep_out = r.flag == 1 ? r.conv_sweep : std::min(r.k - 1, budget);
+  return VTM_OK;
+}
+
 vtm_status build_general_operators(vtm_plan_s* P) {
   cudaStream_t s = P->stream;
   const size_t bytes = std::max<int64_t>(P->E_elems, 8) * sizeof(double);
@@ -281,7 +604,9 @@ vtm_status general_sweeps(vtm_plan_s* P, double bnorm2, double target2, int budg
   *P->h_ctrl = h;
   VTM_CUDA_TRY(cudaMemcpyAsync(P->d_ctrl.p, P->h_ctrl, sizeof(SweepCtrl), cudaMemcpyHostToDevice, s));
   VTM_CUDA_TRY(cudaMemsetAsync(P->d_gin.p, 0, 2 * std::max<int64_t>(P->n_in, 1) * sizeof(double), s));
-  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gout.p, 0, 2 * std::max<int64_t>(P->n_out, 1) * sizeof(double), s));
+  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gout.p, 0, kGenSlots * std::max<int64_t>(P->n_out, 1) * sizeof(double), s));
+  if (P->gen_ctas == 0) VTM_TRY(plan_general_resident(P));
+  if (P->gen_ctas > 0) return general_sweeps_resident(P, budget, hist, hist_len, sweep_out, flag_out);
   // four groups of up to 256 threads per tile (one output each; eight groups
   // of 128 measured slower on the 1024^2 VCCS grid)
   constexpr int KS = 4;

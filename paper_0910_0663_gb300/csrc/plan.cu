@@ -608,7 +608,7 @@ static vtm_status build_general(vtm_plan_s* P) {
   VTM_TRY(upload(P->d_in_tile, in_tile, st));
   VTM_TRY(dev_alloc(P->d_cg, std::max<int64_t>(P->n_out, 1) * sizeof(double)));
   VTM_TRY(dev_alloc(P->d_gin, 2 * std::max<int64_t>(P->n_in, 1) * sizeof(double)));
-  VTM_TRY(dev_alloc(P->d_gout, 2 * std::max<int64_t>(P->n_out, 1) * sizeof(double)));
+  VTM_TRY(dev_alloc(P->d_gout, kGenSlots * std::max<int64_t>(P->n_out, 1) * sizeof(double)));
   VTM_CUDA_TRY(cudaStreamSynchronize(st));
   return VTM_OK;
 }
@@ -619,7 +619,7 @@ using namespace vtm;
 
 std::vector<DevBuf*> vtm_plan_s::all_bufs() {
   return {&tabs.node_off, &tabs.bw, &tabs.band_off, &tabs.port_off, &tabs.T_off, &tabs.T_ld,
-          &tabs.order, &d_rowptr, &d_colidx, &d_vals, &d_perm, &d_iperm, &d_Lc, &d_Uc, &d_Lc32, &d_Uc32, &d_v32, &d_v32b, &d_bb_off, &d_bb_order, &d_bb_Li, &d_bb_Ui, &d_bb_Li32, &d_bb_Ui32, &d_refl_items, &d_refl_order, &d_refl_scratch, &d_dg_items, &d_dg_chunks, &d_dg_off, &d_dg_T, &d_dg_texp, &d_dg_w, &d_dg_wexp, &d_res, &d_slabs, &d_slab_part, &d_cut_p1, &d_cut_p2, &d_cut_flags, &d_ppij, &d_ppji, &d_port_g, &d_port_W, &d_port_d,
+          &tabs.order, &d_rowptr, &d_colidx, &d_vals, &d_perm, &d_iperm, &d_Lc, &d_Uc, &d_Lc32, &d_Uc32, &d_v32, &d_v32b, &d_bb_off, &d_bb_order, &d_bb_Li, &d_bb_Ui, &d_bb_Li32, &d_bb_Ui32, &d_refl_items, &d_refl_order, &d_refl_scratch, &d_dg_items, &d_dg_chunks, &d_dg_off, &d_dg_T, &d_dg_texp, &d_dg_w, &d_dg_wexp, &d_gen_ctas, &d_gen_pair, &d_gen_res, &d_gen_part, &d_res, &d_slabs, &d_slab_part, &d_cut_p1, &d_cut_p2, &d_cut_flags, &d_ppij, &d_ppji, &d_port_g, &d_port_W, &d_port_d,
           &d_lag_pos, &d_lag_back, &d_lag_rho, &d_in_item, &d_out_item, &d_vals_new, &d_port_tile, &d_ell_val, &d_ell_col, &d_ell_len,
           &d_port_loc, &d_port_pos, &d_tdesc,
           &d_twin, &d_beta, &d_bout, &d_beta32, &d_bout32, &d_rho, &d_kd, &d_kd32, &d_run, &d_T64, &d_T32, &d_T16, &d_Tp32, &d_Tp16, &d_Tpdf, &d_dfstate, &d_cdf, &d_kddf, &d_nbr_off, &d_nbr, &d_done, &d_flow, &d_part4, &d_fstate32, &d_c64, &d_c32, &d_state64,

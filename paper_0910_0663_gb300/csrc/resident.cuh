@@ -33,6 +33,8 @@
 // one-warp-per-tile kernels stay: shared memory then holds few of the blocks.
 #pragma once
 
+#include "gridctl.cuh"
+
 namespace vtm {
 
 // tile warps per CTA: with the control warp 128 registers per thread, and 168 for
@@ -69,61 +71,11 @@ struct ResArgs {
   void* state3;
   int64_t nports;
   SweepCtrl* ctrl;
-  // low word: arrivals; high word: the decision, (flag << 28) | the sweep it was
-  // made in (a CTA that reads the word late must not act on the next sweep's
-  // decision); bit 63: a wait ran out
-  unsigned long long* bar;
+  unsigned long long* bar;  // the barrier word (gridctl.cuh)
   double* part;             // [2][grid]
   double* hist;
   int hist_len, nparts, pp, tpc, wpt, nres;
   uint32_t max_polls;
-};
-
-// The residual rule of sweep_decide with its state in the deciding thread.
-struct ResDecision {
-  double tol2, bnorm2, first, best, last;
-  int k_max, stall, best_k, conv;
-  __device__ void load(const SweepCtrl* c) {
-    tol2 = c->tol2;
-    bnorm2 = c->bnorm2;
-    first = best = last = 0.0;
-    k_max = c->k_max;
-    stall = c->stall;
-    best_k = conv = 0;
-  }
-  __device__ int close(int k, double tot, double* hist, int hist_len) {
-    int flag = 0;
-    if (k > 1) {
-      const int ks = k - 1;
-      if (hist && ks <= hist_len) hist[ks - 1] = sqrt(tot / bnorm2);
-      if (ks == 1) first = tot;
-      last = tot;
-      if (ks == 1 || tot < 0.81 * best) {
-        best = tot;
-        best_k = ks;
-      }
-      if (!isfinite(tot) || (ks > 1 && tot > 1e12 * first && first > 0)) {
-        flag = 3;
-      } else if (tot <= tol2) {
-        flag = 1;
-        conv = ks;
-      } else if (stall > 0 && ks - best_k >= stall) {
-        flag = 4;
-        conv = ks;
-      }
-    }
-    if (!flag && k >= k_max) flag = 2;
-    return flag;
-  }
-  __device__ void store(SweepCtrl* c, int k, int flag) const {
-    c->k = k + 1;
-    c->conv_sweep = conv;
-    c->best_k = best_k;
-    c->best_res2 = best;
-    c->first_res2 = first;
-    c->last_res2 = last;
-    c->flag = flag;
-  }
 };
 
 // The incident waves of a tile in shared memory.  Double-float keeps them in the
@@ -171,12 +123,6 @@ __host__ __device__ constexpr size_t res_base_bytes(int pp, int tpc, int warps) 
   using M = ResMode<TT>;
   return (size_t)tpc * pp * (ResWaves<TT>::kBytes + 4 * sizeof(typename M::WV) + 4) +
          (size_t)warps * pp * sizeof(typename M::AC);
-}
-
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
 }
 
 // One lane's share of a packed block: rows r1 and r1 + 8 (r1 = lane / 4),
@@ -395,13 +341,6 @@ __device__ __forceinline__ double res_partial(const typename ResMode<TT>::WV* sv
   return v * pow2d(2 * e);
 }
 
-// fixed-order sum of the warps' partials (one warp, valid in lane 0)
-__device__ __forceinline__ double res_sum(const double* part, int count, int lane) {
-  double v = lane < count ? part[lane] : 0.0;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 template <class TT, int PPL>
 __global__ void __launch_bounds__(32 * (res_warps(std::is_same<TT, double>::value) + 1), 1)
     sweep_resident_kernel(const ResArgs A) {
@@ -431,45 +370,7 @@ __global__ void __launch_bounds__(32 * (res_warps(std::is_same<TT, double>::valu
   __syncthreads();
   if (warp == nw) {
     // ---- control warp ----
-    ResDecision dec;
-    dec.load(A.ctrl);
-    for (int k = 1;; ++k) {
-      __syncthreads();  // the waves of sweep k - 1 are out and the flag is read
-      if (*((volatile int*)&s_flag)) break;
-      int f = 0;
-      if (k > 1) {
-        const double v = res_sum(s_part[(k - 1) & 1], nw, lane);
-        if (lane == 0) A.part[(size_t)((k - 1) & 1) * gridDim.x + blockIdx.x] = v;
-        if (blockIdx.x == 0 && k > 2) {  // the partials of sweep k - 2 came with barrier k - 1
-          const double* pk = A.part + (size_t)(k & 1) * gridDim.x;
-          double t = 0.0;
-          for (int i = lane; i < (int)gridDim.x; i += 32) t += __ldcg(pk + i);
-          for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(FULL, t, o);
-          if (lane == 0 && (f = dec.close(k - 2, t, A.hist, A.hist_len))) dec.store(A.ctrl, k - 2, f);
-        }
-      }
-      __syncthreads();  // every wave of sweep k is written
-      if (lane == 0) {
-        if (f) atomicAdd(A.bar, (unsigned long long)((uint32_t)f << 28 | (uint32_t)k) << 32);
-        __threadfence();  // the CTA's waves and partial before its arrival
-        atomicAdd(A.bar, 1ull);
-        const unsigned need = (unsigned)k * gridDim.x;
-        uint32_t i = 0;
-        unsigned long long w;
-        while (true) {
-          w = ld_acquire_u64(A.bar);
-          if ((unsigned)w >= need || (w >> 63)) break;
-          if (++i >= A.max_polls) {  // give up; the word tells every CTA still waiting
-            atomicCAS(&A.ctrl->flag, 0, 5);
-            atomicOr(A.bar, 1ull << 63);
-            w = 1ull << 63;
-            break;
-          }
-        }
-        if (w >> 63) *((volatile int*)&s_flag) = 5;
-        else if ((uint32_t)(w >> 32) && (int)((w >> 32) & 0x0fffffffu) == k) *((volatile int*)&s_flag) = (int)(w >> 60);
-      }
-    }
+    res_control(A.ctrl, A.bar, A.part, A.hist, A.hist_len, A.max_polls, &s_flag, s_part[0], 16, nw, lane);
   } else {
     // ---- tile warps ----
     const int slot = warp / wpt, part = warp % wpt;

@@ -304,6 +304,10 @@ struct vtm_plan_s {
   int64_t E_elems = 0;
   int32_t max_in = 0, max_out = 0;
   int64_t n_in = 0, n_out = 0;
+  // channel-form sweeps in one launch (gen_ctas: 0 not planned, -1 not possible)
+  vtm::DevBuf d_gen_ctas, d_gen_pair, d_gen_res, d_gen_part;
+  int gen_ctas = 0, gen_nslots = 0, gen_vmax = 0;
+  int64_t gen_smem = 0;
   vtm::DevBuf d_in_off, d_out_off, d_in_src, d_in_kind, d_in_twin, d_in_own_out, d_in_loc,
       d_res_perm, d_res_run, d_out_loc, d_in_coef, d_in_sigma, d_out_scale, d_out_diag, d_E_off,
       d_E_ld, d_E, d_cg, d_gin, d_gout, d_in_tile, d_in_d;
@@ -372,6 +376,7 @@ vtm_status ensure_host_ports(vtm_plan_s* P);
 // general.cu (channel form: lagged couplings and block Jacobi)
 vtm_status build_general_operators(vtm_plan_s* P);
 vtm_status general_const(vtm_plan_s* P, const double* x0_perm);
+constexpr int kGenSlots = 8;  // slots of the outputs (the launch-per-sweep form uses two)
 vtm_status general_sweeps(vtm_plan_s* P, double bnorm2, double target2, int budget, double* hist,
                           int hist_len, int* sweep_out, int* flag_out);
 vtm_status general_inject(vtm_plan_s* P, int sweep, double* v);
