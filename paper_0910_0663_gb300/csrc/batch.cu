@@ -2274,7 +2274,7 @@ vtm_status ensure_vals_df(vtm_plan_s* P) {
 }
 
 // Lists and digits of the tensor-core FP64 sweep; *ok = false where it does not serve.
-static vtm_status prepare_digits(vtm_plan_s* P, int nt8, bool* ok) {
+static vtm_status prepare_digits(vtm_plan_s* P, int ngroups, bool* ok) {
   cudaStream_t s = P->stream;
   *ok = false;
   if (P->dg_res == 0) {
@@ -2286,18 +2286,18 @@ static vtm_status prepare_digits(vtm_plan_s* P, int nt8, bool* ok) {
     for (int32_t t = 0; t < P->nparts; ++t) {
       const int32_t p = P->port_off[t + 1] - P->port_off[t], nb = (p + 15) / 16;
       off[t] = blocks;
-      for (int32_t m = 0; m < nb; m += kDgBlocks) items.push_back(DgItem{t, m, kb, (int32_t)chunks.size(), blocks, 0});
+      for (int32_t m = 0; 128 * m < p; ++m) items.push_back(DgItem{t, m, kb, (int32_t)chunks.size(), blocks, 0});
       for (int32_t m = 0; m < p; m += 16 * kDgChunk) chunks.push_back(DgChunk{t, m, kb + m / 16, 0});
       kb += nb;
-      blocks += (int64_t)nb * nb;
+      blocks += (int64_t)nb * ((p + 7) / 8) * kDg * 16;  // 16-byte units
     }
     P->dg_chunks = (int)chunks.size();
     for (int32_t t = 0; t < P->nparts; ++t)  // the residual's items after them
       for (int32_t m = 0; m < P->port_off[t + 1] - P->port_off[t]; m += 32) chunks.push_back(DgChunk{t, m, 0, 0});
     P->dg_res = (int)chunks.size() - P->dg_chunks;
     auto cost = [&](const DgItem& d) {
-      const int nb = (P->port_off[d.tile + 1] - P->port_off[d.tile] + 15) / 16;
-      return nb * std::min(kDgBlocks, nb - d.mb0);
+      const int p = P->port_off[d.tile + 1] - P->port_off[d.tile];
+      return (p + 15) / 16 * std::min(16, (p - 128 * d.m + 7) / 8);
     };
     std::stable_sort(items.begin(), items.end(), [&](const DgItem& a, const DgItem& b) { return cost(a) > cost(b); });
     VTM_TRY(upload(P->d_dg_items, items, s));
@@ -2308,10 +2308,10 @@ static vtm_status prepare_digits(vtm_plan_s* P, int nt8, bool* ok) {
     P->dg_blocks = blocks;
     P->dg_kb = kb;
   }
-  const size_t bytes = (size_t)P->dg_blocks * kDg * 32 * sizeof(uint4);
+  const size_t bytes = std::max<size_t>((size_t)P->dg_blocks * sizeof(uint4), 16);
   if (bytes > ((size_t)32 << 30)) return VTM_OK;
   if (dev_alloc(P->d_dg_T, bytes) != VTM_OK || dev_alloc(P->d_dg_texp, P->port_node.size() * sizeof(int)) != VTM_OK ||
-      dev_alloc(P->d_dg_w, (size_t)P->dg_kb * nt8 * kDg * 32 * sizeof(uint2)) != VTM_OK ||
+      dev_alloc(P->d_dg_w, (size_t)P->dg_kb * ngroups * kDg * 256) != VTM_OK ||
       dev_alloc(P->d_dg_wexp, (size_t)P->dg_chunks * 64 * sizeof(int)) != VTM_OK) {
     cudaGetLastError();
     dev_free(P->d_dg_T);
@@ -2324,7 +2324,7 @@ static vtm_status prepare_digits(vtm_plan_s* P, int nt8, bool* ok) {
                                                    P->d_dg_texp.as<int>());
     pack_digits_kernel<<<dim3(P->nparts, 16), 256, 0, s>>>(
         P->d_T64.as<double>(), P->tabs.T_off.as<int64_t>(), P->tabs.T_ld.as<int32_t>(), P->tabs.port_off.as<int32_t>(),
-        P->d_dg_off.as<int64_t>(), P->d_dg_texp.as<int>(), P->d_dg_T.as<uint4>());
+        P->d_dg_off.as<int64_t>(), P->d_dg_texp.as<int>(), P->d_dg_T.as<uint2>());
     VTM_CUDA_TRY(cudaGetLastError());
     P->launch_count += 2;
     P->dg_ready = true;
@@ -2408,7 +2408,9 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
   // that passes 32 GB or memory runs out)
   const int nt8 = (R + 7) / 8;
   bool dg_ok = false;
-  if (prec == VTM_PREC_FP64 && npt > 0 && P->opts.batch_kernel == 0) VTM_TRY(prepare_digits(P, nt8, &dg_ok));
+  // 8-column groups per work item, items side by side (their T_P digits from HBM once)
+  const int dg_nt = nt8 == 4 ? 2 : std::min(nt8, kDgMaxNt), dg_ny = (nt8 + dg_nt - 1) / dg_nt;
+  if (prec == VTM_PREC_FP64 && npt > 0 && P->opts.batch_kernel == 0) VTM_TRY(prepare_digits(P, dg_nt * dg_ny, &dg_ok));
   const bool lowp = prec != VTM_PREC_FP64;
   const size_t wsz = lowp ? sizeof(float) : sizeof(double);
   VTM_TRY(dev_alloc(P->d_bV, (size_t)n * R * sizeof(double)));
@@ -2578,26 +2580,24 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
           return;
         }
         if (kv == 5) {  // FP64 on the tensor cores: the waves' digits, then the products
-          const int NT = nt8 == 4 ? 2 : std::min(nt8, kDgMaxNt), ny = (nt8 + NT - 1) / NT;
-          auto go_dg = [&](auto* kern) {
-            const size_t smem = kDgStages * (kDgBlocks * kDg * 32 * sizeof(uint4) + (size_t)NT * kDg * 32 * sizeof(uint2));
-            if (dry) {
-              cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-              return;
-            }
-            batch_digits_kernel<<<P->dg_chunks + P->dg_res, 256, 0, s>>>(
-                P->d_dg_chunks.as<DgChunk>(), P->dg_chunks, P->tabs.port_off.as<int32_t>(), P->d_twin.as<int32_t>(),
-                P->d_kd.as<double2>(), P->d_run.as<uint8_t>(), P->d_bstate.as<double>(), npt, R, nt8,
-                P->d_dg_w.as<uint2>(), P->d_dg_wexp.as<int>(), P->d_bctrl.as<BatchCtrl>(), P->d_bpart.as<double>(),
-                P->d_btol2.as<double>(), bhist, bhist_len);
-            kern<<<P->dg_items * ny, 32 * kDgBlocks, smem, s>>>(
-                P->d_dg_items.as<DgItem>(), P->tabs.port_off.as<int32_t>(), P->d_dg_T.as<uint4>(),
-                P->d_dg_texp.as<int>(), P->d_dg_w.as<uint2>(), P->d_dg_wexp.as<int>(), nt8, ny, P->d_bc.as<double>(),
-                P->d_bstate.as<double>(), npt, R, P->d_bctrl.as<BatchCtrl>());
-          };
-          if (NT == 1) go_dg(batch_sweep_digits_kernel<1>);
-          else if (NT == 2) go_dg(batch_sweep_digits_kernel<2>);
-          else go_dg(batch_sweep_digits_kernel<3>);
+          const size_t smem = dg_smem(dg_nt);
+          int sms = 152;
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device);
+          if (dry) {
+            cudaFuncSetAttribute(batch_sweep_digits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)dg_smem(kDgMaxNt));
+            return;
+          }
+          batch_digits_kernel<<<P->dg_chunks + P->dg_res, 256, 0, s>>>(
+              P->d_dg_chunks.as<DgChunk>(), P->dg_chunks, P->tabs.port_off.as<int32_t>(), P->d_twin.as<int32_t>(),
+              P->d_kd.as<double2>(), P->d_run.as<uint8_t>(), P->d_bstate.as<double>(), npt, R, dg_nt, dg_ny,
+              P->d_dg_w.as<uint32_t>(), P->d_dg_wexp.as<int>(), P->d_bctrl.as<BatchCtrl>(), P->d_bpart.as<double>(),
+              P->d_btol2.as<double>(), bhist, bhist_len);
+          batch_sweep_digits_kernel<<<std::min(P->dg_items * dg_ny, sms), kDgThreads, smem, s>>>(
+              P->d_dg_items.as<DgItem>(), P->dg_items, dg_nt, dg_ny, P->tabs.port_off.as<int32_t>(),
+              P->d_dg_T.as<unsigned char>(), P->d_dg_texp.as<int>(), P->d_dg_w.as<unsigned char>(),
+              P->d_dg_wexp.as<int>(), P->d_bc.as<double>(), P->d_bstate.as<double>(), npt, R,
+              P->d_bctrl.as<BatchCtrl>());
           return;
         }
         auto go = [&](auto* kern, int threads, const auto* T, const auto* cc, auto* st) {

@@ -15,24 +15,24 @@
 // The nine group sums join as 64-bit integers, one FP64 rounding per 256 inputs.
 //
 // Per sweep two launches.  batch_digits_kernel: the incident waves (twins' outgoing
-// ones) and their digits in the B fragment order of mma.m16n8k16 (a CTA per 256
-// ports), the residual of sweep k - 1 in FP64 (a CTA per 32 ports); its last CTA
-// closes the sweep before, so a converged sweep never reads T_P.  batch_sweep_digits_kernel (a CTA
-// per 128 outputs and up to 24 columns, 8 warps of 16 outputs): 45 MMAs per 16
-// inputs and 8 columns, T_P's digits (fragment order, built once per
-// factorisation, 18 bytes per entry) and W's through a three-stage cp.async ring.
-// Bound: the rate of mma.sync (about 4 cycles per m16n8k16 and SM); its floor in HBM
-// traffic (18 bytes of digits per entry) is a third of that at 24 columns.  Measured
-// per sweep, thermal grid of 147,456 nodes in 110 boxes, 18 columns: FP64 CUDA
-// cores 6.54 ms, here 0.08 + 0.43 ms (the same with 15 warps of 8 columns: 0.45).
+// ones) and their digits in the B operand's core matrices (a CTA per 256 ports), the
+// residual of sweep k - 1 in FP64 (a CTA per 32 ports); its last CTA closes the sweep
+// before, so a converged sweep never reads T_P.  batch_sweep_digits_kernel (persistent,
+// one CTA per SM; an item is 128 outputs and up to 24 columns): tcgen05.mma with the
+// nine groups of sums side by side in TMEM (below), T_P's digits (built once per
+// factorisation, 18 bytes per entry) and W's by bulk copies through a ring of five
+// steps, two sets of accumulators so that a chunk is joined while the next one runs.
+// Bound: HBM (18 bytes of digits per entry of T_P).  Measured per sweep, thermal grid
+// of 147,456 nodes in 110 boxes, 18 columns: FP64 CUDA cores 6.54 ms; digits with
+// mma.sync 0.08 + 0.43 ms (its rate, about 4 cycles per m16n8k16 and SM); here
+// 0.08 + 0.21 ms, the same bits.
 // Errors of the iterates against quad precision are those of the FP64 kernel to two
 // digits (1 to 20 sweeps; 3e-16 thermal, 8e-15 grids).
 
 constexpr int kDg = 9;          // digits
 constexpr int kDgChunk = 16;    // 16-input blocks between two joins of the group sums
-constexpr int kDgStages = 3;
-constexpr int kDgMaxNt = 3;     // 8-column groups per work item
-constexpr int kDgBlocks = 8;    // 16-output blocks (warps) per work item
+constexpr int kDgStages = 5;
+constexpr int kDgMaxNt = 3;     // 8-column groups per work item (nine groups of 24 columns: 216 of 256 TMEM columns)
 
 // biased exponent of |v| (0x7ff: not finite)
 __device__ __forceinline__ int exp_bits(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7ff); }
@@ -87,32 +87,38 @@ __global__ void __launch_bounds__(256) row_exponents_kernel(const double* __rest
   }
 }
 
-// T_P's digits: block (mb, kb) of a tile at (off + mb nb + kb) 9 32 uint4s, digit i
-// at [i][lane] = the lane's A fragment (rows g, g + 8, columns 2t, 2t + 1, 2t + 8, 2t + 9)
+// T_P's digits in the canonical K-major layout of tcgen05.mma without swizzle (8 x 8
+// core matrices of 128 bytes, the two of a row group's 16 inputs adjacent): per tile,
+// blocks of 128 outputs, per block every step of 16 inputs, per step the nine digits
+// of the block's row groups.  A block's last row group may be ragged, its steps
+// shorter; what a short step leaves of its stage only reaches rows past the tile.
+__host__ __device__ __forceinline__ int dg_groups(int p, int m) { return min(16, (p - 128 * m + 7) / 8); }
+
 __global__ void __launch_bounds__(256) pack_digits_kernel(const double* __restrict__ T,
                                                           const int64_t* __restrict__ T_off,
                                                           const int32_t* __restrict__ T_ld,
                                                           const int32_t* __restrict__ port_off,
                                                           const int64_t* __restrict__ dg_off,
-                                                          const int* __restrict__ E, uint4* __restrict__ out) {
+                                                          const int* __restrict__ E, uint2* __restrict__ out) {
   const int t = blockIdx.x, p0 = port_off[t], p = port_off[t + 1] - p0, ld = T_ld[t];
-  const int nb = (p + 15) / 16;
+  const int nb = (p + 15) / 16, ng = (p + 7) / 8;
   const double* Tb = T + T_off[t];
-  const int lane = threadIdx.x & 31, g = lane >> 2, t2 = 2 * (lane & 3);
-  for (int b = blockIdx.y * 8 + (threadIdx.x >> 5); b < nb * nb; b += gridDim.y * 8) {
-    const int mb = b / nb, kb = b - mb * nb;
-    int d[8][kDg];
+  // a warp takes 16 inputs of a row group: lane = (quad of inputs, row)
+  const int lane = threadIdx.x & 31, row = lane & 7, kq = lane >> 3;
+  for (int b = blockIdx.y * 8 + (threadIdx.x >> 5); b < nb * ng; b += gridDim.y * 8) {
+    const int gr = b / nb, kb = b - gr * nb, m = gr / 16, rg = dg_groups(p, m);
+    const int s = 8 * gr + row, q = 16 * kb + 4 * kq;
+    int d[4][kDg];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int s = 16 * mb + g + 8 * ((e >> 1) & 1), q = 16 * kb + t2 + (e & 1) + 8 * (e >> 2);
-      const double v = s < p && q < p ? Tb[(size_t)q * ld + s] : 0.0;
+    for (int e = 0; e < 4; ++e) {
+      const double v = s < p && q + e < p ? Tb[(size_t)(q + e) * ld + s] : 0.0;
       digits_of(v, s < p ? E[p0 + s] : 0, d[e]);
     }
-    uint4* o = out + (dg_off[t] + b) * kDg * 32 + lane;
+    uint2* o = out + dg_off[t] * 2 + ((int64_t)m * nb * 16 + (int64_t)kb * rg) * kDg * 32 + (gr & 15) * 32 +
+               (kq >> 1) * 16 + row * 2 + (kq & 1);
 #pragma unroll
     for (int i = 0; i < kDg; ++i)
-      o[i * 32] = make_uint4(bf16_pair(d[0][i], d[1][i]), bf16_pair(d[2][i], d[3][i]), bf16_pair(d[4][i], d[5][i]),
-                             bf16_pair(d[6][i], d[7][i]));
+      o[(int64_t)i * rg * 32] = make_uint2(bf16_pair(d[0][i], d[1][i]), bf16_pair(d[2][i], d[3][i]));
   }
 }
 
@@ -125,7 +131,7 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
     const DgChunk* __restrict__ chunks, int nchunks, const int32_t* __restrict__ port_off,
     const int32_t* __restrict__ twin, const double2* __restrict__ kd, const uint8_t* __restrict__ run,
     double* __restrict__ state, int64_t nports,
-    int R, int nt, uint2* __restrict__ wd, int* __restrict__ wexp, BatchCtrl* __restrict__ ctrl,
+    int R, int NT, int ny, uint32_t* __restrict__ wd, int* __restrict__ wexp, BatchCtrl* __restrict__ ctrl,
     double* __restrict__ partials, const double* __restrict__ tol2, double* __restrict__ hist, int hist_len) {
   __shared__ double rsq[32][64];
   __shared__ double red[64];
@@ -166,12 +172,12 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
     }
     __syncthreads();
     if (tid < 64) wexp[blockIdx.x * 64 + tid] = cmax[tid] - 1022;
-    // digits, a pair of rows per item: (16-input block, column group, lane, half)
-    const int kbn = k > 1 ? (m1 - ch.m0 + 15) / 16 : 0;
-    uint32_t* out = reinterpret_cast<uint32_t*>(wd);
+    // digits, a pair of rows per item, in the K-major core matrices of the B operand:
+    // [16 inputs][column group of the items][digit][8 columns][input half][column][input]
+    const int kbn = k > 1 ? (m1 - ch.m0 + 15) / 16 : 0, nt = NT * ny;
     for (int i = tid; i < kbn * nt * 64; i += 256) {
-      const int h = i & 1, lane = (i >> 1) & 31, u = i >> 6, n = u % nt, kb = u / nt;
-      const int c = 8 * n + (lane >> 2), q = ch.m0 + 16 * kb + 2 * (lane & 3) + 8 * h;
+      const int w = i & 63, u = i >> 6, n = u % nt, kb = u / nt;
+      const int c = 8 * n + ((w >> 2) & 7), q = ch.m0 + 16 * kb + 8 * (w >> 5) + 2 * (w & 3);
       int d0[kDg], d1[kDg];
       const bool col = c < R;
       const double v0 = col && q < p ? prev[(size_t)twin[p0 + q] * 2 * R + R + c] : 0.0;
@@ -179,9 +185,9 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
       const int E = col ? cmax[c] - 1022 : 0;
       digits_of(v0, E, d0);
       digits_of(v1, E, d1);
-      uint32_t* o = out + ((size_t)(ch.kb + kb) * nt + n) * kDg * 64 + lane * 2 + h;
+      uint32_t* o = wd + (((size_t)(ch.kb + kb) * ny + n / NT) * kDg * NT + n % NT) * 64 + w;
 #pragma unroll
-      for (int j = 0; j < kDg; ++j) o[j * 64] = bf16_pair(d0[j], d1[j]);
+      for (int j = 0; j < kDg; ++j) o[(size_t)j * NT * 64] = bf16_pair(d0[j], d1[j]);
     }
   }
   if (tid == 0) {
@@ -194,121 +200,241 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
   batch_finish(ctrl, partials, gridDim.x - nchunks, R, tol2, hist, hist_len, k, &rsq[0][0]);
 }
 
-// Work item of the sweep: up to kDgBlocks 16-output blocks of a tile.
+// Work item of the sweep: 128 outputs of a tile.
 struct __align__(16) DgItem {
-  int32_t tile, mb0, kb, chunk;  // first 16-output block; W's first block and first chunk of the tile
-  int64_t off;                   // block (0, 0) of the tile's digits
+  int32_t tile, m, kb, chunk;  // block of 128 outputs; W's first 16-input step and first chunk of the tile
+  int64_t off;                 // the tile's digits (16-byte units)
   int64_t pad;
 };
 
-template <int NT>
-__global__ void __launch_bounds__(32 * kDgBlocks, 1) batch_sweep_digits_kernel(
-    const DgItem* __restrict__ items, const int32_t* __restrict__ port_off, const uint4* __restrict__ Td,
-    const int* __restrict__ texp, const uint2* __restrict__ wd, const int* __restrict__ wexp, int nt_all, int ny,
-    const double* __restrict__ c, double* __restrict__ state, int64_t nports, int R,
-    const BatchCtrl* __restrict__ ctrl) {
-  extern __shared__ __align__(16) unsigned char dsm[];
-  const int flag = *((volatile const int*)&ctrl->flag);
-  if (flag) return;
-  const int k = *((volatile const int*)&ctrl->k) - 1;  // the digits kernel has closed the sweep before
-  // the column groups of an item run side by side (its T_P digits from HBM once)
-  const DgItem it = items[blockIdx.x / ny];
-  const int n0 = (blockIdx.x % ny) * NT;  // first 8-column group
+// Per step of 16 inputs nine tcgen05.mma (M = 128): digit i of T_P against the digits
+// 0 .. 8 - i of W side by side (N = (9 - i) nc columns), accumulated at TMEM column
+// i nc -- so the product of digits i and j lands in group i + j, and the first MMA of a
+// chunk clears all groups.  N is a multiple of 16: with an odd number of column groups
+// the last eight columns of an MMA go to a tenth group that nothing reads.
+constexpr int kDgThreads = 320;    // warp 0: copies; warp 1: MMAs; eight warps join
+constexpr uint32_t kDgABytes = kDg * 128 * 16 * 2;
+constexpr uint32_t kDgTmem = 256;  // TMEM columns per accumulator set (two sets)
+constexpr uint32_t dg_b_bytes(int NT) { return kDg * NT * 256; }
+constexpr uint32_t dg_stage(int NT) { return kDgABytes + dg_b_bytes(NT) + 256; }  // (+ the rounded-up N)
+constexpr size_t dg_smem(int NT) { return kDgStages * (size_t)dg_stage(NT) + 1024; }
+
+// canonical K-major, no swizzle: 128 bytes between the two core matrices of 16 inputs,
+// 256 between row groups
+__device__ __forceinline__ uint64_t dg_desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFF) >> 4) | (uint64_t)(128 >> 4) << 16 | (uint64_t)(256 >> 4) << 32 | (uint64_t)1 << 46;
+}
+__device__ __forceinline__ void dg_mma(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t n, uint32_t acc) {
+  // F32 accumulate, BF16 A and B, both K-major, M = 128
+  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// four columns of the nine groups, this warp's 32 rows
+__device__ __forceinline__ void dg_ld(uint32_t addr, uint32_t nc, uint32_t (&v)[kDg][4]) {
+#define DG_R(g) "=r"(v[g][0]), "=r"(v[g][1]), "=r"(v[g][2]), "=r"(v[g][3])
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%36];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%37];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%38];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%39];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16,%17,%18,%19}, [%40];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%20,%21,%22,%23}, [%41];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%24,%25,%26,%27}, [%42];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%28,%29,%30,%31}, [%43];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%32,%33,%34,%35}, [%44];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : DG_R(0), DG_R(1), DG_R(2), DG_R(3), DG_R(4), DG_R(5), DG_R(6), DG_R(7), DG_R(8)
+      : "r"(addr), "r"(addr + nc), "r"(addr + 2 * nc), "r"(addr + 3 * nc), "r"(addr + 4 * nc), "r"(addr + 5 * nc),
+        "r"(addr + 6 * nc), "r"(addr + 7 * nc), "r"(addr + 8 * nc)
+      : "memory");
+#undef DG_R
+}
+
+__global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
+    const DgItem* __restrict__ items, int nitems, int NT, int ny, const int32_t* __restrict__ port_off,
+    const unsigned char* __restrict__ Td, const int* __restrict__ texp, const unsigned char* __restrict__ wd,
+    const int* __restrict__ wexp, const double* __restrict__ c, double* __restrict__ state, int64_t nports, int R,
+    BatchCtrl* __restrict__ ctrl) {
+  extern __shared__ __align__(1024) unsigned char dsm[];
+  __shared__ uint64_t full[kDgStages], empty[kDgStages], tfull[2], tempty[2], drain;
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_k, s_flag;
+  __shared__ volatile int s_abort;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int p0 = port_off[it.tile], p = port_off[it.tile + 1] - p0, nb = (p + 15) / 16;
-  const int mb = it.mb0 + warp;
-  const bool active = mb < nb;
-  constexpr int kA = kDg * 32;       // uint4s of one warp's T_P digits per stage
-  constexpr int kB = NT * kDg * 32;  // uint2s of the W digits per stage
-  constexpr size_t kStage = kDgBlocks * kA * sizeof(uint4) + kB * sizeof(uint2);
-  const int nn = min(NT, nt_all - n0);  // column groups this item has
-  auto issue = [&](int kb) {
-    if (kb < nb) {
-      unsigned char* st = dsm + (kb % kDgStages) * kStage;
-      if (active) {
-        const uint4* src = Td + (it.off + (int64_t)mb * nb + kb) * kA + lane;
-        uint4* dst = reinterpret_cast<uint4*>(st) + warp * kA + lane;
-#pragma unroll
-        for (int i = 0; i < kDg; ++i) cp_async16_cg(dst + i * 32, src + i * 32);
-      }
-      const uint4* bsrc = reinterpret_cast<const uint4*>(wd + ((int64_t)(it.kb + kb) * nt_all + n0) * kDg * 32);
-      uint4* bdst = reinterpret_cast<uint4*>(st) + kDgBlocks * kA;
-      for (int e = tid; e < nn * kDg * 16; e += 32 * kDgBlocks) cp_async16_cg(bdst + e, bsrc + e);
+  if (tid == 0) {
+    s_flag = *((volatile int*)&ctrl->flag);
+    s_k = *((volatile int*)&ctrl->k) - 1;  // the digits kernel has closed the sweep before
+    s_abort = 0;
+    for (int i = 0; i < kDgStages; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], 1);
     }
-    cp_async_commit();
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], 8);
+    }
+    mbar_init(&drain, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (s_flag) return;
+  const int k = s_k, G = gridDim.x, total = nitems * ny;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                 "r"(2 * kDgTmem)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = s_tmem, nc = 8 * NT;
+  unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)dsm + 1023) & ~(uintptr_t)1023);
+  const uint32_t stage = dg_stage(NT), bbytes = dg_b_bytes(NT);
+  // Every wait is bounded; one that runs out sets flag 5 (VTM_ETIMEOUT), and each role
+  // goes on to its end without waiting, copying or issuing.
+  auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    if (s_abort) return false;
+    if (mbar_wait_bounded(bar, parity, kTcPolls)) return true;
+    atomicCAS(&ctrl->flag, 0, 5);
+    s_abort = 1;
+    return false;
   };
-  float acc[NT][kDg][4];
-  double out[NT][4];
-#pragma unroll
-  for (int n = 0; n < NT; ++n)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      out[n][e] = 0.0;
-#pragma unroll
-      for (int g = 0; g < kDg; ++g) acc[n][g][e] = 0.f;
-    }
-  const int g8 = lane >> 2, t2 = 2 * (lane & 3);
-  // the group sums of a chunk joined: S = sum_g acc_g 2^(7 (8 - g)), exact in two
-  // 64-bit halves, scaled by the chunk's column exponents
-  auto join = [&](int chunk) {
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      if (n >= nn) break;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        long long hi = 0, lo = 0;
-#pragma unroll
-        for (int g = 0; g < 4; ++g) hi = hi * 128 + __float2int_rn(acc[n][g][e]);
-#pragma unroll
-        for (int g = 4; g < kDg; ++g) lo = lo * 128 + __float2int_rn(acc[n][g][e]);
-        const double S = fma((double)hi, 34359738368.0, (double)lo);  // hi 2^35 + lo
-        out[n][e] += ldexp(S, wexp[chunk * 64 + 8 * (n0 + n) + t2 + (e & 1)]);
-#pragma unroll
-        for (int g = 0; g < kDg; ++g) acc[n][g][e] = 0.f;
+  // the items by falling cost, the CTAs forth and back
+  auto item_at = [&](int r) { return r * G + ((r & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x); };
+  uint32_t issued = 0;
+  if (warp == 0) {
+    if (lane == 0 && k > 1) {
+      uint32_t g = 0;
+      for (int r = 0, idx; (idx = item_at(r)), r * G < total; ++r) {
+        if (idx >= total) continue;
+        const DgItem it = items[idx / ny];
+        const int y = idx % ny, p = port_off[it.tile + 1] - port_off[it.tile], nb = (p + 15) / 16;
+        const uint32_t dig = dg_groups(p, it.m) * 256;  // bytes of a digit's rows
+        const unsigned char* a = Td + it.off * 16 + (int64_t)it.m * nb * kDgABytes;
+        const unsigned char* b = wd + ((int64_t)it.kb * ny + y) * bbytes;
+        for (int kb = 0; kb < nb; ++kb, ++g) {
+          const uint32_t st = g % kDgStages;
+          if (g >= kDgStages && !wait(&empty[st], (g / kDgStages - 1) & 1)) break;
+          if (s_abort) break;
+          unsigned char* dst = base + st * stage;
+          mbar_arrive_expect_tx(&full[st], kDg * dig + bbytes);
+          issued = g + 1;
+          if (dig == 4096) {
+            bulk_copy_g2s(dst, a, kDgABytes, &full[st]);
+          } else {
+            for (int i = 0; i < kDg; ++i) bulk_copy_g2s(dst + i * 4096, a + i * dig, dig, &full[st]);
+          }
+          bulk_copy_g2s(dst + kDgABytes, b, bbytes, &full[st]);
+          a += kDg * dig;
+          b += (int64_t)ny * bbytes;
+        }
       }
     }
-  };
-  if (k > 1) {
+  } else if (warp == 1) {
+    if (lane == 0 && k > 1) {
+      uint32_t g = 0, ch = 0;
+      for (int r = 0, idx; (idx = item_at(r)), r * G < total; ++r) {
+        if (idx >= total) continue;
+        const int tile = items[idx / ny].tile, nb = (port_off[tile + 1] - port_off[tile] + 15) / 16;
+        for (int kb = 0; kb < nb; ++kb, ++g) {
+          const uint32_t st = g % kDgStages, buf = ch & 1;
+          const bool first = kb % kDgChunk == 0;
+          if (first && ch >= 2 && !wait(&tempty[buf], ((ch >> 1) - 1) & 1)) break;
+          if (!wait(&full[st], (g / kDgStages) & 1)) break;
+          tc_fence_after();
+          const uint32_t a0 = smem_u32(base + st * stage), b0 = a0 + kDgABytes, d0 = tmem + buf * kDgTmem;
+          const uint64_t bd = dg_desc(b0);
 #pragma unroll
-    for (int b = 0; b < kDgStages - 1; ++b) issue(b);
-    for (int kb = 0; kb < nb; ++kb) {
-      cp_async_wait<kDgStages - 2>();
-      __syncthreads();  // the stage has landed; the one refilled below is read
-      issue(kb + kDgStages - 1);
-      if (active) {
-        const unsigned char* st = dsm + (kb % kDgStages) * kStage;
-        const uint4* As = reinterpret_cast<const uint4*>(st) + warp * kA + lane;
-        const uint2* Bs = reinterpret_cast<const uint2*>(st + kDgBlocks * kA * sizeof(uint4)) + lane;
-#pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          if (n < nn) {
-            uint2 b[kDg];
-#pragma unroll
-            for (int j = 0; j < kDg; ++j) b[j] = Bs[(n * kDg + j) * 32];
-#pragma unroll
-            for (int i = 0; i < kDg; ++i) {
-              const uint4 a = As[i * 32];
-#pragma unroll
-              for (int j = 0; i + j < kDg; ++j) mma_bf16(acc[n][i + j], a.x, a.y, a.z, a.w, b[j].x, b[j].y);
-            }
+          for (int i = 0; i < kDg; ++i)
+            dg_mma(d0 + i * nc, dg_desc(a0 + i * 4096), bd, ((kDg - i) * nc + 15) & ~15u, (first && i == 0) ? 0u : 1u);
+          tc_commit(&empty[st]);
+          if (kb % kDgChunk == kDgChunk - 1 || kb == nb - 1) {
+            tc_commit(&tfull[buf]);
+            ++ch;
           }
         }
-        if (kb % kDgChunk == kDgChunk - 1 || kb == nb - 1) join(it.chunk + kb / kDgChunk);
       }
     }
-    cp_async_wait<0>();
-  }
-  if (!active) return;
-  double* cur = state + (size_t)(k & 1) * nports * 2 * R;
+  } else {
+    // eight warps: TMEM lanes 32 (warp % 4).., quads of columns h, h + 2, ...
+    const int quarter = warp & 3, h = (warp - 2) >> 2, nq = 2 * NT;
+    uint32_t ch = 0;
+    double* cur = state + (size_t)(k & 1) * nports * 2 * R;
+    for (int r = 0, idx; (idx = item_at(r)), r * G < total; ++r) {
+      if (idx >= total) continue;
+      const DgItem it = items[idx / ny];
+      const int c0 = (idx % ny) * (int)nc, p0 = port_off[it.tile], p = port_off[it.tile + 1] - p0, nb = (p + 15) / 16;
+      const int s = 128 * it.m + 32 * quarter + lane;
+      double out[kDgMaxNt][4];
 #pragma unroll
-  for (int n = 0; n < NT; ++n) {
+      for (int u = 0; u < kDgMaxNt; ++u)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int s = 16 * mb + g8 + 8 * (e >> 1), r = 8 * (n0 + n) + t2 + (e & 1);
-      if (s < p && r < R) {
+        for (int e = 0; e < 4; ++e) out[u][e] = 0.0;
+      if (k > 1) {
+        const int nch = (nb + kDgChunk - 1) / kDgChunk;
+        for (int j = 0; j < nch; ++j, ++ch) {
+          const uint32_t buf = ch & 1;
+          if (!__all_sync(0xffffffffu, wait(&tfull[buf], (ch >> 1) & 1))) break;  // (the warp together)
+          tc_fence_after();
+#pragma unroll
+          for (int u = 0; u < kDgMaxNt; ++u) {
+            const int q = h + 2 * u;
+            if (q >= nq) break;
+            uint32_t v[kDg][4];
+            dg_ld(tmem + ((uint32_t)(32 * quarter) << 16) + buf * kDgTmem + 4 * q, nc, v);
+            // the groups joined: S = sum_g v_g 2^(7 (8 - g)), exact in two 64-bit halves,
+            // scaled by the chunk's column exponent
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int col = c0 + 4 * q + e;
+              if (col >= R) break;
+              long long hi = 0, lo = 0;
+#pragma unroll
+              for (int g = 0; g < 4; ++g) hi = hi * 128 + __float2int_rn(__uint_as_float(v[g][e]));
+#pragma unroll
+              for (int g = 4; g < kDg; ++g) lo = lo * 128 + __float2int_rn(__uint_as_float(v[g][e]));
+              const double S = fma((double)hi, 34359738368.0, (double)lo);  // hi 2^35 + lo
+              out[u][e] += ldexp(S, wexp[(it.chunk + j) * 64 + col]);
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tempty[buf]);
+        }
+      }
+      if (s < p && !s_abort) {
         const size_t ps = (size_t)(p0 + s);
-        cur[ps * 2 * R + R + r] = c[ps * R + r] + ldexp(out[n][e], texp[ps] - 68);
+        const int te = texp[ps] - 68;
+#pragma unroll
+        for (int u = 0; u < kDgMaxNt; ++u) {
+          const int q = h + 2 * u;
+          if (q >= nq) break;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int col = c0 + 4 * q + e;
+            if (col < R) cur[ps * 2 * R + R + col] = c[ps * R + col] + ldexp(out[u][e], te);
+          }
+        }
       }
     }
   }
+  __syncwarp();
+  // after an abort: copies in flight land before the CTA's shared memory goes, and the
+  // MMAs issued complete before its TMEM (both bounded)
+  if (warp == 0 && lane == 0 && s_abort)
+    for (uint32_t g = issued > kDgStages ? issued - kDgStages : 0; g < issued; ++g)
+      mbar_wait_bounded(&full[g % kDgStages], (g / kDgStages) & 1, kTcPolls);
+  if (warp == 1 && lane == 0 && s_abort) {
+    tc_commit(&drain);
+    mbar_wait_bounded(&drain, 0, kTcPolls);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kDgTmem) : "memory");
 }
