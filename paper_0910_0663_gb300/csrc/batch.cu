@@ -2293,11 +2293,11 @@ static vtm_status prepare_digits(vtm_plan_s* P, int ngroups, bool* ok) {
     }
     P->dg_chunks = (int)chunks.size();
     for (int32_t t = 0; t < P->nparts; ++t)  // the residual's items after them
-      for (int32_t m = 0; m < P->port_off[t + 1] - P->port_off[t]; m += 32) chunks.push_back(DgChunk{t, m, 0, 0});
+      for (int32_t m = 0; m < P->port_off[t + 1] - P->port_off[t]; m += kDgRes) chunks.push_back(DgChunk{t, m, 0, 0});
     P->dg_res = (int)chunks.size() - P->dg_chunks;
     auto cost = [&](const DgItem& d) {
       const int p = P->port_off[d.tile + 1] - P->port_off[d.tile];
-      return (p + 15) / 16 * std::min(16, (p - 128 * d.m + 7) / 8);
+      return (p + 15) / 16 * dg_groups(p, d.m);
     };
     std::stable_sort(items.begin(), items.end(), [&](const DgItem& a, const DgItem& b) { return cost(a) > cost(b); });
     VTM_TRY(upload(P->d_dg_items, items, s));

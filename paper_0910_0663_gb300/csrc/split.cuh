@@ -16,7 +16,7 @@
 //
 // Per sweep two launches.  batch_digits_kernel: the incident waves (twins' outgoing
 // ones) and their digits in the B operand's core matrices (a CTA per 256 ports), the
-// residual of sweep k - 1 in FP64 (a CTA per 32 ports); its last CTA closes the sweep
+// residual of sweep k - 1 in FP64 (a CTA per 64 ports); its last CTA closes the sweep
 // before, so a converged sweep never reads T_P.  batch_sweep_digits_kernel (persistent,
 // one CTA per SM; an item is 128 outputs and up to 24 columns): tcgen05.mma with the
 // nine groups of sums side by side in TMEM (below), T_P's digits (built once per
@@ -25,7 +25,7 @@
 // Bound: HBM (18 bytes of digits per entry of T_P).  Measured per sweep, thermal grid
 // of 147,456 nodes in 110 boxes, 18 columns: FP64 CUDA cores 6.54 ms; digits with
 // mma.sync 0.08 + 0.43 ms (its rate, about 4 cycles per m16n8k16 and SM); here
-// 0.08 + 0.21 ms, the same bits.
+// 0.06 + 0.20 ms, the same bits (1.03 GB per sweep: 0.15 ms at the copy rate).
 // Errors of the iterates against quad precision are those of the FP64 kernel to two
 // digits (1 to 20 sweeps; 3e-16 thermal, 8e-15 grids).
 
@@ -122,7 +122,8 @@ __global__ void __launch_bounds__(256) pack_digits_kernel(const double* __restri
   }
 }
 
-// Work item of the digits kernel: 256 ports of a tile (digits), or 32 (residual).
+// Work item of the digits kernel: 256 ports of a tile (digits), or kDgRes (residual).
+constexpr int kDgRes = 64;  // (128: 60 us a launch instead of 58)
 struct __align__(16) DgChunk {
   int32_t tile, m0, kb, pad;  // first port in the tile, first 16-input block of W's digits
 };
@@ -133,8 +134,8 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
     double* __restrict__ state, int64_t nports,
     int R, int NT, int ny, uint32_t* __restrict__ wd, int* __restrict__ wexp, BatchCtrl* __restrict__ ctrl,
     double* __restrict__ partials, const double* __restrict__ tol2, double* __restrict__ hist, int hist_len) {
-  __shared__ double rsq[32][64];
-  __shared__ double red[64];
+  __shared__ double rsq[256];
+  __shared__ int stw[16 * kDgChunk];
   __shared__ int cmax[64];
   __shared__ int s_k, s_flag;
   __shared__ bool s_last;
@@ -143,45 +144,79 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
     s_k = *((volatile int*)&ctrl->k);
     s_flag = *((volatile int*)&ctrl->flag);
   }
-  if (tid < 64) {
-    red[tid] = 0.0;
-    cmax[tid] = 0;
-  }
+  if (tid < 64) cmax[tid] = 0;
   __syncthreads();
   if (s_flag) return;
   const int k = s_k;
   const DgChunk ch = chunks[blockIdx.x];
   const int p0 = port_off[ch.tile], p = port_off[ch.tile + 1] - p0;
   const double* prev = state + (size_t)((k - 1) & 1) * nports * 2 * R;
+  // thread = (row slot, column): rows tid / R, + G, ...
+  const int G = 256 / R, g = tid / R, r = tid - g * R;
+  const size_t R2 = 2 * (size_t)R;
   if ((int)blockIdx.x >= nchunks) {
-    // residual of sweep k - 1 at the nodes whose ports start in these 32
+    // residual of sweep k - 1 at the nodes whose ports start in these kDgRes; with
+    // a = w_out(s) - w_in(t), b = w_out(t) - w_in(s) the term of batch_residual is
+    // d/2 ((a + b)/2 - (g/W) (a - b)): seven FP64 operations (their rate bounds it)
     const int ticket = blockIdx.x - nchunks, nres = gridDim.x - nchunks;
-    if (k > 1) batch_residual<double, double>(twin, kd, run, prev, p0, ch.m0, min(p, ch.m0 + 32), R, rsq, red);
-    for (int r = tid; r < R; r += 256) partials[(size_t)ticket * R + r] = k > 1 ? red[r] : 0.0;
+    double sq = 0.0;
+    if (k > 1 && g < G) {
+      const int s1 = p0 + min(p, ch.m0 + kDgRes);
+#pragma unroll 4
+      for (int s = p0 + ch.m0 + g; s < s1; s += G) {
+        const int nr = run[s];
+        double sum = 0.0;
+        for (int q = s; q < s + nr; ++q) {
+          const double* a = prev + (size_t)q * R2 + r;
+          const double* b = prev + (size_t)twin[q] * R2 + r;
+          const double wi_s = a[0], wo_s = a[R], wi_t = b[0], wo_t = b[R];
+          const double2 k2 = kd[q];
+          const double da = wo_s - wi_t, db = wo_t - wi_s;
+          sum = fma(k2.y, fma(0.5, da + db, -(k2.x * (da - db))), sum);
+        }
+        sq = fma(sum, sum, sq);
+      }
+    }
+    rsq[tid] = sq;
     __syncthreads();
-    batch_item_done(ctrl, ticket, nres, R, partials, &rsq[0][0]);
+    if (tid < R) {
+      double a = 0.0;
+      for (int i = 0; i < G; ++i) a += rsq[i * R + tid];
+      partials[(size_t)ticket * R + tid] = 0.25 * a;  // the halves of d/2
+    }
+    __syncthreads();
+    batch_item_done(ctrl, ticket, nres, R, partials, rsq);
   } else {
     const int m1 = min(p, ch.m0 + 16 * kDgChunk);
     double* cur = state + (size_t)(k & 1) * nports * 2 * R;
     // this sweep's incident waves and the largest exponent of each column
-    for (int i = tid; i < (m1 - ch.m0) * R; i += 256) {
-      const int s = p0 + ch.m0 + i / R, r = i % R;
-      const double w = k > 1 ? prev[(size_t)twin[s] * 2 * R + R + r] : 0.0;
-      cur[(size_t)s * 2 * R + r] = w;
-      if (w != 0.0) atomicMax(&cmax[r], exp_bits(w));
+    const int nrow = m1 - ch.m0;
+    for (int i = tid; i < nrow; i += 256) stw[i] = twin[p0 + ch.m0 + i];
+    __syncthreads();
+    if (g < G) {
+      int mx = 0;
+#pragma unroll 4
+      for (int i = g; i < nrow; i += G) {
+        const double w = k > 1 ? prev[(size_t)stw[i] * R2 + R + r] : 0.0;
+        cur[(size_t)(p0 + ch.m0 + i) * R2 + r] = w;
+        mx = max(mx, w != 0.0 ? exp_bits(w) : 0);
+      }
+      if (mx) atomicMax(&cmax[r], mx);
     }
     __syncthreads();
     if (tid < 64) wexp[blockIdx.x * 64 + tid] = cmax[tid] - 1022;
     // digits, a pair of rows per item, in the K-major core matrices of the B operand:
     // [16 inputs][column group of the items][digit][8 columns][input half][column][input]
     const int kbn = k > 1 ? (m1 - ch.m0 + 15) / 16 : 0, nt = NT * ny;
-    for (int i = tid; i < kbn * nt * 64; i += 256) {
-      const int w = i & 63, u = i >> 6, n = u % nt, kb = u / nt;
-      const int c = 8 * n + ((w >> 2) & 7), q = ch.m0 + 16 * kb + 8 * (w >> 5) + 2 * (w & 3);
+    const int w = tid & 63;
+#pragma unroll 2
+    for (int u = tid >> 6; u < kbn * nt; u += 4) {
+      const int n = u % nt, kb = u / nt;
+      const int c = 8 * n + ((w >> 2) & 7), i = 16 * kb + 8 * (w >> 5) + 2 * (w & 3);
       int d0[kDg], d1[kDg];
       const bool col = c < R;
-      const double v0 = col && q < p ? prev[(size_t)twin[p0 + q] * 2 * R + R + c] : 0.0;
-      const double v1 = col && q + 1 < p ? prev[(size_t)twin[p0 + q + 1] * 2 * R + R + c] : 0.0;
+      const double v0 = col && i < nrow ? prev[(size_t)stw[i] * R2 + R + c] : 0.0;
+      const double v1 = col && i + 1 < nrow ? prev[(size_t)stw[i + 1] * R2 + R + c] : 0.0;
       const int E = col ? cmax[c] - 1022 : 0;
       digits_of(v0, E, d0);
       digits_of(v1, E, d1);
@@ -197,7 +232,7 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  batch_finish(ctrl, partials, gridDim.x - nchunks, R, tol2, hist, hist_len, k, &rsq[0][0]);
+  batch_finish(ctrl, partials, gridDim.x - nchunks, R, tol2, hist, hist_len, k, rsq);
 }
 
 // Work item of the sweep: 128 outputs of a tile.
@@ -254,13 +289,30 @@ __device__ __forceinline__ void dg_ld(uint32_t addr, uint32_t nc, uint32_t (&v)[
 #undef DG_R
 }
 
+// The group sums joined: S = sum_g v_g 2^(7 (8 - g)), |v_g| <= (g + 1) 2^20.  In pairs
+// (below 2^31), then two exact halves hi 2^35 + lo (|hi| < 2^45, |lo| < 2^51) that
+// become doubles by adding them to the bits of 1.5 2^52: four FP64 operations with the
+// scaling in place of a dozen (64-bit conversions and ldexp made the joins, 13.8 k
+// cycles of the FP64 pipe per 256 inputs, longer than the products of short tiles).
+__device__ __forceinline__ double dg_join(const uint32_t (&v)[kDg]) {
+  int x[kDg];
+#pragma unroll
+  for (int g = 0; g < kDg; ++g) x[g] = __float2int_rn(__uint_as_float(v[g]));
+  const long long hi = (long long)(x[0] * 128 + x[1]) * 16384 + (x[2] * 128 + x[3]);
+  const long long lo = ((long long)(x[4] * 128 + x[5]) * 16384 + (x[6] * 128 + x[7])) * 128 + x[8];
+  constexpr double M = 6755399441055744.0;  // 1.5 2^52
+  constexpr long long MB = 0x4338000000000000ll;
+  return fma(__longlong_as_double(hi + MB) - M, 34359738368.0, __longlong_as_double(lo + MB) - M);
+}
+
 __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
     const DgItem* __restrict__ items, int nitems, int NT, int ny, const int32_t* __restrict__ port_off,
     const unsigned char* __restrict__ Td, const int* __restrict__ texp, const unsigned char* __restrict__ wd,
     const int* __restrict__ wexp, const double* __restrict__ c, double* __restrict__ state, int64_t nports, int R,
     BatchCtrl* __restrict__ ctrl) {
   extern __shared__ __align__(1024) unsigned char dsm[];
-  __shared__ uint64_t full[kDgStages], empty[kDgStages], tfull[2], tempty[2], drain;
+  __shared__ uint64_t full[kDgStages], empty[kDgStages], tfull[2], tempty[2], ufull[2], uempty[2], drain;
+  __shared__ volatile int s_unit[2];
   __shared__ uint32_t s_tmem;
   __shared__ int s_k, s_flag;
   __shared__ volatile int s_abort;
@@ -276,13 +328,15 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], 8);
+      mbar_init(&ufull[i], 1);
+      mbar_init(&uempty[i], 9);
     }
     mbar_init(&drain, 1);
     fence_mbar_init();
   }
   __syncthreads();
   if (s_flag) return;
-  const int k = s_k, G = gridDim.x, total = nitems * ny;
+  const int k = s_k, total = nitems * ny;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                  "r"(2 * kDgTmem)
@@ -304,14 +358,21 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
     s_abort = 1;
     return false;
   };
-  // the items by falling cost, the CTAs forth and back
-  auto item_at = [&](int r) { return r * G + ((r & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x); };
   uint32_t issued = 0;
   if (warp == 0) {
-    if (lane == 0 && k > 1) {
+    // units (an item and a column group, the largest first) from a counter: the SMs' shares
+    // of the bandwidth differ, equal shares of the bytes leave the slowest 1.3 times the mean
+    if (lane == 0) {
       uint32_t g = 0;
-      for (int r = 0, idx; (idx = item_at(r)), r * G < total; ++r) {
-        if (idx >= total) continue;
+      int next = (int)atomicAdd(&ctrl->work, 1u);
+      for (uint32_t u = 0;; ++u) {
+        const int idx = next < total ? next : -1;
+        if (u >= 2 && !wait(&uempty[u & 1], ((u >> 1) - 1) & 1)) break;
+        s_unit[u & 1] = idx;
+        mbar_arrive(&ufull[u & 1]);
+        if (idx < 0) break;
+        next = (int)atomicAdd(&ctrl->work, 1u);
+        if (k == 1) continue;
         const DgItem it = items[idx / ny];
         const int y = idx % ny, p = port_off[it.tile + 1] - port_off[it.tile], nb = (p + 15) / 16;
         const uint32_t dig = dg_groups(p, it.m) * 256;  // bytes of a digit's rows
@@ -336,10 +397,14 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && k > 1) {
+    if (lane == 0) {
       uint32_t g = 0, ch = 0;
-      for (int r = 0, idx; (idx = item_at(r)), r * G < total; ++r) {
-        if (idx >= total) continue;
+      for (uint32_t u = 0;; ++u) {
+        if (!wait(&ufull[u & 1], (u >> 1) & 1)) break;
+        const int idx = s_unit[u & 1];
+        mbar_arrive(&uempty[u & 1]);
+        if (idx < 0) break;
+        if (k == 1) continue;
         const int tile = items[idx / ny].tile, nb = (port_off[tile + 1] - port_off[tile] + 15) / 16;
         for (int kb = 0; kb < nb; ++kb, ++g) {
           const uint32_t st = g % kDgStages, buf = ch & 1;
@@ -365,8 +430,12 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
     const int quarter = warp & 3, h = (warp - 2) >> 2, nq = 2 * NT;
     uint32_t ch = 0;
     double* cur = state + (size_t)(k & 1) * nports * 2 * R;
-    for (int r = 0, idx; (idx = item_at(r)), r * G < total; ++r) {
-      if (idx >= total) continue;
+    for (uint32_t unit = 0;; ++unit) {
+      if (!__all_sync(0xffffffffu, wait(&ufull[unit & 1], (unit >> 1) & 1))) break;  // (the warp together)
+      const int idx = s_unit[unit & 1];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&uempty[unit & 1]);
+      if (idx < 0) break;
       const DgItem it = items[idx / ny];
       const int c0 = (idx % ny) * (int)nc, p0 = port_off[it.tile], p = port_off[it.tile + 1] - p0, nb = (p + 15) / 16;
       const int s = 128 * it.m + 32 * quarter + lane;
@@ -379,6 +448,7 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
         const int nch = (nb + kDgChunk - 1) / kDgChunk;
         for (int j = 0; j < nch; ++j, ++ch) {
           const uint32_t buf = ch & 1;
+          const int wx = lane < (int)nc && c0 + lane < R ? wexp[(it.chunk + j) * 64 + c0 + lane] : 0;
           if (!__all_sync(0xffffffffu, wait(&tfull[buf], (ch >> 1) & 1))) break;  // (the warp together)
           tc_fence_after();
 #pragma unroll
@@ -387,19 +457,16 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
             if (q >= nq) break;
             uint32_t v[kDg][4];
             dg_ld(tmem + ((uint32_t)(32 * quarter) << 16) + buf * kDgTmem + 4 * q, nc, v);
-            // the groups joined: S = sum_g v_g 2^(7 (8 - g)), exact in two 64-bit halves,
-            // scaled by the chunk's column exponent
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              const int col = c0 + 4 * q + e;
-              if (col >= R) break;
-              long long hi = 0, lo = 0;
+              if (c0 + 4 * q + e >= R) break;
+              const int we = __shfl_sync(0xffffffffu, wx, 4 * q + e);
+              uint32_t x[kDg];
 #pragma unroll
-              for (int g = 0; g < 4; ++g) hi = hi * 128 + __float2int_rn(__uint_as_float(v[g][e]));
-#pragma unroll
-              for (int g = 4; g < kDg; ++g) lo = lo * 128 + __float2int_rn(__uint_as_float(v[g][e]));
-              const double S = fma((double)hi, 34359738368.0, (double)lo);  // hi 2^35 + lo
-              out[u][e] += ldexp(S, wexp[(it.chunk + j) * 64 + col]);
+              for (int g = 0; g < kDg; ++g) x[g] = v[g][e];
+              const double S = dg_join(x);
+              if (we > -960 && we < 960) out[u][e] = fma(S, __longlong_as_double((long long)(we + 1023) << 52), out[u][e]);
+              else out[u][e] += ldexp(S, we);
             }
           }
           tc_fence_before();
