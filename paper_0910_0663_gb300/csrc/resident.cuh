@@ -532,14 +532,15 @@ __global__ void __launch_bounds__(32 * (res_warps(std::is_same<TT, double>::valu
         ap.flush(bj, lane, acc);
       }
       group_sync();
-      // outputs: c, then the tile's warps in order
+      // outputs: the tile's warps in order, then c (FP32: c first)
       for (int s = lane + 32 * part; s < p; s += 32 * wpt) {
         const AC* a = acc_all + (size_t)(slot * wpt) * pp + s;
         if constexpr (DF) {
           const float2 c0 = __ldg(reinterpret_cast<const float2*>(A.c) + p0 + s);
-          dacc o = {c0.x, c0.y};
+          dacc o = a[0];
 #pragma unroll 4
-          for (int w = 0; w < wpt; ++w) o = dacc_add(o, a[(size_t)w * pp]);
+          for (int w = 1; w < wpt; ++w) o = dacc_add(o, a[(size_t)w * pp]);
+          o = dacc_add(dacc{c0.x, c0.y}, o);  // c last: its low part would round every sum before it
           const df v = dacc_value(o), wi = wv.get(s);
           wo[s] = v;
           cur[p0 + s] = make_float4(wi.h, wi.l, v.h, v.l);
@@ -696,7 +697,7 @@ __global__ void __launch_bounds__(32 * (kSmallRows + kSmallSide + 1), 1) sweep_s
       else asm volatile("bar.sync %0, %1;" ::"r"(1 + tile), "r"(32 * rpt) : "memory");
       const float4* Tr = Ts + (size_t)tile * nstep * pr + row;
       if constexpr (DF) {
-        dacc2 a = {make_float2(c0.x, 0.f), make_float2(c0.y, 0.f)}, b = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        dacc2 a = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, b = a;
 #pragma unroll 2
         for (int i = 0; i < nst; i += 2) {
           const float4 t0 = Tr[(size_t)i * pr], w0 = wt[i];
@@ -706,7 +707,9 @@ __global__ void __launch_bounds__(32 * (kSmallRows + kSmallSide + 1), 1) sweep_s
           const float2 h1 = make_float2(w1.x, w1.y);
           dacc2_fma(b, make_float2(t1.x, t1.y), make_float2(t1.z, t1.w), h1, f2neg(h1), make_float2(w1.z, w1.w));
         }
-        const df o = dacc_value(dacc_add(dacc_add(dacc2_lo(a), dacc2_hi(a)), dacc_add(dacc2_lo(b), dacc2_hi(b))));
+        // c last: in a chain's E its low part would cost a rounding at 2^-48 |c| per step
+        const dacc t = dacc_add(dacc_add(dacc2_lo(a), dacc2_hi(a)), dacc_add(dacc2_lo(b), dacc2_hi(b)));
+        const df o = dacc_value(dacc_add(dacc{c0.x, c0.y}, t));
         if (port >= 0) st[(size_t)(k % kResSlots) * np + port] = make_float4(wi.h, wi.l, o.h, o.l);
       } else {
         float2 a = make_float2(c0.x, 0.f), b = make_float2(0.f, 0.f);
