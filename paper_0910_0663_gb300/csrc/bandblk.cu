@@ -329,7 +329,7 @@ static void launch_blk_t(vtm_plan_s* P, FT* v, const FT* Lc, const FT* Uc, const
   const int per_sm = (P->nparts * (multi ? (ncols + 3) / 4 : ncols) + sms - 1) / sms;
   const size_t smem = std::max(S * bytes, per_sm <= 3 ? (size_t)(224 / (per_sm + 1) + 1) * 1024 : 0);
   auto go = [&](auto* kern, int nc) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kern, smem);
     kern<<<P->nparts * ((ncols + nc - 1) / nc), 32 * NW, smem, s>>>(
         P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(), P->tabs.band_off.as<int64_t>(),
         P->d_bb_off.as<int32_t>(), P->d_bb_order.as<int32_t>(), Lc, Uc, Li, Ui, v, stride, P->nparts, ncols, stage, S);

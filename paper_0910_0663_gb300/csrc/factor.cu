@@ -347,7 +347,7 @@ vtm_status factor_tiles(vtm_plan_s* P) {
   if (panel <= 222 * 1024) {
     const int threads = P->max_bw <= 48 ? 128 : 256;
     auto go = [&](auto* kern) {
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel);
+      allow_smem(kern, panel);
       kern<<<P->nparts, threads, panel, s>>>(P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(),
                                              P->tabs.band_off.as<int64_t>(), P->d_Lc.as<double>(),
                                              P->d_Uc.as<double>(), P->d_err.as<int>());

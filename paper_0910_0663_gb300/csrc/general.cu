@@ -485,9 +485,7 @@ static vtm_status plan_general_resident(vtm_plan_s* P) {
   const int nslots = (int)((optin - (int64_t)fa.sharedSizeBytes - fixed) / (kGenThreads * 16));
   if (nslots < kGenMinSlots) return VTM_OK;
   P->gen_smem = fixed + (int64_t)nslots * kGenThreads * 16;
-  // the same limit for every plan: another thread's plan never lowers it
-  VTM_CUDA_TRY(cudaFuncSetAttribute(general_resident_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    optin - (int)fa.sharedSizeBytes));
+  VTM_CUDA_TRY(allow_smem(general_resident_kernel, (size_t)P->gen_smem));
   VTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, general_resident_kernel, kGenThreads + 32,
                                                              (size_t)P->gen_smem));
   if (fits < 1) return VTM_OK;

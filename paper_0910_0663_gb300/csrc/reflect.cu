@@ -256,7 +256,7 @@ vtm_status build_reflections_blk(vtm_plan_s* P) {
     P->refl_items = (int)items.size();
   }
   const size_t smem = rf_smem(P->max_bw);
-  VTM_CUDA_TRY(cudaFuncSetAttribute(build_reflection_blk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  VTM_CUDA_TRY(allow_smem(build_reflection_blk_kernel, smem));
   int sms = 152, per_sm = 1;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device);
   VTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_reflection_blk_kernel, kRfThreads, smem));

@@ -2652,7 +2652,7 @@ template <class TT, class WT, int VEC>
 static void launch_slab(vtm_plan_s* P, const TT* T, const WT* c, WT* state, double* hist, int hist_len) {
   static_assert(256 * VEC * sizeof(WT) <= kSlabStages * 256 * 16, "the partial sums reuse the ring");
   const size_t smem = kSlabStages * 256 * 16 + (size_t)P->max_ports * sizeof(WT) + 16;
-  cudaFuncSetAttribute(sweep_slab_kernel<TT, WT, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(sweep_slab_kernel<TT, WT, VEC>, smem);
   launch_packed(P, sweep_slab_kernel<TT, WT, VEC>, P->nslabs, 256, smem, P->stream, T,
                 (const SlabItem*)P->d_slabs.as<SlabItem>(), P->slab_width / VEC,
                 (const int32_t*)P->d_twin.as<int32_t>(), kd_of<WT>(P), (const uint8_t*)P->d_run.as<uint8_t>(), c, state,
@@ -2895,7 +2895,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, P->device);
     with_res([&](auto* kern) {
       res_ok = coop &&
-               cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem) == cudaSuccess &&
+               allow_smem(kern, res_smem) == cudaSuccess &&
                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, res_threads, res_smem) ==
                    cudaSuccess &&
                per_sm >= 1;

@@ -354,6 +354,21 @@ namespace vtm {
 
 vtm_status dev_alloc(DevBuf& b, size_t bytes);
 void dev_free(DevBuf& b);
+// Raises a kernel's limit of dynamic shared memory to the device's, never lowers it:
+// another thread's plan with less of it cannot take the limit away between this call
+// and the launch.
+template <class K>
+inline cudaError_t allow_smem(K* kern, size_t bytes) {
+  cudaFuncAttributes fa{};
+  const cudaError_t e = cudaFuncGetAttributes(&fa, (const void*)kern);
+  if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= bytes) return e;
+  int dev = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              optin - (int)fa.sharedSizeBytes);
+}
+
 template <class T>
 vtm_status upload(DevBuf& b, const std::vector<T>& h, cudaStream_t s) {
   VTM_TRY(dev_alloc(b, h.size() * sizeof(T) > 0 ? h.size() * sizeof(T) : 16));
