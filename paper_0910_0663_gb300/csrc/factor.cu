@@ -267,13 +267,14 @@ __global__ void __launch_bounds__(256, 2) band_factor_panel_kernel(
         if (q < nc && q <= r && r - q <= bw) uc[(size_t)(j0 + r) * B + r - q] = q == r ? 1.0 : l_at(r, q);
       }
     __syncthreads();  // the panel's slots are free
+    // columns j0 + C .. take them: also where no row lies below the panel (half bandwidth 0)
+    const int cin = min(N, n - (j0 + C));
+    for (int e = tid; e < cin * B; e += nt) {
+      const int q = e / B, a = e - q * B;
+      cp_async8(Lw + slot(q) + a, lc + (size_t)(j0 + C + q) * B + a);
+      if (kLU) cp_async8(Uw + slot(q) + a, uc + (size_t)(j0 + C + q) * B + a);
+    }
     if (M > 0) {
-      const int cin = min(N, n - (j0 + C));  // columns j0 + C .. take the panel's slots
-      for (int e = tid; e < cin * B; e += nt) {
-        const int q = e / B, a = e - q * B;
-        cp_async8(Lw + slot(q) + a, lc + (size_t)(j0 + C + q) * B + a);
-        if (kLU) cp_async8(Uw + slot(q) + a, uc + (size_t)(j0 + C + q) * B + a);
-      }
       // trailing window, rows and columns N .. R - 1, in 4 x 4 tiles
       const int T = (M + 3) / 4, ntile = kLU ? T * T : T * (T + 1) / 2;
       for (int e = tid; e < ntile; e += nt) {
@@ -319,9 +320,9 @@ __global__ void __launch_bounds__(256, 2) band_factor_panel_kernel(
           }
         }
       }
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      __syncthreads();
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
   }
   if (s_bad && tid == 0) atomicMax(err, t + 1);
 }
