@@ -603,7 +603,9 @@ __global__ void __launch_bounds__(32 * (kSmallRows + kSmallSide + 1), 1) sweep_s
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int B = kSymB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_flag;
+  // the decision of sweep k in word (k + 1) & 1, read behind barrier k + 1: every warp leaves at
+  // the same sweep (one word could be read late, with the decision that this sweep has just made)
+  __shared__ int s_flag[2];
   __shared__ double s_part[2][kSmallSide];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthreads = blockDim.x;
   const int pr = A.pp;           // rows and columns of a tile: a multiple of 32
@@ -656,7 +658,7 @@ __global__ void __launch_bounds__(32 * (kSmallRows + kSmallSide + 1), 1) sweep_s
     kds[s] = reinterpret_cast<const KD*>(A.kd)[s];
   }
   for (int i = tid; i < A.nparts * nstep; i += nthreads) ws[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (tid == 0) s_flag = 0;
+  if (tid < 2) s_flag[tid] = 0;
   if (tid < 2 * kSmallSide) s_part[0][tid] = 0.0;
   // row warps: tile, row, port
   const int tile = warp / rpt, row = 32 * (warp % rpt) + lane;
@@ -676,7 +678,7 @@ __global__ void __launch_bounds__(32 * (kSmallRows + kSmallSide + 1), 1) sweep_s
   dec.load(A.ctrl);
   for (int k = 1;; ++k) {
     __syncthreads();  // the waves of sweep k - 1 and the flag
-    if (*((volatile int*)&s_flag)) break;
+    if (*((volatile int*)&s_flag[k & 1])) break;
     const PAIR* prev = st + (size_t)((k - 1) % kResSlots) * np;
     if (warp < nrow) {
       float4* wt = ws + (size_t)tile * nstep;
@@ -777,7 +779,7 @@ __global__ void __launch_bounds__(32 * (kSmallRows + kSmallSide + 1), 1) sweep_s
       const int f = dec.close(k - 1, t, A.hist, A.hist_len);
       if (f) {
         dec.store(A.ctrl, k - 1, f);
-        *((volatile int*)&s_flag) = f;
+        *((volatile int*)&s_flag[(k + 1) & 1]) = f;
       }
     }
   }

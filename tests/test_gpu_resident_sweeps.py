@@ -77,3 +77,19 @@ def test_a_barrier_that_runs_out_is_reported_and_the_plan_recovers():
     plan.set_options(wait_polls=0)
     x2, _ = plan.solve(b)
     assert torch.equal(x, x2)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_one_sm_with_several_warps_per_tile_ends_every_warp_at_one_sweep(precision):
+    """Tiles of 33..64 ports take two warps each, which meet at a barrier of their own
+    in every sweep; the runs end by tolerance and by the sweep limit, at odd and even
+    sweeps, with the same bits each time."""
+    w, plan = _plan(ONE[2], precision)
+    b = torch.from_numpy(w.b[0]).cuda()
+    for limit in (1, 2, 3, 4, 17, 18, 200000):
+        plan.set_options(max_sweeps=limit)
+        x, info = plan.solve(b, check=False)
+        assert info["sweeps"] == limit or info["relres"] <= 1e-10
+        for _ in range(20):
+            y, again = plan.solve(b, check=False)
+            assert torch.equal(x, y) and again["sweeps"] == info["sweeps"]
