@@ -2697,9 +2697,11 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
       cudaGraphExec_t gexec = nullptr, gsmall = nullptr;
       if (P->stream && P->opts.graphs != 1) {
         SweepGraph& G = P->batch_graph[prec];
-        const uint64_t key = ((uint64_t)kv << 56) ^ ((uint64_t)nb << 32) ^ ((uint64_t)R << 8) ^
-                             (uint64_t)(uintptr_t)P->d_bstate.p ^ ((uint64_t)(uintptr_t)bhist << 3) ^
-                             ((uint64_t)bhist_len << 40);
+        const uint64_t key =
+            graph_key({(uint64_t)kv, (uint64_t)nb, (uint64_t)R, key_of(bhist), (uint64_t)bhist_len,
+                       key_of(P->d_bstate.p), key_of(P->d_bc.p), key_of(P->d_bpart.p), key_of(P->d_bctrl.p),
+                       key_of(P->d_btol2.p), key_of(P->d_Ttc.p), key_of(P->d_dg_T.p), key_of(P->d_dg_w.p),
+                       key_of(P->d_dg_wexp.p)});
         if (!G.exec || G.key != key) {
           G.reset();
           for (int g = 0; g < 2; ++g) {

@@ -2904,7 +2904,6 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   }
   if (res_ok) {
     VTM_TRY(dev_alloc(P->d_res, 64 + 2 * (size_t)res_grid * sizeof(double)));
-    if (prec != VTM_PREC_FP64) VTM_TRY(dev_alloc(P->d_fstate32, 2 * kResSlots * (size_t)std::max<int64_t>(npt, 1) * sizeof(float)));
   }
   if (wdf_ok || (res_ok && prec == VTM_PREC_FP64)) {
     VTM_TRY(dev_alloc(P->d_dfstate, kResSlots * (size_t)std::max<int64_t>(npt, 1) * sizeof(float4)));
@@ -2924,7 +2923,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
     ra.kd = prec == VTM_PREC_FP64 ? P->d_kddf.p : P->d_kd32.p;
     ra.run = P->d_run.as<uint8_t>();
     ra.c = prec == VTM_PREC_FP64 ? P->d_cdf.p : P->d_c32.p;
-    ra.state3 = prec == VTM_PREC_FP64 ? P->d_dfstate.p : P->d_fstate32.p;
+    ra.state3 = P->d_dfstate.p;  // (FP32 and 16 bits: below)
     ra.nports = npt;
     ra.ctrl = P->d_ctrl.as<SweepCtrl>();
     ra.bar = reinterpret_cast<unsigned long long*>(P->d_res.p);
@@ -3164,8 +3163,12 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
     VTM_TRY(dev_alloc(P->d_flow, kFlowBytes));
     VTM_TRY(dev_alloc(P->d_part4, 16 * (size_t)P->nparts * sizeof(double)));
   }
-  // three wave slots: the dataflow kernels and the one-warp-per-tile sweeps
-  if (sym_ok) VTM_TRY(dev_alloc(P->d_fstate32, 6 * (size_t)std::max<int64_t>(npt, 1) * sizeof(float)));
+  // wave slots of the packed kernels: three, kernel 13 four (always four: a later solve of
+  // the plan may take another kernel, and captured launches hold the address)
+  if (sym_ok) {
+    VTM_TRY(dev_alloc(P->d_fstate32, 2 * kResSlots * (size_t)std::max<int64_t>(npt, 1) * sizeof(float)));
+    ra.state3 = P->d_fstate32.p;
+  }
   // one cooperative launch runs sweeps 1.. until a flag (k_max in ctrl)
   auto launch_flow = [&]() -> cudaError_t {
     cudaMemsetAsync(P->d_done.p, 0, (size_t)P->nparts * sizeof(int), s);
@@ -3391,8 +3394,10 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   cudaGraphExec_t gexec = nullptr, gsmall = nullptr;
   if (P->stream && P->opts.graphs != 1) {
     SweepGraph& G = P->sweep_graph[prec];
-    const uint64_t key = ((uint64_t)kern << 56) ^ ((uint64_t)(P->opts.pdl == 1) << 52) ^
-                         ((uint64_t)batch << 32) ^ (uint64_t)(uintptr_t)hist ^ ((uint64_t)hist_len << 16);
+    const uint64_t key =
+        graph_key({(uint64_t)kern, (uint64_t)(P->opts.pdl == 1), (uint64_t)batch, key_of(hist), (uint64_t)hist_len,
+                   key_of(P->d_state32.p), key_of(P->d_state64.p), key_of(P->d_fstate32.p), key_of(P->d_dfstate.p),
+                   key_of(P->d_c32.p), key_of(P->d_c64.p), key_of(P->d_cdf.p), key_of(P->d_slab_part.p)});
     if (!G.exec || G.key != key) {
       G.reset();
       for (int g = 0; g < 2; ++g) {

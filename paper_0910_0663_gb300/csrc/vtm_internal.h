@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -132,9 +133,10 @@ struct TileTables {
 }  // namespace vtm
 
 namespace vtm {
-// A captured batch of sweep launches (CUDA graph) and what it was made for.
-// Captured sweep launches: `exec` replays check_every launches, `small` a
-// quarter of that (the tail up to a hinted sweep count)
+// Captured sweep launches (CUDA graphs): `exec` replays check_every launches, `small`
+// a quarter of that (the tail up to a hinted sweep count).  `key` is what they were
+// captured for: the options and the address of every buffer that a solve may allocate
+// again (the operators are not among them: a factorisation drops the graphs)
 struct SweepGraph {
   cudaGraphExec_t exec = nullptr;
   cudaGraphExec_t small = nullptr;
@@ -146,6 +148,13 @@ struct SweepGraph {
     key = 0;
   }
 };
+inline uint64_t graph_key(std::initializer_list<uint64_t> what) {  // FNV-1a over the words' bytes
+  uint64_t h = 14695981039346656037ull;
+  for (uint64_t w : what)
+    for (int i = 0; i < 8; ++i) h = (h ^ (w >> 8 * i & 255)) * 1099511628211ull;
+  return h ? h : 1;
+}
+inline uint64_t key_of(const void* p) { return (uint64_t)(uintptr_t)p; }
 }  // namespace vtm
 
 struct vtm_plan_s {

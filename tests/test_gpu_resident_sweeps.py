@@ -93,3 +93,22 @@ def test_one_sm_with_several_warps_per_tile_ends_every_warp_at_one_sweep(precisi
         for _ in range(20):
             y, again = plan.solve(b, check=False)
             assert torch.equal(x, y) and again["sweeps"] == info["sweeps"]
+
+
+@pytest.mark.parametrize("forced", [9, 11])
+def test_captured_sweeps_do_not_outlive_their_buffers(forced):
+    """A plan with a stream of its own captures its sweeps; a later solve that may take
+    the resident form must leave the captured launches a buffer that still exists."""
+    from paper_0910_0663_gb300 import vtm
+    w = wl.grid2d(240, 240, 12, 12, ground=0.05, seed=7)
+    A = w.csr()
+    b = torch.from_numpy(w.b[0]).cuda()
+    plan = vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts, precision="fp16", stream=torch.cuda.Stream(),
+                    sweep_kernel=forced)
+    x, _ = plan.solve(b)
+    for kernel in (0, forced, 0, 5, forced):
+        plan.set_options(sweep_kernel=kernel)
+        y, info = plan.solve(b)
+        assert O.residual_norms(A, y.cpu().numpy()[None], w.b[:1]).max() <= 1e-10
+        if kernel == forced:
+            assert torch.equal(x, y)
