@@ -3268,18 +3268,29 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   int kern = (vecload || symload) ? choice : (staged ? 2 : 1);
   if (P->opts.method == VTM_METHOD_ASYNC) kern = wflow_ok ? 10 : 8;  // its own iteration: not autotuned
   else if (P->opts.sweep_kernel == 0) {
-    if (P->tuned_kernel[prec] == 0) {
-      const bool can_st = nv_max <= 4 * 256 && st_smem <= 200 * 1024;
-      const bool can_vec = nv_max <= 256;
-      const bool can_vec128 = nv_max <= 128;
+    // the candidates of this solve: what the sweep limit, the precisions' copies and the
+    // device allow.  A choice made among others is made again
+    const bool can[14] = {false,
+                          true,
+                          nv_max <= 4 * 256 && st_smem <= 200 * 1024,
+                          nv_max <= 256,
+                          nv_max <= 128,
+                          sym_ok,
+                          sym_ok,
+                          symb_ok,
+                          flow_ok,
+                          sym_ok,
+                          wflow_ok,
+                          wmma_ok,
+                          wdf_ok,
+                          res_ok};
+    int mask = 0;
+    for (int cand = 1; cand <= 13; ++cand) mask |= (int)can[cand] << cand;
+    if (P->tuned_kernel[prec] == 0 || P->tuned_among[prec] != mask) {
       float best = 1e30f;
       int best_k = 1;
       for (int cand = 1; cand <= 13; ++cand) {
-        if ((cand == 2 && !can_st) || (cand == 3 && !can_vec) || (cand == 4 && !can_vec128) ||
-            ((cand == 5 || cand == 6 || cand == 9) && !sym_ok) || (cand == 7 && !symb_ok) ||
-            (cand == 8 && !flow_ok) || (cand == 10 && !wflow_ok) || (cand == 11 && !wmma_ok) ||
-            (cand == 12 && !wdf_ok) || (cand == 13 && !res_ok))
-          continue;
+        if (!can[cand]) continue;
         if (cand == 8 || cand == 10 || cand == 13) {  // one launch, per-sweep time against the others' 6
           SweepCtrl t = h;
           // (kernel 13 fills shared memory first: more sweeps to set against that)
@@ -3331,6 +3342,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
         }
       }
       P->tuned_kernel[prec] = best_k;
+      P->tuned_among[prec] = mask;
       P->tuned_ms[prec] = best / 6.0f;
       // back to the initial state of this inner solve
       if (hist) VTM_CUDA_TRY(cudaMemsetAsync(hist, 0, hist_len * sizeof(double), s));

@@ -280,6 +280,7 @@ struct vtm_plan_s {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, evs0 = nullptr, evs1 = nullptr;
   // sweep-kernel autotuning and graphs, per precision
   int tuned_kernel[4] = {0, 0, 0, 0};
+  int tuned_among[4] = {0, 0, 0, 0};  // the candidates it was chosen among (bit = kernel)
   int dataflow_kernel = 8;  // kernel of the last sweeps run (8 or 10 for asynchronous VTM)
   float tuned_ms[4] = {0.f, 0.f, 0.f, 0.f};
   int sweep_hint[4][8] = {};  // sweeps of refinement step i of the last solve, per precision

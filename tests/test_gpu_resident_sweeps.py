@@ -112,3 +112,33 @@ def test_captured_sweeps_do_not_outlive_their_buffers(forced):
         assert O.residual_norms(A, y.cpu().numpy()[None], w.b[:1]).max() <= 1e-10
         if kernel == forced:
             assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
+def test_the_choice_follows_what_a_later_solve_allows(precision):
+    """The kernel chosen by an earlier solve may not serve a later one: a sweep limit
+    that the grid barrier cannot count to, or an FP64 plan that went to FP32 and back
+    (its hi + lo copy is gone)."""
+    from paper_0910_0663_gb300 import vtm
+    w, plan = _plan(GRID[1], precision)
+    A = w.csr()
+    b = torch.from_numpy(w.b[0]).cuda()
+
+    def solves(**opts):
+        plan.set_options(**opts)
+        x, info = plan.solve(b)
+        assert O.residual_norms(A, x.cpu().numpy()[None], w.b[:1]).max() <= 1e-10
+        return x
+
+    x = solves()
+    solves(max_sweeps=1 << 30)
+    solves(max_sweeps=200000)
+    if precision == "fp64":
+        plan.set_options(precision="fp32")
+        with pytest.raises(vtm.VTMError):
+            plan.solve(b)  # not factored for FP32
+        plan.factor()
+        solves()
+        solves(precision="fp64")
+        plan.factor()
+        solves()
