@@ -2724,7 +2724,7 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
       const int step = std::min(outer, 7);
       const int hint = P->batch_hint[prec][step];
       int reps = 1, sreps = 0;
-      const int need = hint > 0 ? std::min(hint + 1, sweeps_left + 1) : 0;  // launch k decides sweep k - 1
+      const int need = hint > 0 ? std::min(hint, sweeps_left) + 1 : 0;  // launch k decides sweep k - 1
       if (gexec && need > 0) {
         reps = std::min(need / nb, 64);
         sreps = gsmall ? (need - reps * nb + snb - 1) / snb : 0;
@@ -2736,7 +2736,7 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
       int launched = 0;
       BatchCtrl hc{};
       while (true) {
-        const int m = gexec ? nb : std::min(first > 0 ? first : nb, sweeps_left + 1 - launched);
+        const int m = gexec ? nb : (int)std::min<int64_t>(first > 0 ? first : nb, (int64_t)sweeps_left + 1 - launched);
         first = 0;
         VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
         if (gexec) {

@@ -604,7 +604,10 @@ vtm_status general_sweeps(vtm_plan_s* P, double bnorm2, double target2, int budg
   VTM_CUDA_TRY(cudaMemsetAsync(P->d_gin.p, 0, 2 * std::max<int64_t>(P->n_in, 1) * sizeof(double), s));
   VTM_CUDA_TRY(cudaMemsetAsync(P->d_gout.p, 0, kGenSlots * std::max<int64_t>(P->n_out, 1) * sizeof(double), s));
   if (P->gen_ctas == 0) VTM_TRY(plan_general_resident(P));
-  if (P->gen_ctas > 0) return general_sweeps_resident(P, budget, hist, hist_len, sweep_out, flag_out);
+  // (the barrier word holds as many arrivals and sweeps as res_counts allows; above that one
+  // launch per sweep)
+  if (P->gen_ctas > 0 && res_counts(budget, P->gen_ctas))
+    return general_sweeps_resident(P, budget, hist, hist_len, sweep_out, flag_out);
   // four groups of up to 256 threads per tile (one output each; eight groups
   // of 128 measured slower on the 1024^2 VCCS grid)
   constexpr int KS = 4;
@@ -616,7 +619,7 @@ vtm_status general_sweeps(vtm_plan_s* P, double bnorm2, double target2, int budg
                                       (int)smem));
   int launched = 0;
   while (true) {
-    const int m = std::min(P->opts.check_every, budget + 1 - launched);
+    const int m = (int)std::min<int64_t>(P->opts.check_every, (int64_t)budget + 1 - launched);
     VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
     for (int i = 0; i < m; ++i)
       general_sweep_kernel<KS><<<P->nparts, threads, smem, s>>>(

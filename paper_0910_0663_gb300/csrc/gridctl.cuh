@@ -15,6 +15,10 @@
 
 namespace vtm {
 
+// What the word can count: 32 bits of arrivals (half of them used, so that no carry
+// reaches the decision), 28 bits of sweep number.
+inline bool res_counts(int budget, int ctas) { return (int64_t)budget * ctas < (1ll << 31) && budget < (1 << 27); }
+
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");

@@ -2869,7 +2869,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
         const int warps = ra.tpc * ra.wpt;
         const size_t b = prec == VTM_PREC_FP64 ? res_base_bytes<double>(pp_max, ra.tpc, warps)
                                                : res_base_bytes<float>(pp_max, ra.tpc, warps);
-        if (b <= kMax && pp_max <= 128 * ra.wpt && (int64_t)budget * res_grid < (1ll << 31) && budget < (1 << 27)) {
+        if (b <= kMax && pp_max <= 128 * ra.wpt && res_counts(budget, res_grid)) {
           ra.nres = std::min((nblk_max + ra.wpt - 1) / ra.wpt, (int)((kMax - b) / ((size_t)warps * blk)));
           res_smem = b + (size_t)warps * ra.nres * blk;
           res_threads = 32 * (warps + 1);
@@ -3439,7 +3439,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   int launched = 0;
   int reps = 1, sreps = 0;
   const int lag = (kern == 9 || kern == 11) ? 2 : 1;  // launches past the hinted sweep
-  const int need = hint > 0 ? std::min(hint + lag, budget + lag) : 0;
+  const int need = hint > 0 ? std::min(hint, budget) + lag : 0;
   if (gexec && need > 0) {
     reps = std::min(need / batch, 64);
     sreps = gsmall ? (need - reps * batch + sbatch - 1) / sbatch : 0;
@@ -3449,7 +3449,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   // without graphs the first round is the hinted count of single launches
   int first = need;
   while (true) {
-    const int m = gexec ? batch : std::min(first > 0 ? first : batch, budget + 1 - launched);
+    const int m = gexec ? batch : (int)std::min<int64_t>(first > 0 ? first : batch, (int64_t)budget + 1 - launched);
     first = 0;
     VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
     if (gexec) {

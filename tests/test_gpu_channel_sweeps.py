@@ -70,3 +70,19 @@ def test_returned_iterate_is_the_sweep_asked_for(vtm, n, tile, sweeps):
     assert info["sweeps"] == k
     r = O.residual_norms(A, x.cpu().numpy().reshape(w.b.shape), w.b).max()
     assert abs(r - h[k - 1]) <= 1e-12 + 1e-9 * r
+
+
+@pytest.mark.parametrize("limit", [1 << 30, (1 << 31) - 1])
+def test_a_sweep_limit_above_what_the_barrier_counts(vtm, limit):
+    """Up to 2^31 arrivals of all CTAs together run in one launch, more take a launch
+    per sweep."""
+    w = wl.vccs_grid(200, 200, 50, 50, seed=12)
+    plan = vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts, Zc=1.0)
+    b = torch.from_numpy(w.b).cuda()
+    x, info = plan.solve(b, tol=1e-9)
+    assert info["kernel_launches"] < info["sweeps"]
+    plan.set_options(max_sweeps=limit)
+    y, many = plan.solve(b, tol=1e-9)
+    assert many["kernel_launches"] > many["sweeps"]
+    assert abs(many["sweeps"] - info["sweeps"]) <= 1  # (sums in another order)
+    assert O.residual_norms(w.csr(), y.cpu().numpy().reshape(w.b.shape), w.b).max() <= 1e-9
