@@ -916,16 +916,17 @@ __global__ void __launch_bounds__(256, 3) sweep_slab_kernel(
   WP* cur = reinterpret_cast<WP*>(state) + (size_t)(k & 1) * nports;
   // incident waves of the tile (delay 1): the twins' outgoing waves
   for (int s = tid; s < p; s += 256) w_in[s] = k > 1 ? prev[twin[p0 + s]].y : (WT)0;
-  // residual of sweep k - 1 at the nodes whose ports start in this slab
-  WT sq = 0;
+  // residual of sweep k - 1 at the nodes whose ports start in this slab, summed and
+  // squared in FP64: the square of an FP32 residual below 1e-22 or above 1e19 is none
+  double sq = 0.0;
   if (k > 1) {
     for (int s = it.m0 + tid; s < min(p, it.m0 + SW); s += 256) {
       const int nr = run[p0 + s];
       if (nr) {
-        WT r = 0;
+        double r = 0.0;
         for (int q = p0 + s; q < p0 + s + nr; ++q) {
           const WP ws = prev[q], wt = prev[twin[q]];
-          r += port_residual<WT>(ws.x, ws.y, wt.x, wt.y, kd[q]);
+          r += (double)port_residual<WT>(ws.x, ws.y, wt.x, wt.y, kd[q]);
         }
         sq += r * r;
       }
@@ -953,7 +954,7 @@ __global__ void __launch_bounds__(256, 3) sweep_slab_kernel(
   __syncthreads();  // the ring becomes the partial sums
 #pragma unroll
   for (int e = 0; e < VEC; ++e) red[g * SW + l * VEC + e] = acc[e];
-  const double slab_sq = sizeof(WT) == 8 ? block_sum_value((double)sq) : (double)block_sum_value_f((float)sq);
+  const double slab_sq = block_sum_value(sq);
   // (the sum's barriers stand between the partials and their readers)
   if (tid < SW && it.m0 + tid < p) {
     const int s = it.m0 + tid;

@@ -37,3 +37,18 @@ def test_slab_sweeps_follow_the_oracle(name, precision):
     k = min(kmax, int(np.count_nonzero((h > 0) & (href[: len(h)] > floor))))
     assert k >= 1
     assert np.allclose(h[:k], href[:k], rtol=rtol, atol=1e-13 if precision == "fp64" else 0)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("scale", [2.0 ** -60, 2.0 ** -45, 2.0 ** 70])
+def test_right_hand_sides_of_any_size(precision, scale):
+    """A power of two on b changes no bit of the sweeps or of their residuals while the
+    waves stay in FP32's range (entries of b from 1e-18 to 1e21 here; squared residuals leave it)."""
+    from paper_0910_0663_gb300 import vtm
+    w = PLANS["boxes"]()
+    plan = vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts, Zc=w.Zc, precision=precision, sweep_kernel=1)
+    b = torch.from_numpy(w.b[0]).cuda()
+    x, info = plan.solve(b, tol=1e-8)
+    y, scaled = plan.solve(b * scale, tol=1e-8)
+    assert scaled["sweeps"] == info["sweeps"] and scaled["outer_steps"] == info["outer_steps"]
+    assert torch.equal(y, x * scale)
