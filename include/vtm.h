@@ -171,7 +171,8 @@ typedef struct {
                         precision, or (2, 4) with a column count that is not a
                         multiple of 8, runs the CUDA-core variant */
   int wait_polls;    /* polls a bounded device-side wait of the sweeps that run in one
-                        launch (kernels 8 and 10, and the resident form) makes before it gives up with VTM_ETIMEOUT;
+                        launch (kernels 8 and 10, the resident form, and those of plans
+                        with lagged couplings) makes before it gives up with VTM_ETIMEOUT;
                         0: default 4194304 (a few seconds).  The bulk-copy waits of
                         kernels 2 and 7 keep their own limit: a CTA never leaves while a
                         copy into its shared memory is in flight */

@@ -532,7 +532,7 @@ static vtm_status general_sweeps_resident(vtm_plan_s* P, int budget, double* his
   a.nparts = P->nparts;
   a.nslots = P->gen_nslots;
   a.vmax = P->gen_vmax;
-  a.max_polls = 1u << 22;  // seconds: a bound, not a limit that a solve can meet
+  a.max_polls = (uint32_t)P->opts.wait_polls;
   VTM_CUDA_TRY(cudaMemsetAsync(P->d_gen_part.p, 0, 64, s));
   void* args[] = {&a};
   VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));

@@ -86,3 +86,16 @@ def test_a_sweep_limit_above_what_the_barrier_counts(vtm, limit):
     assert many["kernel_launches"] > many["sweeps"]
     assert abs(many["sweeps"] - info["sweeps"]) <= 1  # (sums in another order)
     assert O.residual_norms(w.csr(), y.cpu().numpy().reshape(w.b.shape), w.b).max() <= 1e-9
+
+
+def test_wait_polls_bounds_the_channel_form_too(vtm):
+    w = wl.vccs_grid(200, 200, 50, 50, seed=12)
+    plan = vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts, Zc=1.0)
+    b = torch.from_numpy(w.b).cuda()
+    x, _ = plan.solve(b)
+    plan.set_options(wait_polls=1)  # the first poll that finds the barrier open gives up
+    with pytest.raises(vtm.VTMError, match="timed out"):
+        plan.solve(b)
+    plan.set_options(wait_polls=0)
+    y, _ = plan.solve(b)
+    assert torch.equal(x, y)
