@@ -61,7 +61,11 @@ typedef enum {
 
 /* Arithmetic of the sub-circuit applies (the reflection-matrix products). */
 enum {
-  VTM_PREC_FP64 = 0, /* plain FP64 VTM */
+  VTM_PREC_FP64 = 0, /* plain FP64 VTM.  Sweeps in FP64 or, on symmetric plans of at most 128
+                        ports per sub-circuit where it is faster (vtm_opts.sweep_kernel 12, an
+                        autotuner candidate), in double-float: about 48 bits, waves within
+                        FP32's exponent range, residuals down to about 1e-13 ||b||.
+                        sweep_kernel 1..4 keep every solve of a plan in FP64 */
   VTM_PREC_FP32 = 1, /* FP32 T_P and waves, FP32 accumulate, inside FP64 iterative refinement */
   VTM_PREC_BF16 = 2, /* BF16 T_P, FP32 waves and accumulate, inside FP64 iterative refinement */
   VTM_PREC_FP16 = 3  /* FP16 T_P, FP32 waves and accumulate, inside FP64 iterative refinement:
@@ -214,10 +218,12 @@ typedef struct {
   int64_t t_bytes;       /* bytes of the stored reflection matrices (all precisions kept) */
   int64_t factor_bytes;  /* bytes of the stored local factors */
   int32_t sweep_kernel;  /* sweep kernel in use for the plan's precision (see vtm_opts); 8 also
-                            stands for the resident form the autotuner may pick on plans of
-                            few sub-circuits: every sweep of an inner solve in one launch,
-                            blocks in shared memory, a grid barrier per sweep (bounded by
-                            wait_polls) or one CTA */
+                            stands for the resident forms that only the autotuner picks
+                            (sweep_kernel 0; requesting 8 gives the dataflow kernel): every
+                            sweep of an inner solve in one launch, operators in shared
+                            memory as far as they fit, a grid barrier per sweep (bounded by
+                            wait_polls) or one CTA; on FP64 plans in FP64 or, in place of
+                            kernel 12, in double-float */
   int64_t sum_tri;       /* sum over sub-circuits of p_P (p_P + 1) / 2: the entries of the
                             symmetric reflection matrices on and above the diagonal */
   int64_t packed_bytes;  /* bytes of the packed symmetric copies (0 if none) */

@@ -877,10 +877,10 @@ __global__ void pack_sym_df_kernel(const double* __restrict__ T64, const TileDes
   }
 }
 
-// the double-float copy serves FP64 plans of a symmetric A: kernel 12 with at most
-// 128 ports per sub-circuit, kernel 13 with at most 256
+// the double-float copy serves FP64 plans of a symmetric A with at most 128
+// ports per sub-circuit (kernel 12 and its resident form, kernel 13)
 static bool packed_df_eligible(const vtm_plan_s* P) {
-  return P->symmetric && !P->general && P->max_ports <= 16 * kSymB && !P->port_node.empty() &&
+  return P->symmetric && !P->general && P->max_ports <= 8 * kSymB && !P->port_node.empty() &&
          P->opts.precision == VTM_PREC_FP64;
 }
 

@@ -259,6 +259,9 @@ __global__ void __launch_bounds__(1024) general_sweep_kernel(
 // sweeps in tiles of 16 x 16 14.8 ms against 24.2, of 8 x 8 21.6 against 44.3).
 constexpr int kGenThreads = 768;  // and a control warp: 80 registers per thread
 constexpr int kGenRing = 4, kGenMinSlots = 8;
+// elements (pairs of outputs times an input) per thread below which fewer CTAs share the work
+template <bool PORTS>
+constexpr int kGenMinElems = PORTS ? 2 : 8;
 struct GenCta {
   int32_t pair0, np;   // first output pair, pairs
   int32_t in0, nin;    // inputs of the tiles it touches
@@ -273,6 +276,7 @@ struct GenRes {
   const int32_t *in_src, *in_own_out, *res_in;
   const uint8_t *in_kind, *res_run;
   const double *coef, *dsc, *c;
+  const double2* kd;  // port form: (g/W, d)
   double *gin, *gout;
   int64_t n_in, n_out;
   SweepCtrl* ctrl;
@@ -282,6 +286,15 @@ struct GenRes {
   uint32_t max_polls;
 };
 
+// PORTS: the sweeps of a plan without lagged couplings, FP64 throughout -- E_P = T_P, the
+// inputs and outputs of a tile its ports in their order, the source of an input its twin.
+// The last sweep leaves (w_in, w_out) pairs in gin.  For symmetric plans of up to 256 ports
+// per tile, like kernel 13.  Measured per sweep, kernel 1 -> here: 64 tiles of 256 ports
+// (33 MB of T_P, 6.9 us of FP64 pipe) 19 -> 11.1 us; 169 tiles of 128 ports 18.4 -> 9.3 us;
+// 9 tiles of 128 ports 16.4 -> 7.0 us.  CTAs with as little as two elements per thread:
+// 81 tiles of 124 ports 7.1 us, with at least eight 8.6 us (the channel form keeps eight:
+// its inputs gather from more tiles).
+template <bool PORTS>
 __global__ void __launch_bounds__(kGenThreads + 32, 1) general_resident_kernel(const GenRes A) {
   constexpr int NT = kGenThreads, NW = NT / 32, S = kGenRing;
   extern __shared__ __align__(16) unsigned char gsm[];
@@ -392,15 +405,16 @@ __global__ void __launch_bounds__(kGenThreads + 32, 1) general_resident_kernel(c
         if (!nr) continue;
         double r = 0.0;
         for (int e = 0; e < nr; ++e) {
-          const int a = A.res_in[q + e], s = A.in_src[a];
+          const int a = PORTS ? q + e : A.res_in[q + e], s = A.in_src[a];
           const double wo_t = __ldcg(prev + s), wi_s = __ldcg(pp + s);
-          if (A.in_kind[a] != 0) {
+          if (!PORTS && A.in_kind[a] != 0) {
             r += A.coef[a] * (wi_s - wo_t);
           } else {
-            const int own = A.in_own_out[a];
+            const int own = PORTS ? a : A.in_own_out[a];
             const double wo_s = __ldcg(prev + own), wi_t = __ldcg(pp + own);
             const double Ss = wi_s + wo_s, St = wi_t + wo_t;
-            r += 0.5 * A.dsc[a] * (0.5 * (Ss + St) - A.coef[a] * (Ss - St) - wi_s - wi_t);
+            const double2 kd = PORTS ? __ldg(A.kd + a) : make_double2(A.coef[a], A.dsc[a]);
+            r += 0.5 * kd.y * (0.5 * (Ss + St) - kd.x * (Ss - St) - wi_s - wi_t);
           }
         }
         sq += r * r;
@@ -415,30 +429,40 @@ __global__ void __launch_bounds__(kGenThreads + 32, 1) general_resident_kernel(c
   // the decision of sweep k - 1 closed sweep k - 3: its iterate, or the one before
   const int it = flag == 1 ? k - 4 : k - 3;
   const double* from = A.gout + (size_t)((it - 1) & (kGenSlots - 1)) * A.n_out;
-  for (int a = C.i0 + tid; a < C.i1; a += NT) A.gin[(size_t)(it & 1) * A.n_in + a] = __ldcg(from + A.in_src[a]);
+  for (int a = C.i0 + tid; a < C.i1; a += NT) {
+    const double w = __ldcg(from + A.in_src[a]);
+    if constexpr (PORTS)
+      reinterpret_cast<double2*>(A.gin)[a] =
+          make_double2(w, __ldcg(A.gout + (size_t)(it & (kGenSlots - 1)) * A.n_out + a));
+    else A.gin[(size_t)(it & 1) * A.n_in + a] = w;
+  }
 }
 
-// the CTAs of the resident form; gen_ctas stays 0 where it does not apply
-static vtm_status plan_general_resident(vtm_plan_s* P) {
+// the CTAs of the resident form; gen_ctas is -1 where it does not apply
+template <bool PORTS>
+static vtm_status plan_resident(vtm_plan_s* P) {
   P->gen_ctas = -1;
+  const std::vector<int32_t>&in_off = PORTS ? P->port_off : P->in_off, &out_off = PORTS ? P->port_off : P->out_off;
+  const std::vector<uint8_t>& run = PORTS ? P->port_run : P->res_run;
+  const int64_t n_in = PORTS ? (int64_t)P->port_node.size() : P->n_in, n_out = PORTS ? n_in : P->n_out;
   int coop = 0, sms = 152;
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, P->device);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, P->device);
-  if (!coop || P->n_in == 0 || P->n_out == 0) return VTM_OK;
-  std::vector<int32_t> pair_off(P->nparts + 1, 0), res_in(P->n_in);
+  if (!coop || n_in == 0 || n_out == 0) return VTM_OK;
+  std::vector<int32_t> pair_off(P->nparts + 1, 0), res_in(PORTS ? 0 : n_in);
   int64_t cost = 0;  // elements of E_P in pairs, and the sums
-  auto pairs = [&](int32_t t) { return (P->out_off[t + 1] - P->out_off[t] + 1) / 2; };
-  auto pair_cost = [&](int32_t t) { return (int64_t)(P->in_off[t + 1] - P->in_off[t]) + 4; };
+  auto pairs = [&](int32_t t) { return (out_off[t + 1] - out_off[t] + 1) / 2; };
+  auto pair_cost = [&](int32_t t) { return (int64_t)(in_off[t + 1] - in_off[t]) + 4; };
   for (int32_t t = 0; t < P->nparts; ++t) {
     pair_off[t + 1] = pair_off[t] + pairs(t);
     cost += pairs(t) * pair_cost(t);
-    for (int32_t a = P->in_off[t]; a < P->in_off[t + 1]; ++a) res_in[a] = P->in_off[t] + P->res_perm[a];
+    if (!PORTS)
+      for (int32_t a = in_off[t]; a < in_off[t + 1]; ++a) res_in[a] = in_off[t] + P->res_perm[a];
   }
-  // at least eight elements per thread
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, cost / (8 * kGenThreads)));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, cost / (kGenMinElems<PORTS> * kGenThreads)));
   std::vector<GenCta> ctas(grid);
   auto run_start = [&](int64_t q) {
-    while (q < P->n_in && !P->res_run[q]) ++q;
+    while (q < n_in && !run[q]) ++q;
     return (int32_t)q;
   };
   int32_t t = 0, pr = 0;  // next pair: pair `pr` of tile t
@@ -453,7 +477,7 @@ static vtm_status plan_general_resident(vtm_plan_s* P) {
     }
     c.pair0 = t < P->nparts ? pair_off[t] + pr : pair_off[P->nparts];
     c.np = 0;
-    c.in0 = t < P->nparts ? P->in_off[t] : 0;
+    c.in0 = t < P->nparts ? in_off[t] : 0;
     int32_t last = t;
     while (t < P->nparts && done < upto) {
       if (pr >= pairs(t)) {
@@ -468,31 +492,32 @@ static vtm_status plan_general_resident(vtm_plan_s* P) {
       done += take * pc;
       last = t;
     }
-    c.nin = c.np > 0 ? P->in_off[last + 1] - c.in0 : 0;
+    c.nin = c.np > 0 ? in_off[last + 1] - c.in0 : 0;
     vmax = std::max(vmax, c.nin);
     if (c.np > kGenThreads) return VTM_OK;
-    c.i0 = (int32_t)(P->n_in * b / grid);
-    c.i1 = (int32_t)(P->n_in * (b + 1) / grid);
+    c.i0 = (int32_t)(n_in * b / grid);
+    c.i1 = (int32_t)(n_in * (b + 1) / grid);
     c.q0 = run_start(c.i0);
     c.q1 = run_start(c.i1);
   }
   vmax = (vmax + 1) / 2 * 2;
   const int64_t fixed = (int64_t)kGenThreads * 16 + 12 * (int64_t)vmax + 8 * kGenThreads;
+  auto* kern = general_resident_kernel<PORTS>;
   int optin = 0, fits = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, P->device);
   cudaFuncAttributes fa{};
-  VTM_CUDA_TRY(cudaFuncGetAttributes(&fa, general_resident_kernel));
+  VTM_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
   const int nslots = (int)((optin - (int64_t)fa.sharedSizeBytes - fixed) / (kGenThreads * 16));
   if (nslots < kGenMinSlots) return VTM_OK;
   P->gen_smem = fixed + (int64_t)nslots * kGenThreads * 16;
-  VTM_CUDA_TRY(allow_smem(general_resident_kernel, (size_t)P->gen_smem));
-  VTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, general_resident_kernel, kGenThreads + 32,
-                                                             (size_t)P->gen_smem));
+  VTM_CUDA_TRY(allow_smem(kern, (size_t)P->gen_smem));
+  VTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fits, kern, kGenThreads + 32, (size_t)P->gen_smem));
   if (fits < 1) return VTM_OK;
   cudaStream_t s = P->stream;
   VTM_TRY(upload(P->d_gen_ctas, ctas, s));
   VTM_TRY(upload(P->d_gen_pair, pair_off, s));
-  VTM_TRY(upload(P->d_gen_res, res_in, s));
+  if (PORTS) VTM_TRY(dev_alloc(P->d_gout, kGenSlots * n_out * sizeof(double)));
+  else VTM_TRY(upload(P->d_gen_res, res_in, s));
   VTM_TRY(dev_alloc(P->d_gen_part, 64 + 2 * (size_t)grid * sizeof(double)));
   VTM_CUDA_TRY(cudaStreamSynchronize(s));  // the host lists are about to go
   P->gen_nslots = nslots;
@@ -501,29 +526,52 @@ static vtm_status plan_general_resident(vtm_plan_s* P) {
   return VTM_OK;
 }
 
-static vtm_status general_sweeps_resident(vtm_plan_s* P, int budget, double* hist, int hist_len, int* sweep_out,
-                                          int* flag_out) {
+// (without the memory for it the plan keeps one launch per sweep)
+template <bool PORTS>
+static vtm_status plan_resident_if_room(vtm_plan_s* P) {
+  const vtm_status st = plan_resident<PORTS>(P);
+  if (st != VTM_ENOMEM) return st;
+  cudaGetLastError();
+  P->gen_ctas = -1;
+  return VTM_OK;
+}
+
+template <bool PORTS>
+static cudaError_t launch_resident(vtm_plan_s* P, double* hist, int hist_len) {
   cudaStream_t s = P->stream;
   GenRes a{};
-  a.E = P->d_E.as<double>();
-  a.E_off = P->d_E_off.as<int64_t>();
-  a.E_ld = P->d_E_ld.as<int32_t>();
-  a.in_off = P->d_in_off.as<int32_t>();
-  a.out_off = P->d_out_off.as<int32_t>();
-  a.pair_off = P->d_gen_pair.as<int32_t>();
   a.ctas = P->d_gen_ctas.as<GenCta>();
-  a.in_src = P->d_in_src.as<int32_t>();
-  a.in_own_out = P->d_in_own_out.as<int32_t>();
-  a.res_in = P->d_gen_res.as<int32_t>();
-  a.in_kind = P->d_in_kind.as<uint8_t>();
-  a.res_run = P->d_res_run.as<uint8_t>();
-  a.coef = P->d_in_coef.as<double>();
-  a.dsc = P->d_in_d.as<double>();
-  a.c = P->d_cg.as<double>();
-  a.gin = P->d_gin.as<double>();
+  a.pair_off = P->d_gen_pair.as<int32_t>();
   a.gout = P->d_gout.as<double>();
-  a.n_in = P->n_in;
-  a.n_out = P->n_out;
+  if constexpr (PORTS) {
+    a.E = P->d_T64.as<double>();
+    a.E_off = P->tabs.T_off.as<int64_t>();
+    a.E_ld = P->tabs.T_ld.as<int32_t>();
+    a.in_off = a.out_off = P->tabs.port_off.as<int32_t>();
+    a.in_src = P->d_twin.as<int32_t>();
+    a.res_run = P->d_run.as<uint8_t>();
+    a.kd = P->d_kd.as<double2>();
+    a.c = P->d_c64.as<double>();
+    a.gin = P->d_state64.as<double>();
+    a.n_in = a.n_out = (int64_t)P->port_node.size();
+  } else {
+    a.E = P->d_E.as<double>();
+    a.E_off = P->d_E_off.as<int64_t>();
+    a.E_ld = P->d_E_ld.as<int32_t>();
+    a.in_off = P->d_in_off.as<int32_t>();
+    a.out_off = P->d_out_off.as<int32_t>();
+    a.in_src = P->d_in_src.as<int32_t>();
+    a.in_own_out = P->d_in_own_out.as<int32_t>();
+    a.res_in = P->d_gen_res.as<int32_t>();
+    a.in_kind = P->d_in_kind.as<uint8_t>();
+    a.res_run = P->d_res_run.as<uint8_t>();
+    a.coef = P->d_in_coef.as<double>();
+    a.dsc = P->d_in_d.as<double>();
+    a.c = P->d_cg.as<double>();
+    a.gin = P->d_gin.as<double>();
+    a.n_in = P->n_in;
+    a.n_out = P->n_out;
+  }
   a.ctrl = P->d_ctrl.as<SweepCtrl>();
   a.bar = reinterpret_cast<unsigned long long*>(P->d_gen_part.p);
   a.part = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(P->d_gen_part.p) + 64);
@@ -533,11 +581,29 @@ static vtm_status general_sweeps_resident(vtm_plan_s* P, int budget, double* his
   a.nslots = P->gen_nslots;
   a.vmax = P->gen_vmax;
   a.max_polls = (uint32_t)P->opts.wait_polls;
-  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gen_part.p, 0, 64, s));
+  cudaError_t e = cudaMemsetAsync(P->d_gen_part.p, 0, 64, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.gout, 0, a.n_out * sizeof(double), s);  // slot 0: the first sweep's waves
+  if (e != cudaSuccess) return e;
   void* args[] = {&a};
+  return cudaLaunchCooperativeKernel((const void*)general_resident_kernel<PORTS>, dim3(P->gen_ctas),
+                                     dim3(kGenThreads + 32), args, (size_t)P->gen_smem, s);
+}
+
+// The port form for run_sweeps: true where it serves this many sweeps.
+vtm_status port_resident_prepare(vtm_plan_s* P, int budget, bool* ok) {
+  if (P->gen_ctas == 0) VTM_TRY(plan_resident_if_room<true>(P));
+  *ok = P->gen_ctas > 0 && res_counts(budget, P->gen_ctas);
+  return VTM_OK;
+}
+cudaError_t launch_port_resident(vtm_plan_s* P, double* hist, int hist_len) {
+  return launch_resident<true>(P, hist, hist_len);
+}
+
+static vtm_status general_sweeps_resident(vtm_plan_s* P, int budget, double* hist, int hist_len, int* sweep_out,
+                                          int* flag_out) {
+  cudaStream_t s = P->stream;
   VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
-  VTM_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)general_resident_kernel, dim3(P->gen_ctas),
-                                           dim3(kGenThreads + 32), args, (size_t)P->gen_smem, s));
+  VTM_CUDA_TRY(launch_resident<false>(P, hist, hist_len));
   VTM_CUDA_TRY(cudaEventRecord(P->evs1, s));
   VTM_CUDA_TRY(cudaMemcpyAsync(P->h_ctrl, P->d_ctrl.p, sizeof(SweepCtrl), cudaMemcpyDeviceToHost, s));
   VTM_CUDA_TRY(cudaStreamSynchronize(s));
@@ -603,7 +669,7 @@ vtm_status general_sweeps(vtm_plan_s* P, double bnorm2, double target2, int budg
   VTM_CUDA_TRY(cudaMemcpyAsync(P->d_ctrl.p, P->h_ctrl, sizeof(SweepCtrl), cudaMemcpyHostToDevice, s));
   VTM_CUDA_TRY(cudaMemsetAsync(P->d_gin.p, 0, 2 * std::max<int64_t>(P->n_in, 1) * sizeof(double), s));
   VTM_CUDA_TRY(cudaMemsetAsync(P->d_gout.p, 0, kGenSlots * std::max<int64_t>(P->n_out, 1) * sizeof(double), s));
-  if (P->gen_ctas == 0) VTM_TRY(plan_general_resident(P));
+  if (P->gen_ctas == 0) VTM_TRY(plan_resident_if_room<false>(P));
   // (the barrier word holds as many arrivals and sweeps as res_counts allows; above that one
   // launch per sweep)
   if (P->gen_ctas > 0 && res_counts(budget, P->gen_ctas))

@@ -990,7 +990,7 @@ extern "C" vtm_status vtm_plan_get_stats(vtm_plan_t P, vtm_plan_stats* s) {
                          P->d_Tp32.bytes + P->d_Tp16.bytes + P->d_Tpdf.bytes);
   s->factor_bytes = 2 * P->band_elems * (int64_t)sizeof(double);
   s->sweep_kernel = P->opts.method == VTM_METHOD_ASYNC   ? P->dataflow_kernel
-                    : P->tuned_kernel[P->opts.precision] == 13 ? 8  // its resident form
+                    : P->tuned_kernel[P->opts.precision] >= 13 ? 8  // the resident forms
                     : P->tuned_kernel[P->opts.precision] ? P->tuned_kernel[P->opts.precision]
                                                          : P->opts.sweep_kernel;
   s->sum_tri = P->sum_tri;

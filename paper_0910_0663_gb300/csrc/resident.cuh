@@ -12,8 +12,10 @@
 //     end.  The last blocks of each range, as many as fit, stay in shared memory;
 //     the others stream from L2 through two register slots, loaded while the grid
 //     barrier is awaited.
-//   * Arithmetic as in kernel 9 (FP32, BF16, FP16 storage) and kernel 12 (FP64
-//     plans: hi + lo FP32 pairs, double-float), for tiles of up to 256 ports.
+//   * Arithmetic as in kernel 9 (FP32, BF16, FP16 storage; tiles of up to 256 ports) and
+//     kernel 12 (FP64 plans: hi + lo FP32 pairs, double-float; up to 128 ports, and only
+//     where kernel 12 is the fastest of the launch-per-sweep kernels: elsewhere FP64 plans
+//     sweep in FP64, in one launch by general_resident_kernel<true> of general.cu).
 //   * The residual terms of sweep k - 1 (from what the gather of sweep k read) are
 //     formed while the grid barrier is awaited, so nothing but the waves is on the
 //     critical path.  The control warp publishes the CTA's partial one sweep later,
@@ -26,7 +28,8 @@
 // double-float the FP32 pipe and the latency of its chains in the block loop (30k
 // instructions per sweep of a 256-port tile).  Measured per sweep, best
 // launch-per-sweep kernel -> this one:
-//   FP64  64 tiles of 256 ports 19 -> 9.7 us; 1504 tiles of 128 ports 36 -> 31 us
+//   FP64  1504 tiles of 128 ports 36 -> 31 us; 121 tiles of 80 ports 13.3 -> 4.0 us (the FP64
+//         resident form 6.7 us)
 //   FP32  256 tiles of 256 ports 13.6 -> 6.7 us; 1232 tiles of 116 ports 13.3 -> 11 us
 //   FP16  256 tiles of 128 ports 6 -> 3.2 us
 // With more than 11 (FP64) or 15 tiles per SM (2048^2 in 4096 tiles) the

@@ -2840,6 +2840,11 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   const int wdf_grid = (P->nparts + wdf_warps - 1) / wdf_warps;
   const int wdf_threads = 32 * (wdf_warps + 4);
   const size_t wdf_smem = wdf_warps * wdf_per_warp;
+  // kernel 14: every sweep in one launch, FP64 throughout (general.cu)
+  bool port_ok = false;
+  if (prec == VTM_PREC_FP64 && P->symmetric && P->max_ports <= 16 * kSymB && P->opts.sweep_kernel == 0 &&
+      P->opts.method != VTM_METHOD_ASYNC)
+    VTM_TRY(port_resident_prepare(P, budget, &port_ok));
   // kernel 13 (every sweep in one launch, blocks in shared memory): packed
   // copies, at most 15 tiles per SM (FP64: 11) and what its warps and shared memory hold
   ResArgs ra{};
@@ -3238,6 +3243,13 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
                     &ct, &p4, &hp, &hl, &np, &ppm, &k0, &mp, &ls};
     return cudaLaunchCooperativeKernel(wflow_kfn, wflow_grid, 32 * kWflowWarps, args, wflow_smem, s);
   };
+  // every sweep of the inner solve in one launch
+  auto launch_whole = [&](int k) -> cudaError_t {
+    return k == 14   ? launch_port_resident(P, hist, hist_len)
+           : k == 13 ? launch_resident()
+           : k == 10 ? launch_wflow()
+                     : launch_flow();
+  };
   const bool symload = ((choice == 5 || choice == 6 || choice == 9) && sym_ok) || (choice == 7 && symb_ok) ||
                        (choice == 8 && flow_ok) || (choice == 10 && wflow_ok) || (choice == 11 && wmma_ok) ||
                        (choice == 12 && wdf_ok);
@@ -3271,7 +3283,7 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
   else if (P->opts.sweep_kernel == 0) {
     // the candidates of this solve: what the sweep limit, the precisions' copies and the
     // device allow.  A choice made among others is made again
-    const bool can[14] = {false,
+    const bool can[15] = {false,
                           true,
                           nv_max <= 4 * 256 && st_smem <= 200 * 1024,
                           nv_max <= 256,
@@ -3284,25 +3296,29 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
                           wflow_ok,
                           wmma_ok,
                           wdf_ok,
-                          res_ok};
+                          res_ok,
+                          port_ok};
     int mask = 0;
-    for (int cand = 1; cand <= 13; ++cand) mask |= (int)can[cand] << cand;
+    for (int cand = 1; cand <= 14; ++cand) mask |= (int)can[cand] << cand;
     if (P->tuned_kernel[prec] == 0 || P->tuned_among[prec] != mask) {
       float best = 1e30f;
       int best_k = 1;
-      for (int cand = 1; cand <= 13; ++cand) {
+      for (int cand = 1; cand <= 14; ++cand) {
         if (!can[cand]) continue;
-        if (cand == 8 || cand == 10 || cand == 13) {  // one launch, per-sweep time against the others' 6
+        // on FP64 plans kernel 13 stands in for kernel 12 only: where an FP64 kernel is
+        // the faster one of 1..12, no sweep runs in double-float
+        if (cand == 13 && prec == VTM_PREC_FP64 && best_k != 12) continue;
+        if (cand == 8 || cand == 10 || cand >= 13) {  // one launch, per-sweep time against the others' 6
           SweepCtrl t = h;
-          // (kernel 13 fills shared memory first: more sweeps to set against that)
-          const int nsw = cand == 13 ? 48 : 8;
+          // (kernels 13 and 14 fill shared memory first: more sweeps to set against that)
+          const int nsw = cand >= 13 ? 48 : 8;
           t.k_max = nsw;
           t.tol2 = -1.0;
           t.stall = 0;
           *P->h_ctrl = t;
           VTM_TRY(upload_ctrl(P, s));
           VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
-          VTM_CUDA_TRY(cand == 13 ? launch_resident() : cand == 10 ? launch_wflow() : launch_flow());
+          VTM_CUDA_TRY(launch_whole(cand));
           VTM_CUDA_TRY(cudaEventRecord(P->evs1, s));
           VTM_CUDA_TRY(cudaEventSynchronize(P->evs1));
           float ms = 0.f;
@@ -3374,9 +3390,9 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
     P->wave_slot = P->d_state64.as<double>();
     return VTM_OK;
   };
-  if (kern == 8 || kern == 10 || kern == 13) {
+  if (kern == 8 || kern == 10 || kern >= 13) {
     VTM_CUDA_TRY(cudaEventRecord(P->evs0, s));
-    VTM_CUDA_TRY(kern == 13 ? launch_resident() : kern == 10 ? launch_wflow() : launch_flow());
+    VTM_CUDA_TRY(launch_whole(kern));
     VTM_CUDA_TRY(cudaEventRecord(P->evs1, s));
     VTM_CUDA_TRY(cudaMemcpyAsync(P->h_ctrl, P->d_ctrl.p, sizeof(SweepCtrl), cudaMemcpyDeviceToHost, s));
     VTM_CUDA_TRY(cudaStreamSynchronize(s));
@@ -3392,6 +3408,10 @@ static vtm_status run_sweeps(vtm_plan_s* P, double bnorm2, double target2, int b
     }
     *flag_out = r.flag;
     *sweep_out = (r.flag == 1 || r.flag == 4) ? r.conv_sweep : std::min(r.k - 1, budget);
+    if (kern == 14) {  // the pairs of that sweep are in the first slot
+      P->wave_slot = P->d_state64.p;
+      return VTM_OK;
+    }
     if (kern == 13 && prec == VTM_PREC_FP64) return join_df();
     const int slots = kern == 13 ? kResSlots : 3;
     P->wave_slot = P->d_fstate32.as<float>() +

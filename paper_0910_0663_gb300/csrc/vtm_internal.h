@@ -314,7 +314,8 @@ struct vtm_plan_s {
   int64_t E_elems = 0;
   int32_t max_in = 0, max_out = 0;
   int64_t n_in = 0, n_out = 0;
-  // channel-form sweeps in one launch (gen_ctas: 0 not planned, -1 not possible)
+  // channel-form sweeps in one launch, and those of FP64 plans without lagged couplings
+  // (kernel 14; gen_ctas: 0 not planned, -1 not possible)
   vtm::DevBuf d_gen_ctas, d_gen_pair, d_gen_res, d_gen_part;
   int gen_ctas = 0, gen_nslots = 0, gen_vmax = 0;
   int64_t gen_smem = 0;
@@ -405,6 +406,8 @@ constexpr int kGenSlots = 8;  // slots of the outputs (the launch-per-sweep form
 vtm_status general_sweeps(vtm_plan_s* P, double bnorm2, double target2, int budget, double* hist,
                           int hist_len, int* sweep_out, int* flag_out);
 vtm_status general_inject(vtm_plan_s* P, int sweep, double* v);
+vtm_status port_resident_prepare(vtm_plan_s* P, int budget, bool* ok);  // (kernel 14)
+cudaError_t launch_port_resident(vtm_plan_s* P, double* hist, int hist_len);
 
 // factor.cu
 vtm_status factor_tiles(vtm_plan_s* P);

@@ -142,3 +142,32 @@ def test_the_choice_follows_what_a_later_solve_allows(precision):
         solves(precision="fp64")
         plan.factor()
         solves()
+
+
+# 9 tiles of up to 128 ports (in one launch, FP64 or double-float by speed) and 6 of up to
+# 256 (FP64)
+FP64 = [((66, 65), (32, 32)), GRID[2]]
+
+
+@pytest.mark.parametrize("shape", ONE + GRID + FP64)
+def test_fp64_histories_at_the_other_kernels_bar(shape):
+    w, plan = _plan(shape, "fp64")
+    plan.set_options(history_len=40, max_sweeps=40)
+    plan.solve(torch.from_numpy(w.b[0]).cuda(), tol=1e-300, check=False)
+    assert plan.stats()["sweep_kernel"] == 8
+    ref = O.vtm_midpoint(w.csr(), w.partition, w.nparts, w.b[:1], W=1 / w.Zc, tol=0, max_sweeps=40)
+    h, href = plan.history, ref.history[:, 0]
+    k = int(np.count_nonzero((h > 0) & (href[: len(h)] > 1e-9)))
+    assert k >= 1 and np.allclose(h[:k], href[:k], rtol=1e-9, atol=1e-13)
+
+
+def test_tiles_above_128_ports_sweep_in_fp64():
+    """53 bits and FP64's range: a residual of 1e-14 is reached (double-float ends near
+    1e-13), and a power of two on b changes no bit."""
+    w, plan = _plan(GRID[2], "fp64", max_sweeps=20000)
+    b = torch.from_numpy(w.b[0]).cuda()
+    x, info = plan.solve(b, tol=1e-14)
+    assert info["relres"] <= 1e-14 and plan.stats()["sweep_kernel"] == 8
+    for e in (-400, 400):
+        y, scaled = plan.solve(b * 2.0 ** e, tol=1e-14)
+        assert scaled["sweeps"] == info["sweeps"] and torch.equal(y, x * 2.0 ** e)
