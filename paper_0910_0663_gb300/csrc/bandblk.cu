@@ -38,13 +38,23 @@ namespace vtm {
 constexpr int kBbN = 32;                 // rows per block
 constexpr uint32_t kBbPolls = 1u << 24;  // mbarrier polls before giving up
 
+// Skeel condition of the diagonal blocks M (largest row sum of |M^-1| |M|) up to which
+// their inverses serve.  A product with the inverse is off by u |M^-1| |t| <= u |M^-1| |M| |u|,
+// so by this many u of the largest element, the bound that substitution has too.  Where no
+// column of K_P outweighs its diagonal |M^-1| <= 1; thermal grids measure 3, resistor and
+// power grids 20 to 26, VCCS grids 22 to 28.  Beyond the limit -- LU of a matrix with
+// large multipliers, say -- the solves substitute row by row, whose residual stays at a few u all
+// the same: 64 rows, half bandwidth 40 and multipliers of -1.8 below the diagonal left
+// 2e-9 by inverses, 3e-16 by substitution.
+constexpr float kBbMaxCond = 256.f;
+
 // Inverses of the unit-triangular diagonal blocks, one warp per (block, pass):
 // lane q keeps column q of the inverse and substitutes through the block.
 // inv[(first block of the tile + k) 1024 + q 32 + r]; rows past n are identity.
 __global__ void __launch_bounds__(128) band_inverse_kernel(
     const int32_t* __restrict__ node_off, const int32_t* __restrict__ bwv, const int64_t* __restrict__ band_off,
     const int32_t* __restrict__ blk_off, int nparts, const double* __restrict__ Lc,
-    const double* __restrict__ Uc, double* __restrict__ Li, double* __restrict__ Ui) {
+    const double* __restrict__ Uc, double* __restrict__ Li, double* __restrict__ Ui, int* __restrict__ cond) {
   __shared__ double sm[4][kBbN * (kBbN + 1)];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = blockIdx.x * 4 + warp;
@@ -68,17 +78,25 @@ __global__ void __launch_bounds__(128) band_inverse_kernel(
   }
   __syncwarp();
   double x[kBbN];
+  float rs = 1.f;  // row sum of |M|
 #pragma unroll
   for (int r = 0; r < kBbN; ++r) {
     double acc = r == lane ? 1.0 : 0.0;
 #pragma unroll
     for (int p = 0; p < r; ++p) acc -= M[r * (kBbN + 1) + p] * x[p];
     x[r] = acc;
+    rs += fabsf((float)M[lane * (kBbN + 1) + r]);
   }
   __syncwarp();
 #pragma unroll
   for (int r = 0; r < kBbN; ++r) M[lane * (kBbN + 1) + r] = x[r];
   __syncwarp();
+  float c = 0.f;  // row `lane` of |M^-1| |M|, summed
+#pragma unroll
+  for (int q = 0; q < kBbN; ++q) c += fabsf((float)M[q * (kBbN + 1) + lane]) * __shfl_sync(0xffffffffu, rs, q);
+  for (int o = 16; o > 0; o >>= 1) c = fmaxf(c, __shfl_xor_sync(0xffffffffu, c, o));
+  // (bits of positive floats order like the floats; a NaN counts as too large)
+  if (lane == 0) atomicMax(cond, __float_as_int(c <= kBbMaxCond ? c : INFINITY));
   double* out = (fwd ? Li : Ui) + (int64_t)g * kBbN * kBbN;
 #pragma unroll 4
   for (int q = 0; q < kBbN; ++q) out[q * kBbN + lane] = M[q * (kBbN + 1) + lane];
@@ -280,6 +298,7 @@ bool band_blk_eligible(const vtm_plan_s* P) { return P->max_bw > 32 && P->max_bw
 
 // The inverted diagonal blocks of the current factors (vtm_factor).
 vtm_status band_blk_prepare(vtm_plan_s* P) {
+  P->bb_ok = false;
   if (!band_blk_eligible(P)) return VTM_OK;
   cudaStream_t s = P->stream;
   if (P->bb_blocks == 0) {
@@ -299,10 +318,12 @@ vtm_status band_blk_prepare(vtm_plan_s* P) {
   const int64_t ne = (int64_t)P->bb_blocks * kBbN * kBbN;
   VTM_TRY(dev_alloc(P->d_bb_Li, ne * sizeof(double)));
   VTM_TRY(dev_alloc(P->d_bb_Ui, ne * sizeof(double)));
+  int* d_cond = P->d_err.as<int>() + 1;
+  VTM_CUDA_TRY(cudaMemsetAsync(d_cond, 0, sizeof(int), s));
   band_inverse_kernel<<<dim3((P->bb_blocks + 3) / 4, 2), 128, 0, s>>>(
       P->tabs.node_off.as<int32_t>(), P->tabs.bw.as<int32_t>(), P->tabs.band_off.as<int64_t>(),
       P->d_bb_off.as<int32_t>(), P->nparts, P->d_Lc.as<double>(), P->d_Uc.as<double>(), P->d_bb_Li.as<double>(),
-      P->d_bb_Ui.as<double>());
+      P->d_bb_Ui.as<double>(), d_cond);
   VTM_CUDA_TRY(cudaGetLastError());
   if (P->opts.precision != VTM_PREC_FP64) {
     VTM_TRY(dev_alloc(P->d_bb_Li32, ne * sizeof(float)));
@@ -310,6 +331,10 @@ vtm_status band_blk_prepare(vtm_plan_s* P) {
     convert_f32(P->d_bb_Li.as<double>(), P->d_bb_Li32.as<float>(), ne, s);
     convert_f32(P->d_bb_Ui.as<double>(), P->d_bb_Ui32.as<float>(), ne, s);
   }
+  float cond = 0.f;
+  VTM_CUDA_TRY(cudaMemcpyAsync(&cond, d_cond, sizeof(float), cudaMemcpyDeviceToHost, s));
+  VTM_CUDA_TRY(cudaStreamSynchronize(s));
+  P->bb_ok = cond <= kBbMaxCond;
   return VTM_OK;
 }
 
@@ -341,14 +366,14 @@ static void launch_blk_t(vtm_plan_s* P, FT* v, const FT* Lc, const FT* Uc, const
 }
 
 bool launch_band_solve_blk(vtm_plan_s* P, double* v, int ncols, int64_t stride, cudaStream_t s) {
-  if (!band_blk_eligible(P) || !P->d_bb_Li.p) return false;
+  if (!P->bb_ok) return false;
   launch_blk_t<double>(P, v, P->d_Lc.as<double>(), P->d_Uc.as<double>(), P->d_bb_Li.as<double>(),
                        P->d_bb_Ui.as<double>(), ncols, stride, s);
   return true;
 }
 
 bool launch_band_solve_blk(vtm_plan_s* P, float* v, int ncols, int64_t stride, cudaStream_t s) {
-  if (!band_blk_eligible(P) || !P->d_bb_Li32.p) return false;
+  if (!P->bb_ok || !P->d_bb_Li32.p) return false;
   launch_blk_t<float>(P, v, P->d_Lc32.as<float>(), P->d_Uc32.as<float>(), P->d_bb_Li32.as<float>(),
                       P->d_bb_Ui32.as<float>(), ncols, stride, s);
   return true;

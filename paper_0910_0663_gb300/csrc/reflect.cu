@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kRfThreads, 2) build_reflection_blk_kernel(
 // Symmetric plans of half bandwidth 33 up to what ring and stages leave room for
 // (about 220); vtm_factor has made the inverted diagonal blocks.
 bool reflect_blk_eligible(const vtm_plan_s* P) {
-  return P->symmetric && !P->general && !P->port_node.empty() && P->max_bw > 32 && rf_smem(P->max_bw) <= 222 * 1024;
+  return P->symmetric && !P->general && !P->port_node.empty() && P->bb_ok && rf_smem(P->max_bw) <= 222 * 1024;
 }
 
 vtm_status build_reflections_blk(vtm_plan_s* P) {

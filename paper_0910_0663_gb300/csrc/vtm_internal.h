@@ -239,6 +239,7 @@ struct vtm_plan_s {
   // first block of each tile, tiles longest first (bandblk.cu)
   vtm::DevBuf d_bb_off, d_bb_order, d_bb_Li, d_bb_Ui, d_bb_Li32, d_bb_Ui32;
   int bb_blocks = 0;
+  bool bb_ok = false;  // the inverses follow the current factors and are well-conditioned
   // reflection build: work items, ports of each tile by row, forward results
   vtm::DevBuf d_refl_items, d_refl_order, d_refl_scratch;
   int refl_items = 0;

@@ -6,6 +6,7 @@ FP64 error stays below 17 * 64 u ~ 1.2e-13 (64 covers the growth of rounding
 along a row's band and inverse)."""
 import numpy as np
 import pytest
+import scipy.sparse as sp
 import scipy.sparse.linalg as sla
 import torch
 
@@ -51,3 +52,27 @@ def test_fp32_sweeps_with_wide_bands(width):
     # cond(A) <= 17 turns the residual bound into one of the error
     assert info["relres"] <= 1e-10
     assert np.linalg.norm(x.cpu().numpy() - ref) <= 17e-10 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("multiplier", [-1.8, -0.5])
+def test_large_multipliers_are_substituted(multiplier):
+    """A = L U with a chain of multipliers in L.  Blocks of a chain of -1.8 have a condition
+    of 1.8^32 and more: products with their inverses leave a residual near 1e-9
+    (1.8^32 u / 16), substitution a few u, and so do the inverses of a chain of -0.5.
+    At 1e-10 one direct solve tells them apart."""
+    from paper_0910_0663_gb300 import vtm
+    rng = np.random.default_rng(1)
+    n, bw = 64, 40
+    off = np.subtract.outer(np.arange(n), np.arange(n))
+    L = np.where((off > 0) & (off <= bw), rng.uniform(-0.01, 0.01, (n, n)), 0.0) + np.eye(n)
+    L[off == 1] = multiplier
+    U = np.where((off < 0) & (off >= -bw), rng.uniform(-0.01, 0.01, (n, n)), 0.0) + np.eye(n)
+    A = sp.csr_matrix(np.where(np.abs(off) <= bw, L @ U, 0.0))
+    A.sort_indices()
+    x0 = rng.uniform(-1, 1, n)
+    b = A @ x0
+    plan = vtm.Plan(A.indptr.astype(np.int64), A.indices.astype(np.int32), A.data, np.zeros(n, np.int32), 1)
+    assert plan.stats()["max_band"] == bw
+    x, info = plan.solve(torch.from_numpy(b).cuda(), tol=1e-10)
+    assert info["outer_steps"] == 1
+    assert np.linalg.norm(b - A @ x.cpu().numpy()) <= 1e-10 * np.linalg.norm(b)
