@@ -315,9 +315,21 @@ vtm_status band_blk_prepare(vtm_plan_s* P) {
     VTM_CUDA_TRY(cudaStreamSynchronize(s));  // the host tables are about to go
     P->bb_blocks = off[P->nparts];
   }
+  // Where the memory for the inverses runs out (512 bytes per unknown, 768 with FP32
+  // sweeps) the solves stay with the row-by-row kernels
   const int64_t ne = (int64_t)P->bb_blocks * kBbN * kBbN;
-  VTM_TRY(dev_alloc(P->d_bb_Li, ne * sizeof(double)));
-  VTM_TRY(dev_alloc(P->d_bb_Ui, ne * sizeof(double)));
+  const bool f32 = P->opts.precision != VTM_PREC_FP64;
+  const size_t sz[4] = {sizeof(double), sizeof(double), sizeof(float), sizeof(float)};
+  DevBuf* const inv[4] = {&P->d_bb_Li, &P->d_bb_Ui, &P->d_bb_Li32, &P->d_bb_Ui32};
+  for (int i = 0; i < (f32 ? 4 : 2); ++i) {
+    const vtm_status st = dev_alloc(*inv[i], ne * sz[i]);
+    if (st == VTM_ENOMEM) {
+      cudaGetLastError();
+      for (DevBuf* b : inv) dev_free(*b);
+      return VTM_OK;
+    }
+    VTM_TRY(st);
+  }
   int* d_cond = P->d_err.as<int>() + 1;
   VTM_CUDA_TRY(cudaMemsetAsync(d_cond, 0, sizeof(int), s));
   band_inverse_kernel<<<dim3((P->bb_blocks + 3) / 4, 2), 128, 0, s>>>(
@@ -325,9 +337,7 @@ vtm_status band_blk_prepare(vtm_plan_s* P) {
       P->d_bb_off.as<int32_t>(), P->nparts, P->d_Lc.as<double>(), P->d_Uc.as<double>(), P->d_bb_Li.as<double>(),
       P->d_bb_Ui.as<double>(), d_cond);
   VTM_CUDA_TRY(cudaGetLastError());
-  if (P->opts.precision != VTM_PREC_FP64) {
-    VTM_TRY(dev_alloc(P->d_bb_Li32, ne * sizeof(float)));
-    VTM_TRY(dev_alloc(P->d_bb_Ui32, ne * sizeof(float)));
+  if (f32) {
     convert_f32(P->d_bb_Li.as<double>(), P->d_bb_Li32.as<float>(), ne, s);
     convert_f32(P->d_bb_Ui.as<double>(), P->d_bb_Ui32.as<float>(), ne, s);
   }

@@ -903,9 +903,9 @@ vtm_status build_reflections(vtm_plan_s* P) {
     return VTM_EINVAL;
   }
   // 32 ports at a time for symmetric plans (reflect.cu); else a warp per port
-  if (reflect_blk_eligible(P)) {
-    VTM_TRY(build_reflections_blk(P));
-  } else if (npt > 0) {
+  bool done = false;
+  VTM_TRY(build_reflections_blk(P, &done));
+  if (!done && npt > 0) {
     if (!P->d_port_tile.p) {
       std::vector<int32_t> port_tile(npt);
       for (int32_t t = 0; t < P->nparts; ++t)

@@ -228,12 +228,15 @@ __global__ void __launch_bounds__(kRfThreads, 2) build_reflection_blk_kernel(
 
 // Symmetric plans of half bandwidth 33 up to what ring and stages leave room for
 // (about 220); vtm_factor has made the inverted diagonal blocks.
-bool reflect_blk_eligible(const vtm_plan_s* P) {
+static bool reflect_blk_eligible(const vtm_plan_s* P) {
   return P->symmetric && !P->general && !P->port_node.empty() && P->bb_ok && rf_smem(P->max_bw) <= 222 * 1024;
 }
 
-vtm_status build_reflections_blk(vtm_plan_s* P) {
+// *done = false where it does not serve
+vtm_status build_reflections_blk(vtm_plan_s* P, bool* done) {
   cudaStream_t s = P->stream;
+  *done = false;
+  if (!reflect_blk_eligible(P)) return VTM_OK;
   if (P->refl_items == 0) {
     const size_t npt = P->port_node.size();
     std::vector<int32_t> by_row(npt);
@@ -262,7 +265,13 @@ vtm_status build_reflections_blk(vtm_plan_s* P) {
   VTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, build_reflection_blk_kernel, kRfThreads, smem));
   const int grid = std::min(P->refl_items, std::max(1, per_sm) * sms);
   const int64_t slab = (int64_t)P->max_nodes * kRfC;
-  VTM_TRY(dev_alloc(P->d_refl_scratch, (size_t)grid * slab * sizeof(double)));
+  const vtm_status st = dev_alloc(P->d_refl_scratch, (size_t)grid * slab * sizeof(double));
+  if (st == VTM_ENOMEM) {  // a warp per port needs none
+    cudaGetLastError();
+    return VTM_OK;
+  }
+  VTM_TRY(st);
+  *done = true;
   int* queue = P->d_err.as<int>() + 4;
   cudaMemsetAsync(queue, 0, sizeof(int), s);
   build_reflection_blk_kernel<<<grid, kRfThreads, smem, s>>>(

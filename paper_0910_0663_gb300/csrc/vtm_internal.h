@@ -435,8 +435,7 @@ void launch_band_solve32(vtm_plan_s* P, float* v, int ncols, int64_t vec_stride,
 void convert_f32(const double* a, float* b, int64_t n, cudaStream_t s);
 
 // reflect.cu
-bool reflect_blk_eligible(const vtm_plan_s* P);
-vtm_status build_reflections_blk(vtm_plan_s* P);
+vtm_status build_reflections_blk(vtm_plan_s* P, bool* done);
 
 // bandblk.cu (band solves of half bandwidths 33..256); the launchers return
 // false where the plan has no inverted blocks

@@ -1,0 +1,43 @@
+"""Workspaces that only make a call faster do not make it fail: with the device's
+memory nearly taken the kernels that need none of them serve.
+
+The bars are those of the same solves with memory to spare (1e-10 of ||b|| asked for)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_0910_0663_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+class _Full:
+    """Takes the device's free memory but for `left` bytes."""
+
+    def __init__(self, left):
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        self.block = torch.empty(max(free - left, 0), dtype=torch.uint8, device="cuda") if free > left else None
+
+    def release(self):
+        self.block = None
+        torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_factor_and_solve_without_room_for_the_inverses(precision):
+    from paper_0910_0663_gb300 import vtm
+    # 537 MB of inverses (FP32 sweeps: 805), 118 MB of T_P; FP32 sweeps 545 MB of factors
+    w = wl.grid2d(1024, 1024, 64, 64, ground=0.1, seed=1)
+    b = torch.from_numpy(w.b[0]).cuda()
+    plan = vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts, precision=precision, factor=False)
+    torch.cuda.synchronize()
+    full = _Full(480 << 20 if precision == "fp64" else 1000 << 20)
+    try:
+        plan.factor()
+        x, info = plan.solve(b, tol=1e-10)
+    finally:
+        full.release()
+    plan.factor()  # with room again
+    y, again = plan.solve(b, tol=1e-10)
+    assert info["relres"] <= 1e-10 and again["relres"] <= 1e-10
