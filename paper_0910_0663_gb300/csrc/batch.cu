@@ -2273,10 +2273,9 @@ vtm_status ensure_vals_df(vtm_plan_s* P) {
   return VTM_OK;
 }
 
-// Lists and digits of the tensor-core FP64 sweep; *ok = false where it does not serve.
-static vtm_status prepare_digits(vtm_plan_s* P, int ngroups, bool* ok) {
+// Work lists of the tensor-core FP64 sweep (once per plan).
+static vtm_status list_digits(vtm_plan_s* P) {
   cudaStream_t s = P->stream;
-  *ok = false;
   if (P->dg_res == 0) {
     std::vector<DgItem> items;
     std::vector<DgChunk> chunks;
@@ -2308,17 +2307,33 @@ static vtm_status prepare_digits(vtm_plan_s* P, int ngroups, bool* ok) {
     P->dg_blocks = blocks;
     P->dg_kb = kb;
   }
+  return VTM_OK;
+}
+
+static void free_digits(vtm_plan_s* P) {
+  for (DevBuf* b : {&P->d_dg_T, &P->d_dg_texp, &P->d_dg_w, &P->d_dg_wexp}) dev_free(*b);
+  P->dg_ready = false;
+}
+
+// T_P's digits and the buffers of the waves'; *ok = false where the sweep does not serve.
+static vtm_status prepare_digits(vtm_plan_s* P, int ngroups, bool* ok) {
+  cudaStream_t s = P->stream;
+  *ok = false;
   const size_t bytes = std::max<size_t>((size_t)P->dg_blocks * sizeof(uint4), 16);
   if (bytes > ((size_t)32 << 30)) return VTM_OK;
   if (dev_alloc(P->d_dg_T, bytes) != VTM_OK || dev_alloc(P->d_dg_texp, P->port_node.size() * sizeof(int)) != VTM_OK ||
       dev_alloc(P->d_dg_w, (size_t)P->dg_kb * ngroups * kDg * 256) != VTM_OK ||
       dev_alloc(P->d_dg_wexp, (size_t)P->dg_chunks * 64 * sizeof(int)) != VTM_OK) {
     cudaGetLastError();
-    dev_free(P->d_dg_T);
-    P->dg_ready = false;
+    free_digits(P);
     return VTM_OK;
   }
   if (!P->dg_ready) {
+    size_t left = 0, total = 0;  // the solve's small buffers come later
+    if (cudaMemGetInfo(&left, &total) == cudaSuccess && left < ((size_t)64 << 20)) {
+      free_digits(P);
+      return VTM_OK;
+    }
     row_exponents_kernel<<<dim3(P->nparts, 16), 256, 0, s>>>(P->d_T64.as<double>(), P->tabs.T_off.as<int64_t>(),
                                                    P->tabs.T_ld.as<int32_t>(), P->tabs.port_off.as<int32_t>(),
                                                    P->d_dg_texp.as<int>());
@@ -2403,14 +2418,17 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
     P->launch_count++;
     P->tc_nitems = nt;
   }
-  // FP64 plans: digits of T_P for the tensor-core sweep (built at the first
-  // batched solve after each factorisation; 18 bytes per entry, so not where
-  // that passes 32 GB or memory runs out)
-  const int nt8 = (R + 7) / 8;
-  bool dg_ok = false;
-  // 8-column groups per work item, items side by side (their T_P digits from HBM once)
-  const int dg_nt = nt8 == 4 ? 2 : std::min(nt8, kDgMaxNt), dg_ny = (nt8 + dg_nt - 1) / dg_nt;
-  if (prec == VTM_PREC_FP64 && npt > 0 && P->opts.batch_kernel == 0) VTM_TRY(prepare_digits(P, dg_nt * dg_ny, &dg_ok));
+  const bool digits = prec == VTM_PREC_FP64 && npt > 0 && P->opts.batch_kernel == 0;
+  if (digits) VTM_TRY(list_digits(P));
+  // a buffer that every variant needs takes the digits' place where memory runs out
+  auto dev_alloc = [&](DevBuf& b, size_t bytes) -> vtm_status {
+    const vtm_status st = vtm::dev_alloc(b, bytes);
+    if (st != VTM_ENOMEM || !P->d_dg_T.p) return st;
+    cudaGetLastError();
+    VTM_CUDA_TRY(cudaStreamSynchronize(s));
+    free_digits(P);
+    return vtm::dev_alloc(b, bytes);
+  };
   const bool lowp = prec != VTM_PREC_FP64;
   const size_t wsz = lowp ? sizeof(float) : sizeof(double);
   VTM_TRY(dev_alloc(P->d_bV, (size_t)n * R * sizeof(double)));
@@ -2449,6 +2467,14 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
   } else {
     VTM_TRY(dev_alloc(P->d_r, (size_t)n * R * sizeof(double)));
   }
+  // FP64 plans: digits of T_P for the tensor-core sweep (built at the first
+  // batched solve after each factorisation; 18 bytes per entry, so not where
+  // that passes 32 GB or the other buffers leave too little memory)
+  const int nt8 = (R + 7) / 8;
+  bool dg_ok = false;
+  // 8-column groups per work item, items side by side (their T_P digits from HBM once)
+  const int dg_nt = nt8 == 4 ? 2 : std::min(nt8, kDgMaxNt), dg_ny = (nt8 + dg_nt - 1) / dg_nt;
+  if (digits) VTM_TRY(prepare_digits(P, dg_nt * dg_ny, &dg_ok));
   float* V32 = P->d_bV32.as<float>();
   double* xacc = P->d_xacc.as<double>();
   double* r = P->d_r.as<double>();  // set again when a double-float solve switches to FP64

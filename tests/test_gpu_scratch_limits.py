@@ -41,3 +41,24 @@ def test_factor_and_solve_without_room_for_the_inverses(precision):
     plan.factor()  # with room again
     y, again = plan.solve(b, tol=1e-10)
     assert info["relres"] <= 1e-10 and again["relres"] <= 1e-10
+
+
+def test_batched_solve_where_the_digits_would_take_the_rest():
+    """Room for the digits of T_P (18 bytes per entry) or for the columns' buffers, not
+    for both: the FP64 sweep on the CUDA cores serves, and the digits again with room."""
+    from paper_0910_0663_gb300 import vtm
+    w = wl.thermal3d(16, 48, 48, 20, nrhs=64, seed=4, min_box=200, max_box=4000)
+    b = torch.from_numpy(w.b).cuda()
+    plan = vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts)
+    p = np.bincount(plan.ports()[2], minlength=w.nparts)
+    digits = int(((p + 15) // 16 * ((p + 7) // 8) * 9 * 256).sum())
+    torch.cuda.synchronize()
+    full = _Full(digits + (120 << 20))
+    try:
+        x, info = plan.solve(b, tol=1e-10)
+        assert plan.stats()["batch_kernel"] == 1
+    finally:
+        full.release()
+    y, again = plan.solve(b, tol=1e-10)
+    assert plan.stats()["batch_kernel"] == 2
+    assert info["relres"] <= 1e-10 and again["relres"] <= 1e-10
