@@ -324,7 +324,6 @@ vtm_status band_blk_prepare(vtm_plan_s* P) {
   for (int i = 0; i < (f32 ? 4 : 2); ++i) {
     const vtm_status st = dev_alloc(*inv[i], ne * sz[i]);
     if (st == VTM_ENOMEM) {
-      cudaGetLastError();
       for (DevBuf* b : inv) dev_free(*b);
       return VTM_OK;
     }

@@ -2324,7 +2324,6 @@ static vtm_status prepare_digits(vtm_plan_s* P, int ngroups, bool* ok) {
   if (dev_alloc(P->d_dg_T, bytes) != VTM_OK || dev_alloc(P->d_dg_texp, P->port_node.size() * sizeof(int)) != VTM_OK ||
       dev_alloc(P->d_dg_w, (size_t)P->dg_kb * ngroups * kDg * 256) != VTM_OK ||
       dev_alloc(P->d_dg_wexp, (size_t)P->dg_chunks * 64 * sizeof(int)) != VTM_OK) {
-    cudaGetLastError();
     free_digits(P);
     return VTM_OK;
   }
@@ -2424,7 +2423,6 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
   auto dev_alloc = [&](DevBuf& b, size_t bytes) -> vtm_status {
     const vtm_status st = vtm::dev_alloc(b, bytes);
     if (st != VTM_ENOMEM || !P->d_dg_T.p) return st;
-    cudaGetLastError();
     VTM_CUDA_TRY(cudaStreamSynchronize(s));
     free_digits(P);
     return vtm::dev_alloc(b, bytes);

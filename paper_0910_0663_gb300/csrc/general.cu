@@ -531,7 +531,6 @@ template <bool PORTS>
 static vtm_status plan_resident_if_room(vtm_plan_s* P) {
   const vtm_status st = plan_resident<PORTS>(P);
   if (st != VTM_ENOMEM) return st;
-  cudaGetLastError();
   P->gen_ctas = -1;
   return VTM_OK;
 }

@@ -22,6 +22,7 @@ vtm_status dev_alloc(DevBuf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   cudaError_t e = cudaMalloc(&b.p, bytes);
   if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next call's check of its launches
     b.p = nullptr;
     set_detail(std::string("cudaMalloc(") + std::to_string(bytes) + "): " + cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? VTM_ENOMEM : VTM_ECUDA;

@@ -266,10 +266,7 @@ vtm_status build_reflections_blk(vtm_plan_s* P, bool* done) {
   const int grid = std::min(P->refl_items, std::max(1, per_sm) * sms);
   const int64_t slab = (int64_t)P->max_nodes * kRfC;
   const vtm_status st = dev_alloc(P->d_refl_scratch, (size_t)grid * slab * sizeof(double));
-  if (st == VTM_ENOMEM) {  // a warp per port needs none
-    cudaGetLastError();
-    return VTM_OK;
-  }
+  if (st == VTM_ENOMEM) return VTM_OK;  // a warp per port needs none
   VTM_TRY(st);
   *done = true;
   int* queue = P->d_err.as<int>() + 4;

@@ -62,3 +62,20 @@ def test_batched_solve_where_the_digits_would_take_the_rest():
     y, again = plan.solve(b, tol=1e-10)
     assert plan.stats()["batch_kernel"] == 2
     assert info["relres"] <= 1e-10 and again["relres"] <= 1e-10
+
+
+def test_a_call_that_ran_out_of_memory_leaves_the_next_one_alone():
+    from paper_0910_0663_gb300 import vtm
+    w = wl.grid2d(1024, 1024, 64, 64, ground=0.1, seed=1)
+    arrays = [torch.from_numpy(a).cuda() for a in (w.indptr, w.indices, w.data, w.partition)]
+    small = wl.grid2d(24, 24, 8, 8, ground=0.1, seed=2)
+    torch.cuda.synchronize()
+    full = _Full(64 << 20)
+    try:
+        with pytest.raises(vtm.VTMError, match="out of memory"):
+            vtm.Plan(*arrays, w.nparts)
+        plan = vtm.Plan(small.indptr, small.indices, small.data, small.partition, small.nparts)
+    finally:
+        full.release()
+    x, info = plan.solve(torch.from_numpy(small.b[0]).cuda())
+    assert info["relres"] <= 1e-10
