@@ -237,6 +237,16 @@ __global__ void __launch_bounds__(1024) general_sweep_kernel(
   }
 }
 
+// 16-byte asynchronous copies into shared memory, completing in groups
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // The same sweeps in one cooperative launch, one bounded grid barrier per sweep (the
 // control warp of gridctl.cuh).  A CTA owns a contiguous range of output pairs -- of
 // one tile or several -- of equal cost (pairs times inputs): thread (pair, group) takes

@@ -65,25 +65,4 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return false;
 }
 
-// Programmatic dependent launch (sm_90+): a sweep launched with the
-// programmatic-serialization attribute may start while the sweep before it
-// finishes.  Before pdl_wait it reads only what no kernel of the solve
-// writes (the reflection blocks, the plan's tables); pdl_wait returns once
-// the previous grid has completed and its writes are visible.  Without the
-// attribute both are no-ops.
-__device__ __forceinline__ void pdl_launch_dependents() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// 16-byte asynchronous copies into shared memory, completing in groups
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 }  // namespace vtm

@@ -841,142 +841,16 @@ struct SymPorts {
   }
 };
 
-// Kernel 1: direct 16-byte loads of the full matrices.  A work item is a slab of
-// SW outputs of one tile: SW / VEC lanes hold VEC outputs each, the 256 threads'
-// G = 256 VEC / SW such groups take the inputs t = g, g + G, ... (each a
-// contiguous piece of row t of T_P^T), and the groups' partial sums are added
-// in a fixed order.  Slabs rather than whole tiles: the tiles of uneven plans
-// (up to 1584 ports beside 200) and plans with few tiles then still give every
-// SM the same bytes; the price is that each slab gathers all of its tile's
-// incident waves (4-8 bytes per input from L2, against SW elements of T).  SW is
-// the largest of 128, 64, 32 that gives four items per SM.  The first rows of
-// T, which need no waves, are loaded before the previous sweep is waited for
-// (programmatic dependent launch).
-// Bound by HBM for FP32 / 16 bits (the matrices once per sweep) and by the FP64
-// pipe for FP64.  Measured per FP32 sweep of a thermal grid in 150
-// boxes of up to 1584 ports (259 MB of T_P, 38 us at the copy bandwidth): one
-// CTA per tile 610 us, slabs with T in a register buffer of 8 loads 105 us
-// (scoreboard waits left two in flight), this ring 58 us.  FP64, 64 tiles of 256
-// ports: 26.4 -> 19 us.
-struct __align__(16) SlabItem {
-  int32_t p0, p, m0, ld;  // first port, ports, first output of the slab, row length
-  int64_t T_off;
-  int32_t pad[2];
-};
-
-constexpr int kSlabStages = 12;  // 16-byte loads in flight per thread
-
-template <class TT, class WT, int VEC>
-__global__ void __launch_bounds__(256, 3) sweep_slab_kernel(
-    const TT* __restrict__ T, const SlabItem* __restrict__ items, int lanes,
-    const int32_t* __restrict__ twin, const typename KdOf<WT>::type* __restrict__ kd,
-    const uint8_t* __restrict__ run, const WT* __restrict__ c, WT* __restrict__ state,
-    int64_t nports, SweepCtrl* __restrict__ ctrl, double* __restrict__ partials,
-    double* __restrict__ hist, int hist_len) {
-  using LD = VecLoadG<TT, VEC>;
-  using WP = typename KdOf<WT>::type;  // a (w_in, w_out) pair
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_k, s_flag;
-  __shared__ bool s_last;
-  const int tid = threadIdx.x;
-  const SlabItem it = items[blockIdx.x];
-  const int p0 = it.p0, p = it.p;
-  const int G = 256 / lanes, g = tid / lanes, l = tid % lanes;
-  const int SW = lanes * VEC;
-  const bool active = it.m0 + l * VEC < it.ld;  // rows are padded to whole vectors
-  const TT* Tb = T + it.T_off + it.m0 + l * VEC;
-  constexpr int ST = kSlabStages;
-  // stage b of this thread: 16 bytes of its own (it copies and reads them
-  // itself, so the ring needs no barrier)
-  uint4* ring = reinterpret_cast<uint4*>(smem_raw) + tid;
-  WT* red = reinterpret_cast<WT*>(smem_raw);  // [256 VEC], once the ring is done
-  WT* w_in = reinterpret_cast<WT*>(smem_raw + ST * 256 * 16);
-  int tn = g, sn = 0;  // next input and stage to load
-  auto issue = [&]() {
-    if (active && tn < p) cp_async16(ring + sn * 256, Tb + (size_t)tn * it.ld);
-    cp_async_commit_group();
-    tn += G;
-    sn = sn + 1 == ST ? 0 : sn + 1;
-  };
-#pragma unroll
-  for (int b = 0; b < ST - 1; ++b) issue();
-  pdl_launch_dependents();
-  pdl_wait();  // the previous sweep's waves, decision and counters
-  if (tid == 0) {
-    s_k = *((volatile int*)&ctrl->k);
-    s_flag = *((volatile int*)&ctrl->flag);
-  }
-  __syncthreads();
-  if (s_flag) {
-    cp_async_wait_group<0>();  // no copy into shared memory outlives the CTA
-    return;
-  }
-  const int k = s_k;
-  const WP* prev = reinterpret_cast<const WP*>(state) + (size_t)((k - 1) & 1) * nports;
-  WP* cur = reinterpret_cast<WP*>(state) + (size_t)(k & 1) * nports;
-  // incident waves of the tile (delay 1): the twins' outgoing waves
-  for (int s = tid; s < p; s += 256) w_in[s] = k > 1 ? prev[twin[p0 + s]].y : (WT)0;
-  // residual of sweep k - 1 at the nodes whose ports start in this slab, summed and
-  // squared in FP64: the square of an FP32 residual below 1e-22 or above 1e19 is none
-  double sq = 0.0;
-  if (k > 1) {
-    for (int s = it.m0 + tid; s < min(p, it.m0 + SW); s += 256) {
-      const int nr = run[p0 + s];
-      if (nr) {
-        double r = 0.0;
-        for (int q = p0 + s; q < p0 + s + nr; ++q) {
-          const WP ws = prev[q], wt = prev[twin[q]];
-          r += (double)port_residual<WT>(ws.x, ws.y, wt.x, wt.y, kd[q]);
-        }
-        sq += r * r;
-      }
-    }
-  }
-  __syncthreads();
-  WT acc[VEC];
-#pragma unroll
-  for (int e = 0; e < VEC; ++e) acc[e] = 0;
-  int sl = 0;
-#pragma unroll 4
-  for (int t = g; t < p; t += G) {
-    issue();
-    cp_async_wait_group<ST - 1>();  // this thread's bytes of input t have landed
-    if (active) {
-      WT val[VEC];
-      LD::unpack(*reinterpret_cast<const typename LD::raw*>(ring + sl * 256), val);
-      const WT wt = w_in[t];
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) acc[e] += val[e] * wt;
-    }
-    sl = sl + 1 == ST ? 0 : sl + 1;
-  }
-  cp_async_wait_group<0>();
-  __syncthreads();  // the ring becomes the partial sums
-#pragma unroll
-  for (int e = 0; e < VEC; ++e) red[g * SW + l * VEC + e] = acc[e];
-  const double slab_sq = block_sum_value(sq);
-  // (the sum's barriers stand between the partials and their readers)
-  if (tid < SW && it.m0 + tid < p) {
-    const int s = it.m0 + tid;
-    WT o = c[p0 + s];
-    for (int a = 0; a < G; ++a) o += red[a * SW + tid];
-    WP pair;
-    pair.x = w_in[s];
-    pair.y = o;
-    cur[p0 + s] = pair;
-  }
-  // the last slab to finish reduces the residual of sweep k - 1
-  if (tid == 0) {
-    partials[blockIdx.x] = slab_sq;
-    __threadfence();
-    s_last = atomicAdd(&ctrl->counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const double tot = block_sum_fixed(partials, gridDim.x);
-  if (tid == 0) sweep_decide(ctrl, k, tot, hist, hist_len);
+// Programmatic dependent launch (sm_90+): a sweep launched with the
+// programmatic-serialization attribute may start while the sweep before it
+// finishes.  Before pdl_wait it reads only what no kernel of the solve
+// writes (the reflection blocks, the plan's tables); pdl_wait returns once
+// the previous grid has completed and its writes are visible.  Without the
+// attribute both are no-ops.
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Incident waves of the tile (zero past p, the padding of the last block)
 // and this thread's share of the squared node residuals of sweep k - 1.
@@ -1284,6 +1158,14 @@ constexpr int kWflowWarps = 4;
 constexpr int kWflowCtasPerSm = 7;
 
 // 16-byte asynchronous copy global -> shared (L2 only), its groups and waits
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 // lane's share of one packed block: the bytes it later reads itself (SymLoad)
 template <class TT>
 __device__ __forceinline__ void copy_block_async(TT* dst, const TT* src, int lane) {
@@ -2580,6 +2462,147 @@ __global__ void __launch_bounds__(32 * kWflowWarps, kWflowCtasPerSm) sweep_wflow
       }
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// the sweep over the full matrices in slabs
+// ---------------------------------------------------------------------------
+
+// Kernel 1: direct 16-byte loads of the full matrices.  A work item is a slab of
+// SW outputs of one tile: SW / VEC lanes hold VEC outputs each, the 256 threads'
+// G = 256 VEC / SW such groups take the inputs t = g, g + G, ... (each a
+// contiguous piece of row t of T_P^T), and the groups' partial sums are added
+// in a fixed order.  Slabs rather than whole tiles: the tiles of uneven plans
+// (up to 1584 ports beside 200) and plans with few tiles then still give every
+// SM the same bytes; the price is that each slab gathers all of its tile's
+// incident waves (4-8 bytes per input from L2, against SW elements of T).  SW is
+// the largest of 128, 64, 32 that gives four items per SM.  The first rows of
+// T, which need no waves, are loaded before the previous sweep is waited for
+// (programmatic dependent launch).
+// Bound by HBM for FP32 / 16 bits (the matrices once per sweep) and by the FP64
+// pipe for FP64.  Measured per FP32 sweep of a thermal grid in 150
+// boxes of up to 1584 ports (259 MB of T_P, 38 us at the copy bandwidth): one
+// CTA per tile 610 us, slabs with T in a register buffer of 8 loads 105 us
+// (scoreboard waits left two in flight), this ring 58 us.  FP64, 64 tiles of 256
+// ports: 26.4 -> 19 us.
+struct __align__(16) SlabItem {
+  int32_t p0, p, m0, ld;  // first port, ports, first output of the slab, row length
+  int64_t T_off;
+  int32_t pad[2];
+};
+
+constexpr int kSlabStages = 12;  // 16-byte loads in flight per thread
+
+template <class TT, class WT, int VEC>
+__global__ void __launch_bounds__(256, 3) sweep_slab_kernel(
+    const TT* __restrict__ T, const SlabItem* __restrict__ items, int lanes,
+    const int32_t* __restrict__ twin, const typename KdOf<WT>::type* __restrict__ kd,
+    const uint8_t* __restrict__ run, const WT* __restrict__ c, WT* __restrict__ state,
+    int64_t nports, SweepCtrl* __restrict__ ctrl, double* __restrict__ partials,
+    double* __restrict__ hist, int hist_len) {
+  using LD = VecLoadG<TT, VEC>;
+  using WP = typename KdOf<WT>::type;  // a (w_in, w_out) pair
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_k, s_flag;
+  __shared__ bool s_last;
+  const int tid = threadIdx.x;
+  const SlabItem it = items[blockIdx.x];
+  const int p0 = it.p0, p = it.p;
+  const int G = 256 / lanes, g = tid / lanes, l = tid % lanes;
+  const int SW = lanes * VEC;
+  const bool active = it.m0 + l * VEC < it.ld;  // rows are padded to whole vectors
+  const TT* Tb = T + it.T_off + it.m0 + l * VEC;
+  constexpr int ST = kSlabStages;
+  // stage b of this thread: 16 bytes of its own (it copies and reads them
+  // itself, so the ring needs no barrier)
+  uint4* ring = reinterpret_cast<uint4*>(smem_raw) + tid;
+  WT* red = reinterpret_cast<WT*>(smem_raw);  // [256 VEC], once the ring is done
+  WT* w_in = reinterpret_cast<WT*>(smem_raw + ST * 256 * 16);
+  int tn = g, sn = 0;  // next input and stage to load
+  auto issue = [&]() {
+    if (active && tn < p) cp_async16(ring + sn * 256, Tb + (size_t)tn * it.ld);
+    cp_async_commit_group();
+    tn += G;
+    sn = sn + 1 == ST ? 0 : sn + 1;
+  };
+#pragma unroll
+  for (int b = 0; b < ST - 1; ++b) issue();
+  pdl_launch_dependents();
+  pdl_wait();  // the previous sweep's waves, decision and counters
+  if (tid == 0) {
+    s_k = *((volatile int*)&ctrl->k);
+    s_flag = *((volatile int*)&ctrl->flag);
+  }
+  __syncthreads();
+  if (s_flag) {
+    cp_async_wait_group<0>();  // no copy into shared memory outlives the CTA
+    return;
+  }
+  const int k = s_k;
+  const WP* prev = reinterpret_cast<const WP*>(state) + (size_t)((k - 1) & 1) * nports;
+  WP* cur = reinterpret_cast<WP*>(state) + (size_t)(k & 1) * nports;
+  // incident waves of the tile (delay 1): the twins' outgoing waves
+  for (int s = tid; s < p; s += 256) w_in[s] = k > 1 ? prev[twin[p0 + s]].y : (WT)0;
+  // residual of sweep k - 1 at the nodes whose ports start in this slab, summed and
+  // squared in FP64: the square of an FP32 residual below 1e-22 or above 1e19 is none
+  double sq = 0.0;
+  if (k > 1) {
+    for (int s = it.m0 + tid; s < min(p, it.m0 + SW); s += 256) {
+      const int nr = run[p0 + s];
+      if (nr) {
+        double r = 0.0;
+        for (int q = p0 + s; q < p0 + s + nr; ++q) {
+          const WP ws = prev[q], wt = prev[twin[q]];
+          r += (double)port_residual<WT>(ws.x, ws.y, wt.x, wt.y, kd[q]);
+        }
+        sq += r * r;
+      }
+    }
+  }
+  __syncthreads();
+  WT acc[VEC];
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) acc[e] = 0;
+  int sl = 0;
+#pragma unroll 4
+  for (int t = g; t < p; t += G) {
+    issue();
+    cp_async_wait_group<ST - 1>();  // this thread's bytes of input t have landed
+    if (active) {
+      WT val[VEC];
+      LD::unpack(*reinterpret_cast<const typename LD::raw*>(ring + sl * 256), val);
+      const WT wt = w_in[t];
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) acc[e] += val[e] * wt;
+    }
+    sl = sl + 1 == ST ? 0 : sl + 1;
+  }
+  cp_async_wait_group<0>();
+  __syncthreads();  // the ring becomes the partial sums
+#pragma unroll
+  for (int e = 0; e < VEC; ++e) red[g * SW + l * VEC + e] = acc[e];
+  const double slab_sq = block_sum_value(sq);
+  // (the sum's barriers stand between the partials and their readers)
+  if (tid < SW && it.m0 + tid < p) {
+    const int s = it.m0 + tid;
+    WT o = c[p0 + s];
+    for (int a = 0; a < G; ++a) o += red[a * SW + tid];
+    WP pair;
+    pair.x = w_in[s];
+    pair.y = o;
+    cur[p0 + s] = pair;
+  }
+  // the last slab to finish reduces the residual of sweep k - 1
+  if (tid == 0) {
+    partials[blockIdx.x] = slab_sq;
+    __threadfence();
+    s_last = atomicAdd(&ctrl->counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const double tot = block_sum_fixed(partials, gridDim.x);
+  if (tid == 0) sweep_decide(ctrl, k, tot, hist, hist_len);
 }
 
 }  // namespace vtm

@@ -117,3 +117,9 @@ def test_profiling_options_name_their_workload(monkeypatch):
     cfg = bench.workload_config(args)
     assert args.band_solve == 0
     assert cfg["n"] == 524288 and "128x128x32" in cfg["workload"] and "400 random boxes" in cfg["workload"]
+
+
+def test_recorded_traffic_belongs_to_the_kernels_in_the_tree():
+    with open(os.path.join(ROOT, "profiles", "sweep_traffic.json")) as fh:
+        rec = json.load(fh)
+    assert rec["kernel_source_sha256"] == bench.sweep_kernel_source_hash()
