@@ -4028,7 +4028,10 @@ extern "C" vtm_status vtm_adjoint(vtm_plan_t P, const double* g, double* lam, in
     }
     P->transposed = T;
   }
-  P->transposed->opts = P->opts;
+  // the plan's options as they are now, with what they need: room for the history, the
+  // precision's copies of the operators
+  VTM_TRY(vtm_set_opts(P->transposed, &P->opts));
+  if (!P->transposed->factored) VTM_TRY(vtm_factor(P->transposed));
   return solve_entry(P->transposed, g, lam, nrhs, tol, info);
 }
 

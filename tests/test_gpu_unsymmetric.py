@@ -78,3 +78,31 @@ def test_adjoint_of_unsymmetric_system(vtm):
     lam, info = plan.adjoint(torch.from_numpy(gvec).cuda(), tol=1e-11)
     lam_star = np.linalg.solve(A.toarray().T, gvec)
     assert np.abs(lam.cpu().numpy() - lam_star).max() <= 1e-8 * np.abs(lam_star).max()
+
+
+def test_adjoint_follows_the_options_of_its_plan(vtm):
+    """Options set after the first adjoint solve: a history longer than any buffer
+    allocated before, then another precision (LU factors inside the tiles, lines across)."""
+    w = wl.grid2d(48, 48, 12, 12, seed=9, ground=0.05)
+    rows = np.repeat(np.arange(w.n), np.diff(w.indptr))
+    data = w.data.copy()
+    data[(w.indices > rows) & (w.partition[rows] == w.partition[w.indices])] *= 0.8
+    At = w.csr()
+    At.data[:] = data
+    At = At.T.tocsr()
+    At.sort_indices()
+    plan = vtm.Plan(w.indptr, w.indices, data, w.partition, w.nparts)
+    g = torch.from_numpy(w.b[0]).cuda()
+    first, _ = plan.adjoint(g)
+    plan.set_options(history_len=5000)
+    lam, _ = plan.adjoint(g)
+    assert torch.equal(first, lam)
+    ref = O.vtm_midpoint(At, w.partition, w.nparts, w.b[:1], W=1.0, tol=0, max_sweeps=40).history[:, 0]
+    h = plan.history[:40]
+    m = h > 0  # entries past convergence stay zero
+    assert m.sum() >= 10 and np.allclose(h[m], ref[m], rtol=1e-9, atol=1e-13)
+    for precision in ("fp32", "fp64"):
+        plan.set_options(precision=precision)
+        plan.factor()
+        lam, info = plan.adjoint(g)
+        assert O.residual_norms(At, lam.cpu().numpy()[None], w.b[:1]).max() <= 1e-10
