@@ -228,8 +228,9 @@ typedef struct {
                             symmetric reflection matrices on and above the diagonal */
   int64_t packed_bytes;  /* bytes of the packed symmetric copies (0 if none) */
   int32_t batch_kernel;  /* batched sweep variant of the last batched solve (see
-                            vtm_opts.batch_kernel; 0: none yet); 2 on an FP64 plan: its
-                            warp-MMA form on exact digits, the autotuner's choice */
+                            vtm_opts.batch_kernel; 0: none yet); 2 on an FP64 plan: exact
+                            digits on tcgen05, the autotuner's choice (requesting 2 there
+                            gives the CUDA cores, 1) */
 } vtm_plan_stats;
 
 /* vtm_plan -- wire tearing (Sec. V) and the port table.

@@ -2620,8 +2620,8 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
           batch_sweep_digits_kernel<<<std::min(P->dg_items * dg_ny, sms), kDgThreads, smem, s>>>(
               P->d_dg_items.as<DgItem>(), P->dg_items, dg_nt, dg_ny, P->tabs.port_off.as<int32_t>(),
               P->d_dg_T.as<unsigned char>(), P->d_dg_texp.as<int>(), P->d_dg_w.as<unsigned char>(),
-              P->d_dg_wexp.as<int>(), P->d_bc.as<double>(), P->d_bstate.as<double>(), npt, R,
-              P->d_bctrl.as<BatchCtrl>());
+              P->d_dg_wexp.as<int>(), P->d_T64.as<double>(), P->tabs.T_off.as<int64_t>(), P->tabs.T_ld.as<int32_t>(),
+              P->d_bc.as<double>(), P->d_bstate.as<double>(), npt, R, P->d_bctrl.as<BatchCtrl>());
           return;
         }
         auto go = [&](auto* kern, int threads, const auto* T, const auto* cc, auto* st) {
@@ -2676,7 +2676,7 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
         if (P->batch_tuned[prec] == 0 || P->batch_tuned_R[prec] != R || (P->batch_tuned[prec] == 6) != dg_ok) {
           float best = 1e30f;
           for (int cand = 0; cand <= 5; ++cand) {
-            if (dg_ok && cand != 5) continue;  // (FP64: faster at every size, by 3 to 40 times)
+            if (dg_ok && cand != 5) continue;  // (1.3 to 30 times the CUDA cores: see split.cuh)
             if (cand == 5 && !dg_ok) continue;
             if (cand == 4 && prec != VTM_PREC_BF16) continue;
             if (cand < 4 && (cand & 1) && !(prec == VTM_PREC_BF16 && R % 8 == 0)) continue;
@@ -2709,7 +2709,7 @@ vtm_status solve_batched(vtm_plan_s* P, const double* d_b, double* d_x, int R, d
         }
         kv = P->batch_tuned[prec] - 1;
       }
-      // (an FP64 plan's tensor-core form counts as 2, warp MMAs)
+      // (an FP64 plan's tensor-core form, digits on tcgen05, counts as 2)
       P->batch_used = kv == 5 ? 2 : kv + 1;
       // batches of check_every launches replayed from a CUDA graph when the
       // plan has its own stream, and quarter batches for the tail up to the

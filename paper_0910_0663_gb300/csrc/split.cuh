@@ -14,6 +14,17 @@
 // (FP64 products round at 2^-53 of their own size, their sum at 2^-53 of itself).
 // The nine group sums join as 64-bit integers, one FP64 rounding per 256 inputs.
 //
+// Fixed point serves where the waves of a tile are of one size.  Where they are not (a
+// column with one hot node decays by 2^-40 across a box), the large ones would leave an
+// error of 2^-58 of themselves in outputs that are small, with a small entry of T_P at
+// their place.  So a column's chunk whose largest wave is more than 2^6 above the largest
+// of some eight neighbouring inputs of the tile is multiplied in FP64 instead, by the
+// warps that join (dg_graded).  Measured, one hot node per column, 30 boxes, converged to
+// 1e-10: entries 1e-30 of the peak were off by 0.3 of themselves, now by 1e-7 like the FP64
+// kernel's; 110 boxes, every column hot, 2 / 18 / 64 columns: 0.89 / 3.0 / 8.5 ms per sweep
+// (CUDA cores 6.9 ms at any count).  Columns of random currents are not graded; the blocks'
+// maxima cost them 1 to 5% (18 columns 0.258 -> 0.260 ms).
+//
 // Per sweep two launches.  batch_digits_kernel: the incident waves (twins' outgoing
 // ones) and their digits in the B operand's core matrices (a CTA per 256 ports), the
 // residual of sweep k - 1 in FP64 (a CTA per 64 ports); its last CTA closes the sweep
@@ -27,11 +38,15 @@
 // mma.sync 0.08 + 0.43 ms (its rate, about 4 cycles per m16n8k16 and SM); here
 // 0.06 + 0.20 ms, the same bits (1.03 GB per sweep: 0.15 ms at the copy rate).
 // Errors of the iterates against quad precision are those of the FP64 kernel to two
-// digits (1 to 20 sweeps; 3e-16 thermal, 8e-15 grids).
+// digits (1 to 20 sweeps; 3e-16 thermal, 8e-15 grids), and those of converged solutions
+// against a refined one, entry by entry, too (random columns 2.5e-11, hot ones 2e-11 at a
+// tolerance of 1e-14).  Against the CUDA cores, per sweep: 2 tiles of 10 ports 19 us / 28,
+// 16 of 32 ports 23 / 48, 64 of 256 ports 46 / 526, 110 boxes 260 / 6800 (18 columns).
 
 constexpr int kDg = 9;          // digits
 constexpr int kDgChunk = 16;    // 16-input blocks between two joins of the group sums
 constexpr int kDgStages = 5;
+constexpr int kDgSpan = 6;      // binary orders between the waves of a tile that the digits may serve
 constexpr int kDgMaxNt = 3;     // 8-column groups per work item (nine groups of 24 columns: 216 of 256 TMEM columns)
 
 // biased exponent of |v| (0x7ff: not finite)
@@ -122,6 +137,11 @@ __global__ void __launch_bounds__(256) pack_digits_kernel(const double* __restri
   }
 }
 
+// A chunk's waves of a column, [smallest block << 16 | largest exponent] (biased): graded
+// where the largest is more than kDgSpan above the smallest block of the tile.
+constexpr int kDgNoBlock = 0x7ff;
+__device__ __forceinline__ bool dg_graded(int wx, int tile_min) { return (wx & 0xffff) - tile_min > kDgSpan; }
+
 // Work item of the digits kernel: 256 ports of a tile (digits), or kDgRes (residual).
 constexpr int kDgRes = 64;  // (128: 60 us a launch instead of 58)
 struct __align__(16) DgChunk {
@@ -136,7 +156,7 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
     double* __restrict__ partials, const double* __restrict__ tol2, double* __restrict__ hist, int hist_len) {
   __shared__ double rsq[256];
   __shared__ int stw[16 * kDgChunk];
-  __shared__ int cmax[64];
+  __shared__ int cmax[64], bmin[64];  // per column: largest exponent, smallest largest of eight inputs
   __shared__ int s_k, s_flag;
   __shared__ bool s_last;
   const int tid = threadIdx.x;
@@ -144,7 +164,10 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
     s_k = *((volatile int*)&ctrl->k);
     s_flag = *((volatile int*)&ctrl->flag);
   }
-  if (tid < 64) cmax[tid] = 0;
+  if (tid < 64) {
+    cmax[tid] = 0;
+    bmin[tid] = kDgNoBlock;
+  }
   __syncthreads();
   if (s_flag) return;
   const int k = s_k;
@@ -204,13 +227,12 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
       if (mx) atomicMax(&cmax[r], mx);
     }
     __syncthreads();
-    if (tid < 64) wexp[blockIdx.x * 64 + tid] = cmax[tid] - 1022;
     // digits, a pair of rows per item, in the K-major core matrices of the B operand:
     // [16 inputs][column group of the items][digit][8 columns][input half][column][input]
     const int kbn = k > 1 ? (m1 - ch.m0 + 15) / 16 : 0, nt = NT * ny;
     const int w = tid & 63;
 #pragma unroll 2
-    for (int u = tid >> 6; u < kbn * nt; u += 4) {
+    for (int u = tid >> 6; u < kbn * nt; u += 4) {  // (a warp together)
       const int n = u % nt, kb = u / nt;
       const int c = 8 * n + ((w >> 2) & 7), i = 16 * kb + 8 * (w >> 5) + 2 * (w & 3);
       int d0[kDg], d1[kDg];
@@ -223,7 +245,14 @@ __global__ void __launch_bounds__(256) batch_digits_kernel(
       uint32_t* o = wd + (((size_t)(ch.kb + kb) * ny + n / NT) * kDg * NT + n % NT) * 64 + w;
 #pragma unroll
       for (int j = 0; j < kDg; ++j) o[(size_t)j * NT * 64] = bf16_pair(d0[j], d1[j]);
+      // the largest of eight inputs (four lanes), unless fewer than four are left of the tile
+      int e8 = max(exp_bits(v0), exp_bits(v1));
+      e8 = max(e8, __shfl_xor_sync(0xffffffffu, e8, 1));
+      e8 = max(e8, __shfl_xor_sync(0xffffffffu, e8, 2));
+      if ((w & 3) == 0 && col && nrow - (16 * kb + 8 * (w >> 5)) >= 4) atomicMin(&bmin[c], e8);
     }
+    __syncthreads();
+    if (tid < 64) wexp[blockIdx.x * 64 + tid] = bmin[tid] << 16 | cmax[tid];
   }
   if (tid == 0) {
     __threadfence();
@@ -308,7 +337,8 @@ __device__ __forceinline__ double dg_join(const uint32_t (&v)[kDg]) {
 __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
     const DgItem* __restrict__ items, int nitems, int NT, int ny, const int32_t* __restrict__ port_off,
     const unsigned char* __restrict__ Td, const int* __restrict__ texp, const unsigned char* __restrict__ wd,
-    const int* __restrict__ wexp, const double* __restrict__ c, double* __restrict__ state, int64_t nports, int R,
+    const int* __restrict__ wexp, const double* __restrict__ T64, const int64_t* __restrict__ T_off,
+    const int32_t* __restrict__ T_ld, const double* __restrict__ c, double* __restrict__ state, int64_t nports, int R,
     BatchCtrl* __restrict__ ctrl) {
   extern __shared__ __align__(1024) unsigned char dsm[];
   __shared__ uint64_t full[kDgStages], empty[kDgStages], tfull[2], tempty[2], ufull[2], uempty[2], drain;
@@ -446,9 +476,14 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
         for (int e = 0; e < 4; ++e) out[u][e] = 0.0;
       if (k > 1) {
         const int nch = (nb + kDgChunk - 1) / kDgChunk;
+        const bool mine = lane < (int)nc && c0 + lane < R;
+        int tmin = kDgNoBlock;  // the tile's smallest block in column c0 + lane
+        for (int j = 0; j < nch; ++j) tmin = min(tmin, mine ? wexp[(it.chunk + j) * 64 + c0 + lane] >> 16 : kDgNoBlock);
         for (int j = 0; j < nch; ++j, ++ch) {
           const uint32_t buf = ch & 1;
-          const int wx = lane < (int)nc && c0 + lane < R ? wexp[(it.chunk + j) * 64 + c0 + lane] : 0;
+          const int wp = mine ? wexp[(it.chunk + j) * 64 + c0 + lane] : 0;
+          const int wx = (wp & 0xffff) - 1022;
+          const uint32_t graded = __ballot_sync(0xffffffffu, mine && dg_graded(wp, tmin));  // by column
           if (!__all_sync(0xffffffffu, wait(&tfull[buf], (ch >> 1) & 1))) break;  // (the warp together)
           tc_fence_after();
 #pragma unroll
@@ -460,6 +495,7 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               if (c0 + 4 * q + e >= R) break;
+              if (graded >> (4 * q + e) & 1) continue;
               const int we = __shfl_sync(0xffffffffu, wx, 4 * q + e);
               uint32_t x[kDg];
 #pragma unroll
@@ -472,6 +508,34 @@ __global__ void __launch_bounds__(kDgThreads, 1) batch_sweep_digits_kernel(
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&tempty[buf]);
+          if (graded) {  // these columns' 256 inputs in FP64, in the digits' scale
+            const int ld = T_ld[it.tile], t0 = 16 * kDgChunk * j, nt = min(p - t0, 16 * kDgChunk), sr = min(s, p - 1);
+            const double* Tr = T64 + T_off[it.tile] + (size_t)t0 * ld + sr;
+            const int te = texp[p0 + sr] - 68;
+#pragma unroll
+            for (int u = 0; u < kDgMaxNt; ++u) {
+              const int q = h + 2 * u;
+              const uint32_t four = q < nq ? graded >> (4 * q) & 15u : 0u;
+              if (!four) continue;
+              double a[4] = {0.0, 0.0, 0.0, 0.0};
+              const double* wr = cur + (size_t)(p0 + t0) * 2 * R + c0 + 4 * q;
+              for (int t = 0; t < nt; t += 8) {
+                double T[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) T[i] = t + i < nt ? __ldg(Tr + (size_t)(t + i) * ld) : 0.0;
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                  if (four >> e & 1) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                      if (t + i < nt) a[e] = fma(T[i], wr[(size_t)(t + i) * 2 * R + e], a[e]);
+                  }
+              }
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (four >> e & 1) out[u][e] += ldexp(a[e], -te);
+            }
+          }
         }
       }
       if (s < p && !s_abort) {

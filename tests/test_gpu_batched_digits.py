@@ -68,3 +68,21 @@ def test_tiles_without_ports_and_non_finite_columns():
         plan.solve(torch.from_numpy(bad).cuda())
     y, _ = plan.solve(torch.from_numpy(w.b).cuda())
     assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("nrhs", [2, 6, 33])
+def test_columns_with_one_hot_node(nrhs):
+    """A column that decays by 1e-20 and more across its boxes keeps its small entries:
+    each within 1e-9 of itself of the CUDA cores' (45 sweeps of sums of up to 2000
+    products whose waves cancel to 1/64 at a place: 45 * 2000 * 64 u = 6e-10).  Columns
+    of random entries lie between them in the same groups of eight."""
+    w = wl.thermal3d(8, 24, 24, 8, nrhs=nrhs, seed=1, min_box=20, max_box=2600)
+    b = w.b.copy()
+    hot = np.random.default_rng(0).integers(0, w.n, nrhs)
+    for r in range(0, nrhs, 2):
+        b[r] = 0.0
+        b[r, hot[r]] = 1.0
+    x, ref = _pair(w, b, max_sweeps=45)
+    assert (np.abs(ref[0]).max() / np.abs(ref[0]).min()) > 1e20
+    assert (np.abs(x - ref)[::2] <= 1e-9 * np.abs(ref[::2])).all()
+    assert (np.abs(x - ref).max(1) <= 45 / 12 * 5.2e-13 * np.abs(ref).max(1)).all()
