@@ -676,13 +676,13 @@ vtm_status general_sweeps(vtm_plan_s* P, double bnorm2, double target2, int budg
   h.bnorm2 = bnorm2 > 0 ? bnorm2 : 1.0;
   *P->h_ctrl = h;
   VTM_CUDA_TRY(cudaMemcpyAsync(P->d_ctrl.p, P->h_ctrl, sizeof(SweepCtrl), cudaMemcpyHostToDevice, s));
-  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gin.p, 0, 2 * std::max<int64_t>(P->n_in, 1) * sizeof(double), s));
-  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gout.p, 0, kGenSlots * std::max<int64_t>(P->n_out, 1) * sizeof(double), s));
   if (P->gen_ctas == 0) VTM_TRY(plan_resident_if_room<false>(P));
   // (the barrier word holds as many arrivals and sweeps as res_counts allows; above that one
   // launch per sweep)
   if (P->gen_ctas > 0 && res_counts(budget, P->gen_ctas))
     return general_sweeps_resident(P, budget, hist, hist_len, sweep_out, flag_out);
+  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gin.p, 0, 2 * std::max<int64_t>(P->n_in, 1) * sizeof(double), s));
+  VTM_CUDA_TRY(cudaMemsetAsync(P->d_gout.p, 0, 2 * std::max<int64_t>(P->n_out, 1) * sizeof(double), s));
   // four groups of up to 256 threads per tile (one output each; eight groups
   // of 128 measured slower on the 1024^2 VCCS grid)
   constexpr int KS = 4;
