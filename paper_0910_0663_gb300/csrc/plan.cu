@@ -942,22 +942,40 @@ extern "C" vtm_status vtm_set_values(vtm_plan_t P, const double* vals) {
   cudaSetDevice(P->device);
   cudaStream_t s = P->stream;
   const size_t bytes = (size_t)P->nnz * sizeof(double);
-  VTM_TRY(dev_alloc(P->d_vals_new, bytes));
+  // into a second buffer, or, without the memory for one, over the old values with a copy
+  // of those on the host
+  vtm_status st = dev_alloc(P->d_vals_new, bytes);
+  const bool in_place = st == VTM_ENOMEM;
+  if (!in_place) VTM_TRY(st);
+  std::vector<double> old;
+  if (in_place) {
+    VTM_TRY(ensure_host_vals(P));
+    old = P->h_vals;
+  }
+  DevBuf& target = in_place ? P->d_vals : P->d_vals_new;
   // the values may come from the plan's stream or from the default stream: the
   // copy follows both
   VTM_CUDA_TRY(cudaStreamSynchronize(s));
-  VTM_CUDA_TRY(cudaMemcpyAsync(P->d_vals_new.p, vals, bytes, cudaMemcpyDefault, cudaStreamLegacy));
+  VTM_CUDA_TRY(cudaMemcpyAsync(target.p, vals, bytes, cudaMemcpyDefault, cudaStreamLegacy));
   VTM_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
+  auto refuse = [&](bool swapped) -> vtm_status {  // the old values again
+    if (in_place) VTM_CUDA_TRY(cudaMemcpy(P->d_vals.p, old.data(), bytes, cudaMemcpyHostToDevice));
+    else if (swapped) std::swap(P->d_vals, P->d_vals_new);
+    return VTM_OK;
+  };
   // finite, symmetric where the plan is, the same torn lines and couplings
-  VTM_TRY(check_values(P, P->d_vals_new.as<double>()));
-  std::swap(P->d_vals, P->d_vals_new);
+  if ((st = check_values(P, target.as<double>())) != VTM_OK) {
+    VTM_TRY(refuse(false));
+    return st;
+  }
+  if (!in_place) std::swap(P->d_vals, P->d_vals_new);
   const bool host_vals = P->host_vals;
   P->host_vals = false;
   std::vector<double> w_sca;
   std::swap(w_sca, P->w_sca);
-  vtm_status st = assemble_ports(P);
+  st = assemble_ports(P);
   if (st != VTM_OK) {
-    std::swap(P->d_vals, P->d_vals_new);
+    VTM_TRY(refuse(true));
     std::swap(w_sca, P->w_sca);
     const std::string why = g_detail;
     P->host_vals = host_vals && P->w_kind != VTM_W_SCA;  // (SCA read the refused values)

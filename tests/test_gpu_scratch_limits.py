@@ -79,3 +79,27 @@ def test_a_call_that_ran_out_of_memory_leaves_the_next_one_alone():
         full.release()
     x, info = plan.solve(torch.from_numpy(small.b[0]).cuda())
     assert info["relres"] <= 1e-10
+
+
+def test_new_values_without_room_for_a_second_copy():
+    from paper_0910_0663_gb300 import vtm
+    w = wl.grid2d(1536, 1536, 32, 32, ground=0.1, seed=1)  # 94 MB of values
+    new = torch.from_numpy(w.data * 1.5).cuda()
+    bad = new.clone()
+    bad[7] = float("nan")
+    b = torch.from_numpy(w.b[0]).cuda()
+    plan = vtm.Plan(w.indptr, w.indices, w.data, w.partition, w.nparts)
+    x0, _ = plan.solve(b)
+    full = _Full(90 << 20)
+    try:
+        with pytest.raises(vtm.VTMError, match="non-finite"):
+            plan.set_values(bad)
+        y, _ = plan.solve(b)  # still factored, the old values
+        plan.set_values(new)
+        plan.factor()
+        x, _ = plan.solve(b)
+    finally:
+        full.release()
+    assert torch.equal(x0, y)
+    ref, _ = vtm.Plan(w.indptr, w.indices, w.data * 1.5, w.partition, w.nparts, sweep_kernel=12).solve(b)
+    assert np.linalg.norm((x - ref).cpu().numpy()) <= 1e-7 * np.linalg.norm(ref.cpu().numpy())
