@@ -171,3 +171,31 @@ def test_tiles_above_128_ports_sweep_in_fp64():
     for e in (-400, 400):
         y, scaled = plan.solve(b * 2.0 ** e, tol=1e-14)
         assert scaled["sweeps"] == info["sweeps"] and torch.equal(y, x * 2.0 ** e)
+
+
+@pytest.mark.parametrize("kind", ["alpha", "wob"])
+def test_fp64_in_one_launch_equals_kernel_1_on_odd_and_lone_tiles(kind):
+    """Odd port counts (a last pair of outputs half empty), ranges of pairs over several
+    tiles, a tile without ports, power waves: the same sums in another order, so
+    histories agree like those of any two FP64 kernels (1e-9, 1e-13 absolute)."""
+    from paper_0910_0663_gb300 import vtm
+    w = wl.grid2d(129, 259, 43, 65, ground=0.3, seed=11)
+    rows = np.repeat(np.arange(w.n), np.diff(w.indptr))
+    lone = (w.partition[rows] == 5) != (w.partition[w.indices] == 5)
+    data = np.where(lone, 0.0, w.data)  # its branches stay on the diagonals: conductances to ground
+    b = torch.from_numpy(w.b[0]).cuda()
+    out = []
+    for kernel in (0, 1):
+        plan = vtm.Plan(w.indptr, w.indices, data, w.partition, w.nparts, sweep_kernel=kernel, factor=False)
+        plan.set_admittance(kind, alpha=0.8)
+        plan.factor()
+        st = plan.stats()
+        assert 128 < st["max_ports"] <= 256
+        plan.set_options(sweep_kernel=kernel, history_len=30)
+        x, info = plan.solve(b, tol=1e-12)
+        assert kernel or plan.stats()["sweep_kernel"] == 8
+        out.append((x, info["sweeps"], plan.history))
+    h0, h1 = out[0][2], out[1][2]
+    k = int(np.count_nonzero((h0 > 1e-9) & (h1 > 1e-9)))
+    assert abs(out[0][1] - out[1][1]) <= 1 and k >= 10
+    assert np.allclose(h0[:k], h1[:k], rtol=1e-9, atol=1e-13)
