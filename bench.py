@@ -320,12 +320,12 @@ def sweep_kernel_name(kernel, nrhs, batch_kernel=0):
                 3: "batch_sweep_kernel (CUDA cores, item per CTA)", 4: "batch_sweep_mma_kernel (warp MMAs, item per CTA)",
                 5: "batch_sweep_tc_kernel (tcgen05, TMEM accumulators, bulk-copy ring)"}.get(
                     batch_kernel, "batched sweep")
-    return {1: "sweep_kernel (direct loads)", 2: "sweep_staged_kernel (bulk-copy ring)",
+    return {1: "sweep_slab_kernel (direct loads, slabs of outputs)", 2: "sweep_staged_kernel (bulk-copy ring)",
             3: "sweep_vec_kernel (256 threads)", 4: "sweep_vec_kernel (128 threads)",
             5: "sweep_sym_kernel (packed symmetric, 128 threads)",
             6: "sweep_sym_kernel (packed symmetric, 64 registers)",
             7: "sweep_symb_kernel (packed symmetric, one bulk copy per tile)",
-            8: "sweep_flow_kernel (dataflow, one cooperative launch)",
+            8: "sweep_flow_kernel (dataflow) or, when autotuned, a resident form (one cooperative launch)",
             9: "sweep_wsym_kernel (packed symmetric, one warp per tile)",
             10: "sweep_wflow_kernel (dataflow, one warp per tile, one cooperative launch)",
             11: "sweep_wmma_kernel (packed symmetric, one warp per tile, block products as warp MMAs)",

@@ -52,7 +52,8 @@ typedef enum {
   VTM_ENOMEM = -2,       /* device or host allocation failed */
   VTM_ESINGULAR = -3,    /* non-positive (Cholesky) or zero (LU) pivot in a local factor */
   VTM_ENOCONV = -4,      /* tolerance not met within max_sweeps / max_outer; x = last iterate */
-  VTM_EDIVERGED = -5,    /* NaN/Inf or residual growth > 1e6 x initial; x = last iterate */
+  VTM_EDIVERGED = -5,    /* NaN/Inf or residual growth > 1e6 x initial; x = last iterate (a band
+                            solve whose bounded wait for a copy ran out marks its column NaN) */
   VTM_ETIMEOUT = -6,     /* a bounded device-side wait ran out (persistent kernels) */
   VTM_ECUDA = -7,        /* a CUDA runtime call failed */
   VTM_EINTERNAL = -8,    /* an internal consistency check failed */
@@ -215,8 +216,10 @@ typedef struct {
   int32_t max_nodes;     /* largest sub-circuit */
   int32_t max_band;      /* largest half-bandwidth of a local matrix after reordering */
   int32_t symmetric;     /* 1: A symmetric -> Cholesky; 0: LU without pivoting */
-  int64_t t_bytes;       /* bytes of the stored reflection matrices (all precisions kept) */
-  int64_t factor_bytes;  /* bytes of the stored local factors */
+  int64_t t_bytes;       /* bytes of the stored reflection matrices (all precisions kept; the
+                            rearranged copies of the batched sweeps not counted) */
+  int64_t factor_bytes;  /* bytes of the stored local factors (their FP32 copies and inverted
+                            diagonal blocks not counted) */
   int32_t sweep_kernel;  /* sweep kernel in use for the plan's precision (see vtm_opts); 8 also
                             stands for the resident forms that only the autotuner picks
                             (sweep_kernel 0; requesting 8 gives the dataflow kernel): every

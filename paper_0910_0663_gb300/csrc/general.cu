@@ -300,7 +300,7 @@ struct GenRes {
 // inputs and outputs of a tile its ports in their order, the source of an input its twin.
 // The last sweep leaves (w_in, w_out) pairs in gin.  For symmetric plans of up to 256 ports
 // per tile, like kernel 13.  Measured per sweep, kernel 1 -> here: 64 tiles of 256 ports
-// (33 MB of T_P, 6.9 us of FP64 pipe) 19 -> 11.1 us; 169 tiles of 128 ports 18.4 -> 9.3 us;
+// (27 MB of T_P, 7.7 us of busy FP64 pipe) 19 -> 11.1 us; 169 tiles of 128 ports 18.4 -> 9.3 us;
 // 9 tiles of 128 ports 16.4 -> 7.0 us.  CTAs with as little as two elements per thread:
 // 81 tiles of 124 ports 7.1 us, with at least eight 8.6 us (the channel form keeps eight:
 // its inputs gather from more tiles).
